@@ -120,16 +120,18 @@ __global__ void k_member_scatter(const uint16_t *__restrict__ gid, uint64_t N, u
 }
 
 // Repetition-0 member records, in member-list order: word 0 = point id,
-// words 1.. = group ids of repetitions 1..R-1, two per word (low half first).
+// words 1.. = group ids of repetitions 1..R-1, two per word (low half first);
+// mg1: the repetition-1 groups alone (0 when R = 1).
 __global__ void k_member_records(const uint32_t *__restrict__ mem, const uint16_t *__restrict__ gid,
                                  uint64_t N, uint32_t R, uint32_t rp, uint32_t rw,
-                                 uint32_t *__restrict__ rec)
+                                 uint32_t *__restrict__ rec, uint16_t *__restrict__ mg1)
 {
     for (uint64_t m = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; m < N;
          m += uint64_t(gridDim.x) * blockDim.x) {
         const uint32_t x = mem[m];
         const uint16_t *g = gid + uint64_t(x) * rp;
         rec[m * rw] = x;
+        mg1[m] = R > 1 ? g[1] : uint16_t(0);
         for (uint32_t w = 1; w < rw; ++w) {
             const uint32_t r = 2 * (w - 1) + 1;
             const uint32_t lo = r < R ? g[r] : 0u;
@@ -137,6 +139,13 @@ __global__ void k_member_records(const uint32_t *__restrict__ mem, const uint16_
             rec[m * rw + w] = lo | (hi << 16);
         }
     }
+}
+
+// mg1 from existing records (a loaded index).
+__global__ void k_member_groups1(const uint32_t *__restrict__ rec, uint64_t N, uint32_t rw, uint16_t *__restrict__ mg1)
+{
+    for (uint64_t m = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; m < N; m += uint64_t(gridDim.x) * blockDim.x)
+        mg1[m] = rw > 1 ? uint16_t(rec[m * rw + 1] & 0xFFFFu) : uint16_t(0);
 }
 
 // The (point, table) entries are taken table-major (t = l n + x): the threads
@@ -575,6 +584,15 @@ int build_heavy(flinng_index *ix, void *scan_ws, uint32_t *list)
     return FLINNG_OK;
 }
 
+int member_groups1(flinng_index *ix, uint64_t n)
+{
+    if (n == 0) return FLINNG_OK;
+    k_member_groups1<<<thread_blocks(n), 256, 0, ix->stream>>>(ix->mrec, n, ix->rw, ix->mg1);
+    count_launch();
+    FL_CUDA(cudaGetLastError());
+    return FLINNG_OK;
+}
+
 size_t perm_check_workspace_bytes(uint32_t R, uint64_t n)
 {
     return carve_bytes<uint32_t>(uint64_t(R) * ((n + 31) / 32) + 1);
@@ -679,7 +697,8 @@ int member_stage(flinng_index *ix, const uint32_t *perm, const uint16_t *groups,
         k_member_scatter<<<thread_blocks(N * R), 256, 0, st>>>(ix->gid, N, R, B, rp, mcur, ix->mem);
         count_launch();
         FL_CUDA(cudaGetLastError());
-        k_member_records<<<thread_blocks(N), 256, 0, st>>>(ix->mem, ix->gid, N, R, rp, ix->rw, ix->mrec);
+        k_member_records<<<thread_blocks(N), 256, 0, st>>>(ix->mem, ix->gid, N, R, rp, ix->rw, ix->mrec,
+                                                             ix->mg1);
         count_launch();
         FL_CUDA(cudaGetLastError());
     }

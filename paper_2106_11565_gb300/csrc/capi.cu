@@ -96,7 +96,7 @@ void free_index(flinng_index *ix)
 {
     if (!ix) return;
     destroy_graphs(ix);
-    void *ptrs[] = {ix->srp_w, ix->bucket_a, ix->bucket_c, ix->gid, ix->moff, ix->mem, ix->mrec, ix->off,
+    void *ptrs[] = {ix->srp_w, ix->bucket_a, ix->bucket_c, ix->gid, ix->moff, ix->mem, ix->mrec, ix->mg1, ix->off,
                     ix->hidx, ix->hbm,
                     ix->cells, ix->cells_tmp, ix->slot_a, ix->slot_b, ix->cell_cnt, ix->flag, ix->qnext,
                     ix->stats, ix->ws.ptr, ix->w_split, ix->w_norm, ix->w_aux, ix->tc_err};
@@ -394,10 +394,11 @@ int flinng_create(const flinng_config *cfg, const flinng_params *params, void *s
     ALLOC(moff, size_t(ix->BR) + 1);
     ALLOC(mem, size_t(R) * cfg->capacity);
     ALLOC(mrec, size_t(ix->rw) * cfg->capacity);
+    ALLOC(mg1, size_t(cfg->capacity) + kMg1Pad);
     ALLOC(off, ix->nslot + 1);
     ALLOC(hidx, ix->nslot + 1);
-    ALLOC(cells, ix->entries_cap);
-    ALLOC(cells_tmp, ix->entries_cap);
+    ALLOC(cells, ix->entries_cap + kCellPad);
+    ALLOC(cells_tmp, ix->entries_cap + kCellPad);
     ALLOC(slot_a, ix->nslot + 1);
     ALLOC(slot_b, ix->nslot + 1);
     ALLOC(cell_cnt, size_t(ix->BR) + 1);
@@ -436,6 +437,7 @@ int flinng_create(const flinng_config *cfg, const flinng_params *params, void *s
         chk(cudaMemsetAsync(ix->off, 0, (ix->nslot + 1) * sizeof(uint32_t), st), "zero off");
         chk(cudaMemsetAsync(ix->hidx, 0xFF, (ix->nslot + 1) * sizeof(uint32_t), st), "clear hidx");
         chk(cudaMemsetAsync(ix->moff, 0, (size_t(ix->BR) + 1) * sizeof(uint32_t), st), "zero moff");
+        chk(cudaMemsetAsync(ix->mg1, 0, (size_t(cfg->capacity) + kMg1Pad) * sizeof(uint16_t), st), "zero mg1");
         chk(cudaMemsetAsync(ix->stats, 0, kStats * sizeof(unsigned long long), st), "zero stats");
         chk(cudaMemsetAsync(ix->tc_err, 0, 4, st), "zero tensor-core flag");
         // the insert's second stream and its fork / join events

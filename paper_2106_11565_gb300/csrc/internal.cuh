@@ -24,6 +24,12 @@ constexpr unsigned long long kEntSign = 1ull << 63;
 __host__ __device__ inline uint64_t ent_row(unsigned long long e) { return (e >> 20) & ((1ull << 43) - 1); }
 __host__ __device__ inline uint32_t ent_col(unsigned long long e) { return uint32_t(e & 0xFFFFF); }
 
+// entries past the last member of flinng_index::mg1, so that a 16-byte load
+// of any member's unit stays inside
+constexpr uint64_t kMg1Pad = 16;
+// the same for the cell lists (read eight aligned cells at a time)
+constexpr uint64_t kCellPad = 8;
+
 // Error plumbing: every internal step returns an int status and leaves a
 // message in the thread-local buffer.
 int set_error(int code, const char *fmt, ...);
@@ -125,6 +131,8 @@ struct flinng_index {
     uint32_t *moff;        // BR + 1: members of cell c are mem[moff[c] .. moff[c+1])
     uint32_t *mem;         // R * capacity point ids
     uint32_t *mrec;        // capacity * rw: repetition-0 members with their other group ids
+    uint16_t *mg1;         // capacity + kMg1Pad: the members' repetition-1 groups alone, in mrec's
+                           // order (padding and unused entries are valid group ids)
     uint32_t *off;         // nslot + 1
     uint32_t *hidx;        // nslot: index of the slot's cell bitmap, or kEmpty32 (light slot)
     uint32_t *hbm;         // n_heavy x BRw words: bitmaps of the heavy slots' cell lists
@@ -200,6 +208,8 @@ size_t perm_check_workspace_bytes(uint32_t R, uint64_t n);
 int check_perm(flinng_index *ix, const uint32_t *perm, uint64_t n, void *ws);
 int check_groups(flinng_index *ix, const uint16_t *groups, uint64_t n);
 int check_result(flinng_index *ix);
+// mg1 from the records of the first n members
+int member_groups1(flinng_index *ix, uint64_t n);
 // Workspace of insert_hashed for n new points (reset: a build from scratch).
 size_t insert_workspace_bytes(const flinng_index *ix, uint64_t n, bool reset);
 int insert_hashed(flinng_index *ix, const uint32_t *buckets, const uint32_t *perm, const uint16_t *groups,

@@ -167,6 +167,7 @@ extern "C" int flinng_load(const char *path, void *stream, flinng_index **out)
     if (rc == FLINNG_OK) rc = undump(fh.f, ix->moff, uint64_t(ix->BR) + 1, st, buf);
     if (rc == FLINNG_OK) rc = undump(fh.f, ix->mem, uint64_t(cfg.R) * n, st, buf);
     if (rc == FLINNG_OK) rc = undump(fh.f, ix->mrec, n * ix->rw, st, buf);
+    if (rc == FLINNG_OK) rc = member_groups1(ix, n);
     if (rc == FLINNG_OK) rc = undump(fh.f, ix->off, ix->nslot + 1, st, buf);
     if (rc == FLINNG_OK) rc = undump(fh.f, ix->hidx, ix->nslot + 1, st, buf);
     if (rc == FLINNG_OK) rc = undump(fh.f, ix->cells, h.n_cells, st, buf);

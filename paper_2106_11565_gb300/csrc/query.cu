@@ -1,6 +1,8 @@
 // Host side of the batched query: launch shapes, shared-memory budgets,
 // the fused form's graphs and the autotuned shapes, and the count-width
 // dispatch. The kernels are in query_impl.cuh.
+#include <algorithm>
+
 #include "query_impl.cuh"
 
 namespace flinng {
@@ -22,6 +24,7 @@ QArgs make_args(flinng_index *ix, const uint32_t *qb, uint32_t nq)
     a.cells = ix->cells;
     a.moff = ix->moff;
     a.mrec = ix->mrec;
+    a.mg1 = ix->mg1;
     a.hidx = ix->hidx;
     a.hbm = ix->hbm;
     a.BRw = ix->BRw;
@@ -38,26 +41,33 @@ QArgs make_args(flinng_index *ix, const uint32_t *qb, uint32_t nq)
 }
 
 // Candidate buffer: room for one full round of members after a compaction
-// to k keys; tune->cap overrides the default when large enough.
-void pick_buffer(QArgs &a, int NT, const QueryTuning *tune, size_t extra, size_t *smem_out, int cw, int unroll)
+// to k keys; tune->cap overrides the default when large enough. The default is
+// kept small: the buffer's 8 bytes per entry cost resident CTAs (10^4 URL
+// queries, k = 10: 1.25 ms with 512 entries, 1.34 with 1,024).
+void pick_buffer(QArgs &a, int NT, const QueryTuning *tune, size_t extra, size_t *smem_out, int cw)
 {
     a.kp = pow2_at_least(a.k_max > 1 ? a.k_max : 2);
-    // the decode appends freely up to cap - (NT + 32) * unroll, then compacts:
-    // that mark must stay above the kp keys a compaction keeps
-    const uint32_t cap_min = pow2_at_least(a.kp + uint32_t(NT + 32) * unroll + 1);
-    uint32_t cap = (tune && tune->cap) ? pow2_at_least(tune->cap) : 2048;
+    // the decode appends freely up to cap - (NT + 32), then compacts: that
+    // mark must stay above the kp keys a compaction keeps
+    const uint32_t cap_min = pow2_at_least(a.kp + uint32_t(NT + 32) + 1);
+    uint32_t cap = pow2_at_least((tune && tune->cap) ? tune->cap : 4 * a.kp + uint32_t(NT + 32));
     if (cap < cap_min) cap = cap_min;
     a.cap = cap;
-    size_t smem = qsmem_bytes(a.cap, a.kp, a.BR, a.B, NT, a.L, cw);
+    a.lcap = a.B < kLevelCells ? (a.B + 7) & ~7u : kLevelCells;
+    size_t smem = qsmem_bytes(a.cap, a.kp, a.BR, a.lcap, NT, a.L, cw);
     while (smem + extra > 227 * 1024 && a.cap > cap_min) {
         a.cap >>= 1;
-        smem = qsmem_bytes(a.cap, a.kp, a.BR, a.B, NT, a.L, cw);
+        smem = qsmem_bytes(a.cap, a.kp, a.BR, a.lcap, NT, a.L, cw);
     }
     *smem_out = smem;
-    // a level group holds about 4,096 members: one stop check per group
+    // one stop check per level group: the first of about 1,024 members (4 k for
+    // larger k), then doubling to 16,384
     const uint32_t per = a.avg_cell ? a.avg_cell : 1u;
-    uint32_t g = 4096u / per;
-    a.gcells = g < 1 ? 1u : (g > uint32_t(NT) ? uint32_t(NT) : g);
+    const uint32_t g0 = std::max(1024u, 4 * a.k_max) / per;
+    a.gcells = std::min(std::max(g0, 1u), a.lcap);
+    a.gmax = std::min(std::max(16384u / per, a.gcells), a.lcap);
+    // eight members per lane need cells that fill them
+    a.wide = a.avg_cell >= 8 ? 1u : 0u;
 }
 
 }  // namespace
@@ -87,16 +97,20 @@ int query_launch_counts(flinng_index *ix, const uint32_t *qbuckets, const uint16
     a.out_ids = out_ids;
     a.out_scores = out_scores;
     a.out_row = out_row;
-    // CTA size: when shared memory admits only one or two CTAs per SM (large
-    // B*R), wider CTAs keep about 1,024 threads per SM decoding
+    // CTA size: the smallest that keeps the most threads on an SM (with large
+    // B*R shared memory admits only one or two CTAs)
     int NT = 256;
-    size_t smem;
-    pick_buffer(a, NT, nullptr, 0, &smem, cw, kPlainUnroll);
-    const size_t fit = (228 * 1024) / (smem + 1024);
-    if (fit < 4) {
-        NT = fit < 2 ? 1024 : 512;
-        pick_buffer(a, NT, nullptr, 0, &smem, cw, kPlainUnroll);
+    size_t smem = 0;
+    uint32_t most = 0;
+    for (int nt = 256; nt <= 1024; nt *= 2) {
+        pick_buffer(a, nt, nullptr, 0, &smem, cw);
+        const uint32_t on = std::min(kPlainThreads, uint32_t(228 * 1024 / (smem + 1024)) * nt);
+        if (on > most) {
+            most = on;
+            NT = nt;
+        }
     }
+    pick_buffer(a, NT, nullptr, 0, &smem, cw);
     if (smem > 227 * 1024)
         return set_error(FLINNG_ERR_INVALID_ARG,
                          "query: k_max=%u with B*R=%u needs %zu bytes of shared memory (> 227 KB)",
@@ -126,7 +140,8 @@ static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t 
                          uint32_t grid_for, FusedPlan *P)
 {
     const uint32_t nq = fq.nq;
-    const int NT = (tune && (tune->threads == 128 || tune->threads == 512)) ? int(tune->threads) : 256;
+    if (!ix->sms) FL_CUDA(cudaDeviceGetAttribute(&ix->sms, cudaDevAttrMultiProcessorCount, ix->device));
+    const int sms = ix->sms;
     QArgs &a = P->a;
     HArgs &h = P->h;
     a = make_args(ix, nullptr, nq);
@@ -166,15 +181,35 @@ static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t 
     // only before the decode keeps candidates, so it shares the candidate
     // buffer with the gather's heavy-table list (the buffer's last NT words)
     // when both fit; otherwise it follows the query state.
-    size_t qbytes;
-    pick_buffer(a, NT, tune, 0, &qbytes, int(ix->cw), 1);
-    if (hash_bytes + size_t(NT) * 4 <= size_t(a.cap) * 8) {
-        h.hash_off = 0;
-        P->smem = qbytes;
-    } else {
-        pick_buffer(a, NT, tune, hash_bytes, &qbytes, int(ix->cw), 1);
-        h.hash_off = qbytes;
-        P->smem = qbytes + hash_bytes;
+    auto shape = [&](int nt) {
+        size_t qbytes;
+        pick_buffer(a, nt, tune, 0, &qbytes, int(ix->cw));
+        if (hash_bytes + size_t(nt) * 4 <= size_t(a.cap) * 8) {
+            h.hash_off = 0;
+            P->smem = qbytes;
+        } else {
+            pick_buffer(a, nt, tune, hash_bytes, &qbytes, int(ix->cw));
+            h.hash_off = qbytes;
+            P->smem = qbytes + hash_bytes;
+        }
+    };
+    // CTA size, unless tuned. A batch that is resident at once takes 512 threads:
+    // it waits for its slowest query, whose phases scale with its CTA (1 query
+    // of the recall-target genomic index: 35 us with 512, 43 with 256, 65 with
+    // 128). A larger batch takes 256 when shared memory still admits four such
+    // CTAs per SM, so that more queries overlap their phases (10^4 URL queries:
+    // 1.24 ms against 1.46 with 512; 1,000 configured genomic queries: 35 us
+    // against 45), else 512.
+    int NT = tune && tune->threads ? int(tune->threads) : 512;
+    shape(NT);
+    if (!tune || !tune->threads) {
+        const uint32_t sm_threads = srp ? 1024 : 2048;     // the kernels' register bounds
+        const uint32_t fit = std::min(uint32_t(228 * 1024 / (P->smem + 1024)), sm_threads / 512);
+        if (fq.nq > uint32_t(sms) * fit) {
+            shape(256);
+            if (228 * 1024 / (P->smem + 1024) >= 4) NT = 256;
+            else shape(512);
+        }
     }
     if (P->smem > 227 * 1024)
         return set_error(FLINNG_ERR_INVALID_ARG, "fused query: %zu bytes of shared memory needed (> 227 KB)", P->smem);
@@ -192,8 +227,6 @@ static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t 
         const uint32_t slot = ix->n_occ < 8 ? ix->n_occ++ : 7;
         ix->occ[slot] = OccEntry{P->fn, NT, P->smem, per_sm};
     }
-    if (!ix->sms) FL_CUDA(cudaDeviceGetAttribute(&ix->sms, cudaDevAttrMultiProcessorCount, ix->device));
-    const int sms = ix->sms;
     uint32_t want = (tune && tune->ctas_per_sm) ? tune->ctas_per_sm : uint32_t(per_sm);
     if (want > uint32_t(per_sm)) want = per_sm;
     uint64_t grid = uint64_t(sms) * want;
@@ -287,7 +320,7 @@ int counts_launch(flinng_index *ix, const uint32_t *qbuckets, uint32_t nq,
     a.cap = kQTmax / 2;      // the heavy-table list takes the buffer's last kQTmax words
     a.kp = 2;
     a.out_counts = out_counts;
-    const size_t smem = qsmem_bytes(a.cap, a.kp, a.BR, a.B, kQTmax, a.L, int(ix->cw));
+    const size_t smem = qsmem_bytes(a.cap, a.kp, a.BR, a.lcap, kQTmax, a.L, int(ix->cw));
     const void *fn = ix->cw == 1 ? counts_kernel_c1() : counts_kernel_c2();
     FL_TRY(ensure_dyn_smem(fn, smem));
     void *args[] = {&a};
