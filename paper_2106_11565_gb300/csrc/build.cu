@@ -7,7 +7,8 @@
 // Member lists: the points of cell c = r*B + b, a counting sort of all points
 // by cell (histogram, scan, scatter).
 //
-// Reverse index: every (point, table l) contributes the R cells r*B + gid_r to
+// Reverse index (from scratch with R >= 2: build_part.cu; this general path
+// otherwise, and for large inserts): every (point, table l) contributes the R cells r*B + gid_r to
 // the list of slot (l, bucket). A counting sort on the slot - a one-digit
 // radix sort whose digit is the whole (table, bucket) key - places old lists
 // and new entries in one array; each slot is then sorted and deduplicated (a
@@ -516,24 +517,32 @@ __global__ void k_heavy_collect(const uint32_t *__restrict__ off, uint64_t nslot
     }
 }
 
-// Warp per heavy slot: its cell bitmap.
-__global__ void k_heavy_fill(const uint32_t *__restrict__ off, const uint16_t *__restrict__ cells,
-                             const uint32_t *__restrict__ list, uint32_t nh, uint32_t BRw,
-                             uint32_t *__restrict__ hbm)
+// Warp per heavy slot: its cell bitmap, collected in shared memory (the list's
+// cells are random words of the row) and written as one coalesced row.
+__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+k_heavy_fill(const uint32_t *__restrict__ off, const uint16_t *__restrict__ cells,
+             const uint32_t *__restrict__ list, uint32_t nh, uint32_t BRw, uint32_t *__restrict__ hbm)
 {
-    const int lane = threadIdx.x & 31;
-    const uint64_t gw = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nw = (uint64_t(gridDim.x) * blockDim.x) >> 5;
-    for (uint64_t i = gw; i < nh; i += nw) {
+    extern __shared__ uint32_t bm_all[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *bm = bm_all + warp * BRw;
+    constexpr uint32_t kU = 4;                       // cells in flight per lane
+    for (uint32_t i = blockIdx.x * kWarpsPerBlock + warp; i < nh; i += gridDim.x * kWarpsPerBlock) {
         const uint32_t s = list[i];
-        uint32_t *bm = hbm + i * BRw;
         for (uint32_t w = lane; w < BRw; w += 32) bm[w] = 0u;
-        __syncwarp();
         const uint32_t beg = off[s], end = off[s + 1];
-        for (uint32_t t = beg + lane; t < end; t += 32) {
-            const uint32_t c = cells[t];
-            atomicOr(&bm[c >> 5], 1u << (c & 31));
+        __syncwarp();
+        for (uint32_t t = beg + lane; t < end; t += 32 * kU) {
+            uint32_t c[kU];
+#pragma unroll
+            for (uint32_t u = 0; u < kU; ++u) c[u] = t + 32 * u < end ? uint32_t(cells[t + 32 * u]) : 0u;
+#pragma unroll
+            for (uint32_t u = 0; u < kU; ++u)
+                if (t + 32 * u < end) atomicOr(&bm[c[u] >> 5], 1u << (c[u] & 31));
         }
+        __syncwarp();
+        uint32_t *row = hbm + uint64_t(i) * BRw;
+        for (uint32_t w = lane; w < BRw; w += 32) row[w] = bm[w];
         __syncwarp();
     }
 }
@@ -543,9 +552,8 @@ __global__ void k_heavy_fill(const uint32_t *__restrict__ off, const uint16_t *_
 // Cell bitmaps of the heavy slots (those whose list has >= heavy_min cells).
 // Uses a word of the build scratch slot_a and a worklist of at least
 // n_cells / heavy_min + 1 entries; grows the bitmap array if needed.
-int build_heavy(flinng_index *ix, void *scan_ws, uint32_t *list)
+int build_heavy(flinng_index *ix, uint32_t *list)
 {
-    (void)scan_ws;
     const cudaStream_t st = ix->stream;
     const uint64_t nslot = ix->nslot;
     uint32_t *count = ix->slot_a;        // build scratch, free at this point
@@ -554,6 +562,13 @@ int build_heavy(flinng_index *ix, void *scan_ws, uint32_t *list)
                                                                     count);
     count_launch();
     FL_CUDA(cudaGetLastError());
+    return heavy_bitmaps(ix, list, count);
+}
+
+// The bitmaps of the listed heavy slots (hidx has their rows).
+int heavy_bitmaps(flinng_index *ix, const uint32_t *list, const uint32_t *count)
+{
+    const cudaStream_t st = ix->stream;
     FL_CUDA(cudaMemcpyAsync(ix->h_flag, count, 4, cudaMemcpyDeviceToHost, st));
     FL_CUDA(cudaStreamSynchronize(st));
     const uint32_t nh = *ix->h_flag;
@@ -575,8 +590,9 @@ int build_heavy(flinng_index *ix, void *scan_ws, uint32_t *list)
     if (nh > 0 && (!ix->hbm || ix->hbm_words < words))
         return set_error(FLINNG_ERR_OOM, "internal: no storage for %u cell bitmaps", nh);
     if (nh > 0) {
-        k_heavy_fill<<<warp_blocks(nh), kWarpsPerBlock * 32, 0, st>>>(ix->off, ix->cells, list, nh, ix->BRw,
-                                                                     ix->hbm);
+        const size_t smem = size_t(kWarpsPerBlock) * ix->BRw * sizeof(uint32_t);
+        FL_TRY(ensure_dyn_smem((const void *)k_heavy_fill, smem));
+        k_heavy_fill<<<warp_blocks(nh), kWarpsPerBlock * 32, smem, st>>>(ix->off, ix->cells, list, nh, ix->BRw, ix->hbm);
         count_launch();
         FL_CUDA(cudaGetLastError());
     }
@@ -631,6 +647,9 @@ uint64_t worklist_entries(const flinng_index *ix, uint64_t n, bool reset)
 
 size_t insert_workspace_bytes(const flinng_index *ix, uint64_t n, bool reset)
 {
+    if ((reset || ix->n_points == 0) && part_build_applies(ix, n))
+        return carve_bytes<uint32_t>(ix->BR + 1) +
+               std::max(part_workspace_bytes(ix, n), scan_workspace_bytes(size_t(ix->BR) + 1)) + 256;
     if (!reset && delta_insert_applies(ix, n))
         return carve_bytes<uint32_t>(ix->BR + 1) +
                std::max(delta_workspace_bytes(ix, n), scan_workspace_bytes(size_t(ix->BR) + 1)) + 256;
@@ -707,7 +726,7 @@ int member_stage(flinng_index *ix, const uint32_t *perm, const uint16_t *groups,
 
 }  // namespace
 
-int insert_hashed(flinng_index *ix, const uint32_t *buckets, const uint32_t *perm, const uint16_t *groups,
+int insert_hashed(flinng_index *ix, uint32_t *buckets, const uint32_t *perm, const uint16_t *groups,
                   uint64_t n, void *ws)
 {
     const cudaStream_t st = ix->stream;
@@ -725,6 +744,23 @@ int insert_hashed(flinng_index *ix, const uint32_t *buckets, const uint32_t *per
         FL_TRY(member_stage(ix, perm, groups, n, mcur, dws));
         TraceRange stage2("reverse index (delta)");
         return insert_delta(ix, buckets, n, dws);
+    }
+    if (n_old == 0 && part_build_applies(ix, n)) {
+        // from scratch: sorted partition by partition in shared memory
+        void *pws = c.base + ((c.used + 255) & ~size_t(255));
+        FL_TRY(member_stage(ix, perm, groups, n, mcur, pws));
+        TraceRange stage2("reverse index (partitioned)");
+        uint32_t *list, *count;
+        FL_TRY(part_build(ix, buckets, n, pws, &list, &count));
+        std::swap(ix->off, ix->slot_b);
+        FL_CUDA(cudaMemcpyAsync(ix->h_flag + 1, ix->off + nslot, 4, cudaMemcpyDeviceToHost, st));
+        stage2.end();
+        TraceRange stage3("heavy bitmaps");
+        const int rc = heavy_bitmaps(ix, list, count);
+        if (rc != FLINNG_OK) cudaStreamSynchronize(st);
+        ix->n_cells = ix->h_flag[1];
+        ix->n_points = N;
+        return rc;
     }
     uint32_t *dtoff = c.take<uint32_t>(nslot + 1);     // new entries of slot s start here
     uint32_t *cursor = c.take<uint32_t>(nslot + 1);    // scatter cursors, then merged lengths
@@ -797,7 +833,7 @@ int insert_hashed(flinng_index *ix, const uint32_t *buckets, const uint32_t *per
     FL_CUDA(cudaMemcpyAsync(ix->h_flag + 1, ix->off + nslot, 4, cudaMemcpyDeviceToHost, st));
     stage2.end();
     TraceRange stage3("heavy bitmaps");
-    const int rc = build_heavy(ix, scan_ws, work);
+    const int rc = build_heavy(ix, work);
     if (rc != FLINNG_OK) cudaStreamSynchronize(st);    // the lists are in place either way
     ix->n_cells = ix->h_flag[1];
     ix->n_points = N;

@@ -212,9 +212,18 @@ int check_result(flinng_index *ix);
 int member_groups1(flinng_index *ix, uint64_t n);
 // Workspace of insert_hashed for n new points (reset: a build from scratch).
 size_t insert_workspace_bytes(const flinng_index *ix, uint64_t n, bool reset);
-int insert_hashed(flinng_index *ix, const uint32_t *buckets, const uint32_t *perm, const uint16_t *groups,
-                  uint64_t n, void *ws);
-int build_heavy(flinng_index *ix, void *scan_ws, uint32_t *list);
+// buckets: n x L in the workspace (may be overwritten)
+int insert_hashed(flinng_index *ix, uint32_t *buckets, const uint32_t *perm, const uint16_t *groups, uint64_t n,
+                  void *ws);
+int build_heavy(flinng_index *ix, uint32_t *list);
+int heavy_bitmaps(flinng_index *ix, const uint32_t *list, const uint32_t *count);
+
+// ---- build_part.cu
+// A build from scratch sorts its entries partition by partition in shared
+// memory where part_build_applies.
+bool part_build_applies(const flinng_index *ix, uint64_t n);
+size_t part_workspace_bytes(const flinng_index *ix, uint64_t n);
+int part_build(flinng_index *ix, uint32_t *buckets, uint64_t n, void *ws, uint32_t **list_out, uint32_t **count_out);
 
 // ---- query.cu
 struct FusedQuery {
