@@ -373,7 +373,10 @@ int flinng_hash_stats(const flinng_index *idx, uint64_t *n_recheck,
 /* All counters of the last cosine hash, or query (Sec. 3.2 signs), on this
  * index: out[0] projections the first pass (fp32 FMA or tensor cores) could
  * not decide; out[1] those decided by the exact accumulator; out[2] fp64
- * re-checks; out[3] compensated fp32 re-checks (tensor-core precision only);
+ * re-checks; out[3] second-stage re-checks of the tensor-core precisions
+ * (compensated fp32, or a dense pass on the two-term split for a large batch of
+ * a single-term form; none for a batch of at most 96 rows, which every
+ * precision hashes in fp32 unless projections are asked for);
  * out[4] flips: first-pass signs that a re-check reversed (the hash-bit flip
  * rate before re-check is out[4] / (n * L * K)). out: 5 HOST uint64, written
  * after the index's stream is synchronised. Errors: INVALID_ARG for NULL. */

@@ -96,10 +96,10 @@ void free_index(flinng_index *ix)
 {
     if (!ix) return;
     destroy_graphs(ix);
-    void *ptrs[] = {ix->srp_w, ix->bucket_a, ix->bucket_c, ix->gid, ix->moff, ix->mem, ix->mrec, ix->mg1, ix->off,
+    void *ptrs[] = {ix->srp_w, ix->bucket_a, ix->bucket_c, ix->gid, ix->moff, ix->mem, ix->mrec, ix->off,
                     ix->hidx, ix->hbm,
                     ix->cells, ix->cells_tmp, ix->slot_a, ix->slot_b, ix->cell_cnt, ix->flag, ix->qnext,
-                    ix->stats, ix->ws.ptr, ix->w_split, ix->w_norm, ix->w_aux, ix->tc_err};
+                    ix->stats, ix->ws.ptr, ix->w_split, ix->w_aux, ix->tc_err};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (ix->h_flag) cudaFreeHost(ix->h_flag);
@@ -385,7 +385,8 @@ int flinng_create(const flinng_config *cfg, const flinng_params *params, void *s
 #define ALLOC(ptr, n)                                      \
     if (rc == FLINNG_OK) rc = dalloc(ix, &ix->ptr, (n));
     if (cfg->metric == FLINNG_COSINE_SRP) {
-        ALLOC(srp_w, size_t(ix->P) * cfg->dim);
+        ALLOC(srp_w, size_t(ix->P) * cfg->dim + ix->P);     // then the rows' norms
+        if (rc == FLINNG_OK) ix->w_norm = ix->srp_w + size_t(ix->P) * cfg->dim;
     } else {
         ALLOC(bucket_a, size_t(ix->P));
         ALLOC(bucket_c, size_t(L));
@@ -393,8 +394,9 @@ int flinng_create(const flinng_config *cfg, const flinng_params *params, void *s
     ALLOC(gid, size_t(cfg->capacity) * ix->rp);
     ALLOC(moff, size_t(ix->BR) + 1);
     ALLOC(mem, size_t(R) * cfg->capacity);
-    ALLOC(mrec, size_t(ix->rw) * cfg->capacity);
-    ALLOC(mg1, size_t(cfg->capacity) + kMg1Pad);
+    const size_t rec_words = (size_t(ix->rw) * cfg->capacity + 3) & ~size_t(3);   // mg1 behind it, 16-byte aligned
+    ALLOC(mrec, rec_words + (size_t(cfg->capacity) + kMg1Pad + 1) / 2);
+    if (rc == FLINNG_OK) ix->mg1 = reinterpret_cast<uint16_t *>(ix->mrec + rec_words);
     ALLOC(off, ix->nslot + 1);
     ALLOC(hidx, ix->nslot + 1);
     ALLOC(cells, ix->entries_cap + kCellPad);
@@ -444,7 +446,8 @@ int flinng_create(const flinng_config *cfg, const flinng_params *params, void *s
         chk(cudaStreamCreateWithFlags(&ix->side, cudaStreamNonBlocking), "create side stream");
         chk(cudaEventCreateWithFlags(&ix->ev_fork, cudaEventDisableTiming), "create event");
         chk(cudaEventCreateWithFlags(&ix->ev_join, cudaEventDisableTiming), "create event");
-        if (rc == FLINNG_OK && cfg->precision != FLINNG_PREC_FP32) rc = srp_tc_prepare_weights(ix);
+        if (rc == FLINNG_OK && cfg->metric == FLINNG_COSINE_SRP)
+            rc = cfg->precision != FLINNG_PREC_FP32 ? srp_tc_prepare_weights(ix) : srp_weight_norms(ix);
         chk(cudaStreamSynchronize(st), "create sync");
     }
     if (rc != FLINNG_OK) {

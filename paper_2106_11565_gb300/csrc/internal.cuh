@@ -110,7 +110,7 @@ struct flinng_index {
     float srp_margin_gamma;   // 2 * gamma_d in fp32, rounded up
     double srp_gamma64;       // 2 * gamma_d for the fp64 recheck
     void *w_split;            // tensor-core precision: bf16 w1 then w2, P x dim each
-    float *w_norm;            // upper bounds of ||w_j||
+    float *w_norm;            // upper bounds of ||w_j|| (behind srp_w)
     float *w_aux;             // single-term tensor forms: P upper bounds of ||w_j - q(w_j)||, then P row scales
     uint32_t *tc_err;         // tensor-core pipeline timeout flag
     uint64_t tc_wait_ns;      // limit of the tensor-core pipeline's waits + 1 (0: the default)
@@ -132,7 +132,7 @@ struct flinng_index {
     uint32_t *mem;         // R * capacity point ids
     uint32_t *mrec;        // capacity * rw: repetition-0 members with their other group ids
     uint16_t *mg1;         // capacity + kMg1Pad: the members' repetition-1 groups alone, in mrec's
-                           // order (padding and unused entries are valid group ids)
+                           // order (padding and unused entries are valid group ids); behind mrec
     uint32_t *off;         // nslot + 1
     uint32_t *hidx;        // nslot: index of the slot's cell bitmap, or kEmpty32 (light slot)
     uint32_t *hbm;         // n_heavy x BRw words: bitmaps of the heavy slots' cell lists
@@ -192,6 +192,8 @@ int doph_hash(flinng_index *ix, const uint64_t *off, const uint32_t *elems,
 // fp64 / exact re-check of listed (row << 20 | projection) entries
 int srp_recheck_list(flinng_index *ix, const float *x, uint64_t ld, const unsigned long long *list,
                      const unsigned long long *count, uint32_t *codes);
+// w_norm: upper bounds of the projection rows' norms
+int srp_weight_norms(flinng_index *ix);
 int add_counter(unsigned long long *dst, const unsigned long long *src, cudaStream_t st);
 
 // ---- srp_tc.cu (tensor-core precision form)

@@ -128,7 +128,7 @@ struct flinng_server {
     uint64_t bytes_used = 0;
     // sizes the slots are laid out for (maximum over the indices)
     uint32_t max_L = 0, max_dim = 0;
-    uint64_t max_P = 0;
+    uint64_t max_srp = 0;         // hash workspace of a full batch
     bool device_gather = false;   // the GPU reads requests' host buffers directly
     cudaEvent_t ref = nullptr;    // recorded when a replay begins: origin of the device times
 };
@@ -166,7 +166,7 @@ Layout layout_for(const flinng_server *srv)
     L.in_el = (size_t)c.take<uint32_t>(in_floats > in_elems ? in_floats : in_elems);
     L.qb = (size_t)c.take<uint32_t>(nb * srv->max_L);
     // re-check lists (fp32 path) or the tensor-core split operands and lists
-    L.srp = (size_t)c.take<unsigned long long>(2 * nb * srv->max_P + 64 + nb * srv->max_dim / 2 + 2 * nb + 1024);
+    L.srp = (size_t)c.take<char>(srv->max_srp);
     L.ids = (size_t)c.take<uint32_t>(nb * km);
     L.sc = (size_t)c.take<uint16_t>(nb * km);
     L.total = c.used + 256;
@@ -275,7 +275,7 @@ int launch_batch(flinng_server *srv, Slot &slot, const flinng_request *reqs, uin
     if (big_srp) {
         uint32_t *qb = reinterpret_cast<uint32_t *>(d + Lo.qb);
         rc = srp_hash(ix, reinterpret_cast<const float *>(d + Lo.in_el), ix->cfg.dim, nb, qb, nullptr, d + Lo.srp,
-                      (2 * size_t(nb) * ix->P + 64) * 8);
+                      srv->max_srp);
         if (slot.direct) {
             dids = out_ids;
             dsc = out_scores;
@@ -374,11 +374,12 @@ int flinng_server_add_index(flinng_server *srv, flinng_index *ix, uint32_t *inde
     if (!srv || !ix) return set_error(FLINNG_ERR_INVALID_ARG, "server: null argument");
     if (ix->probes > 1) return set_error(FLINNG_ERR_INVALID_ARG, "server: multi-probe indices are not served");
     const uint32_t L0 = srv->max_L, d0 = srv->max_dim;
-    const uint64_t P0 = srv->max_P;
+    const uint64_t s0 = srv->max_srp;
     if (ix->cfg.L > srv->max_L) srv->max_L = ix->cfg.L;
     if (ix->cfg.metric == FLINNG_COSINE_SRP) {
         if (ix->cfg.dim > srv->max_dim) srv->max_dim = ix->cfg.dim;
-        if (ix->P > srv->max_P) srv->max_P = ix->P;
+        const uint64_t need_srp = srp_workspace_bytes(ix, srv->cfg.max_batch);
+        if (need_srp > srv->max_srp) srv->max_srp = need_srp;
     }
     const Layout Lo = layout_for(srv);
     const uint64_t slots_bytes = uint64_t(Lo.total) * srv->slots.size();
@@ -388,7 +389,7 @@ int flinng_server_add_index(flinng_server *srv, flinng_index *ix, uint32_t *inde
     if (others + need > srv->cfg.hbm_budget) {
         srv->max_L = L0;
         srv->max_dim = d0;
-        srv->max_P = P0;
+        srv->max_srp = s0;
         return set_error(FLINNG_ERR_OOM, "server: index needs %llu bytes, %llu of the %llu-byte budget are taken",
                          (unsigned long long)need, (unsigned long long)others,
                          (unsigned long long)srv->cfg.hbm_budget);

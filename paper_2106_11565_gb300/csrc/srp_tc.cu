@@ -55,6 +55,7 @@
 #include <cuda_fp8.h>
 
 #include "internal.cuh"
+#include "srp_rows.cuh"
 
 namespace flinng {
 namespace {
@@ -236,6 +237,10 @@ struct TcArgs {
     float *proj;           // optional n x P
     unsigned long long *rlist;
     unsigned long long *rcount;
+    uint32_t *mask;        // dense second pass: per row ceil(P / 32) words of undecided projections, then as
+                           // many of their first-pass signs
+    unsigned long long *nund;    // masks written: undecided projections
+    unsigned long long *stats;   // masks read: the hash counters
     uint32_t *err;         // set to 1 on a wait timeout
     uint64_t wait_ns;      // limit of the pipeline's waits (the drains after an abort keep kWaitNs)
 };
@@ -245,7 +250,11 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-template <int FORM>
+// MASK: 0 undecided projections are listed; 1 they are marked in a.mask (the
+// first pass of a single-term form whose undecided share is large); 2 only the
+// marked ones are decided (its second pass, on the two-term split), the rest
+// listed.
+template <int FORM, int MASK>
 __global__ void __launch_bounds__(kTcThreads, 1)
 k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtensorMap mx2,
          const __grid_constant__ CUtensorMap mw1, const __grid_constant__ CUtensorMap mw2, TcArgs a)
@@ -419,10 +428,23 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
             if constexpr (FORM != kFormBf16x2) xr = a.xres[row];
             if constexpr (FORM == kFormFp8) xs = a.xscale[row];
             uint32_t cur_l = 0xFFFFFFFFu, cur_bits = 0u;
+            // this thread's two words of the masks: undecided, first-pass signs
+            const uint32_t pw = (a.P + 31) / 32, w0 = (col0 + 64u * half) / 32;
+            uint32_t und[2] = {0u, 0u}, sgn[2] = {0u, 0u}, decided = 0u, flips = 0u;
+            uint32_t *mrow = MASK ? a.mask + row * (2 * pw) + w0 : nullptr;
+            if constexpr (MASK == 2) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    if (w0 + i < pw) {
+                        und[i] = mrow[i];
+                        sgn[i] = mrow[pw + i];
+                    }
+            }
 #pragma unroll
             for (int j = 0; j < 64; ++j) {
                 const uint32_t col = col0 + 64u * half + j;
                 if (col >= a.P) break;
+                if (MASK == 2 && !((und[j / 32] >> (j % 32)) & 1u)) continue;
                 float p = acc[j];
                 if constexpr (FORM == kFormFp8) p *= xs * a.wscale[col];    // powers of two: exact
                 const float wn = a.wnorm[col];
@@ -440,6 +462,10 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
                              (1.f + ldexpf(1.f, -20));
                 }
                 if (fabsf(p) > margin) {
+                    if constexpr (MASK == 2) {
+                        ++decided;
+                        flips += (p > 0.f) != (((sgn[j / 32] >> (j % 32)) & 1u) != 0u) ? 1u : 0u;
+                    }
                     if (p > 0.f) {
                         const uint32_t l = col / a.K;
                         if (l != cur_l) {
@@ -449,12 +475,31 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
                         }
                         cur_bits |= 1u << (col % a.K);
                     }
+                } else if constexpr (MASK == 1) {
+                    und[j / 32] |= 1u << (j % 32);
+                    if (p > 0.f) sgn[j / 32] |= 1u << (j % 32);
                 } else {
+                    // the tentative sign a later re-check may reverse is the first pass's
+                    const bool pos = MASK == 2 ? ((sgn[j / 32] >> (j % 32)) & 1u) != 0u : p > 0.f;
                     const unsigned long long slot = atomicAdd(a.rcount, 1ull);
-                    a.rlist[slot] = (p > 0.f ? kEntSign : 0ull) | ((unsigned long long)row << 20) | col;
+                    a.rlist[slot] = (pos ? kEntSign : 0ull) | ((unsigned long long)row << 20) | col;
                 }
             }
             if (cur_bits) atomicOr(&a.codes[row * a.L + cur_l], cur_bits);
+            if constexpr (MASK == 1) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    if (w0 + i < pw) {
+                        mrow[i] = und[i];
+                        mrow[pw + i] = sgn[i];
+                    }
+                const uint32_t c = __popc(und[0]) + __popc(und[1]);
+                if (c) atomicAdd(a.nund, (unsigned long long)c);
+            }
+            if constexpr (MASK == 2) {
+                if (decided) atomicAdd(&a.stats[3], (unsigned long long)decided);
+                if (flips) atomicAdd(&a.stats[4], (unsigned long long)flips);
+            }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -477,39 +522,98 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
     __syncthreads();
 }
 
-// x -> (bf16(x), bf16(x - bf16(x))) and an upper bound of each row's norm
+// Upper bounds of a row's norm and of its residual's norm, by one warp, from
+// the lanes' fp32 sums of squares (at most m roundings each). The residuals are
+// exact in fp32 (a float minus its rounding to fewer bits); squares lost to
+// underflow are covered by the range check for the row and by an absolute term
+// for the residual. Out of range (values near 1e18 or 1e-14 alone): fp64.
+template <class Residual>
+__device__ __forceinline__ void row_bounds(float ss, float rr, bool any, const float *xr, uint32_t d, Residual res_of,
+                                           float *norm, float *res)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        ss += __shfl_xor_sync(0xffffffffu, ss, o);
+        rr += __shfl_xor_sync(0xffffffffu, rr, o);
+    }
+    any = __any_sync(0xffffffffu, any);
+    if (norm_in_range(ss, any)) {
+        *norm = norm_up(ss, d / 32 + 16);
+        *res = norm_up(__fadd_ru(rr, any ? float(d) * 0x1p-148f : 0.f), d / 32 + 16);
+        return;
+    }
+    double s64 = 0.0, r64 = 0.0;
+    for (uint32_t t = lane; t < d; t += 32) {
+        const double v = xr[t], e = res_of(xr[t]);
+        s64 += v * v;
+        r64 += e * e;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s64 += __shfl_xor_sync(0xffffffffu, s64, o);
+        r64 += __shfl_xor_sync(0xffffffffu, r64, o);
+    }
+    *norm = norm_up64(s64);
+    *res = norm_up64(r64);
+}
+
+__device__ __forceinline__ uint2 pack_bf16x4(__nv_bfloat16 a, __nv_bfloat16 b, __nv_bfloat16 c, __nv_bfloat16 d)
+{
+    return make_uint2(uint32_t(__bfloat16_as_ushort(a)) | uint32_t(__bfloat16_as_ushort(b)) << 16,
+                      uint32_t(__bfloat16_as_ushort(c)) | uint32_t(__bfloat16_as_ushort(d)) << 16);
+}
+
+// x -> x1 = bf16(x) and, TWO, x2 = bf16(x - x1); upper bounds of each row's
+// norm and of ||x - x1||. A warp per row, four floats per lane and step (d is a
+// multiple of 8, so the 8-byte stores are aligned). Bound by the bytes: 10^4
+// rows of 4,096 split in 178 us with fp64 sums of squares (the FP64 pipe's
+// rate) and 4-byte loads, in 52 us (6.3 TB/s) now.
+template <bool VEC, bool TWO>
 __global__ void k_split_rows(const float *__restrict__ x, uint64_t ld, uint64_t n, uint32_t d,
                              __nv_bfloat16 *__restrict__ x1, __nv_bfloat16 *__restrict__ x2,
-                             float *__restrict__ norm)
+                             float *__restrict__ norm, float *__restrict__ res)
 {
     const int lane = threadIdx.x & 31;
     const uint64_t gw = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const uint64_t nw = (uint64_t(gridDim.x) * blockDim.x) >> 5;
     for (uint64_t r = gw; r < n; r += nw) {
-        double ss = 0.0;
-        for (uint32_t t = lane; t < d; t += 32) {
-            const float v = x[r * ld + t];
-            const __nv_bfloat16 h = __float2bfloat16_rn(v);
-            const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
-            x1[r * d + t] = h;
-            x2[r * d + t] = l;
-            ss += double(v) * double(v);
-        }
+        const float *xr = x + r * ld;
+        float ss = 0.f, rr = 0.f;
+        bool any = false;
+#pragma unroll 4
+        for (uint32_t t = lane * 4; t < d; t += 128) {
+            const float4 q = load4<VEC>(xr, t, d, true);
+            const float v[4] = {q.x, q.y, q.z, q.w};
+            __nv_bfloat16 h[4], l[4];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        // fp64 sum of d squares, sqrt, rounded up with room to spare
-        if (lane == 0) norm[r] = __double2float_ru(sqrt(ss * (1.0 + 1e-12)) * (1.0 + 1e-7));
+            for (int i = 0; i < 4; ++i) {
+                h[i] = __float2bfloat16_rn(v[i]);
+                const float e = v[i] - __bfloat162float(h[i]);
+                l[i] = __float2bfloat16_rn(e);
+                ss = fmaf(v[i], v[i], ss);
+                rr = fmaf(e, e, rr);
+                any |= v[i] != 0.f;
+            }
+            *reinterpret_cast<uint2 *>(x1 + r * d + t) = pack_bf16x4(h[0], h[1], h[2], h[3]);
+            if constexpr (TWO) *reinterpret_cast<uint2 *>(x2 + r * d + t) = pack_bf16x4(l[0], l[1], l[2], l[3]);
+        }
+        float nrm, rn;
+        row_bounds(ss, rr, any, xr, d,
+                   [](float v) { return double(v) - double(__bfloat162float(__float2bfloat16_rn(v))); }, &nrm, &rn);
+        if (lane == 0) {
+            norm[r] = nrm;
+            if (res) res[r] = rn;
+        }
     }
 }
 
-// Single-term quantisers: q = bf16(x) (FORM kFormBf16) or q = e4m3(x / s) with
-// s = 2^e, e the smallest with max |x| / s < 448 (FORM kFormFp8; a value whose
-// quantised magnitude would be below 2^-6, an E4M3 subnormal, becomes 0). Per
-// row: upper bounds of ||x|| and of ||x - s q|| (exact fp64 differences, fp64
-// sums of squares, rounded up), and s.
-template <int FORM>
+// E4M3 rows: q = e4m3(x / s) with s = 2^e, e the smallest with max |x| / s < 448
+// (a value whose quantised magnitude would be below 2^-6, an E4M3 subnormal,
+// becomes 0). Per row: upper bounds of ||x|| and of ||x - s q||, and s.
+template <bool VEC>
 __global__ void k_quant_rows(const float *__restrict__ x, uint64_t ld, uint64_t n, uint32_t d,
-                             void *__restrict__ q, float *__restrict__ norm, float *__restrict__ res,
+                             __nv_fp8_e4m3 *__restrict__ q, float *__restrict__ norm, float *__restrict__ res,
                              float *__restrict__ scale)
 {
     const int lane = threadIdx.x & 31;
@@ -517,58 +621,57 @@ __global__ void k_quant_rows(const float *__restrict__ x, uint64_t ld, uint64_t 
     const uint64_t nw = (uint64_t(gridDim.x) * blockDim.x) >> 5;
     for (uint64_t r = gw; r < n; r += nw) {
         const float *xr = x + r * ld;
+        float mx = 0.f;
+#pragma unroll 4
+        for (uint32_t t = lane * 4; t < d; t += 128) {
+            const float4 v = load4<VEC>(xr, t, d, true);
+            mx = fmaxf(mx, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         float s = 1.f;
-        if constexpr (FORM == kFormFp8) {
-            float mx = 0.f;
-            for (uint32_t t = lane; t < d; t += 32) mx = fmaxf(mx, fabsf(xr[t]));
+        if (mx > 0.f) {
+            int e;
+            frexpf(mx / 448.f, &e);      // mx / 448 = f 2^e with f in [0.5, 1): mx / 2^e < 448
+            s = ldexpf(1.f, e);
+        }
+        auto quant = [&](float v) {
+            __nv_fp8_e4m3 h(v / s);                       // round to nearest, saturating
+            if (fabsf(float(h)) < 0x1p-6f) h = __nv_fp8_e4m3(0.f);
+            return h;
+        };
+        float ss = 0.f, rr = 0.f;
+#pragma unroll 2
+        for (uint32_t t = lane * 4; t < d; t += 128) {
+            const float4 v4 = load4<VEC>(xr, t, d, true);
+            const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+            uint32_t w = 0;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-            if (mx > 0.f) {
-                int e;
-                frexpf(mx / 448.f, &e);      // mx / 448 = f 2^e with f in [0.5, 1): mx / 2^e < 448
-                s = ldexpf(1.f, e);
+            for (int i = 0; i < 4; ++i) {
+                const __nv_fp8_e4m3 h = quant(v[i]);
+                w |= uint32_t(h.__x) << (8 * i);
+                const float e = v[i] - float(h) * s;      // exact: s is a power of two
+                ss = fmaf(v[i], v[i], ss);
+                rr = fmaf(e, e, rr);
             }
+            *reinterpret_cast<uint32_t *>(q + r * d + t) = w;
         }
-        double ss = 0.0, rr = 0.0;
-        for (uint32_t t = lane; t < d; t += 32) {
-            const float v = xr[t];
-            float back;
-            if constexpr (FORM == kFormBf16) {
-                const __nv_bfloat16 h = __float2bfloat16_rn(v);
-                static_cast<__nv_bfloat16 *>(q)[r * d + t] = h;
-                back = __bfloat162float(h);
-            } else {
-                __nv_fp8_e4m3 h(v / s);                       // round to nearest, saturating
-                float hf = float(h);
-                if (fabsf(hf) < ldexpf(1.f, -6)) {
-                    h = __nv_fp8_e4m3(0.f);
-                    hf = 0.f;
-                }
-                static_cast<__nv_fp8_e4m3 *>(q)[r * d + t] = h;
-                back = hf * s;                                // exact: s is a power of two
-            }
-            const double e = double(v) - double(back);        // exact in fp64
-            ss += double(v) * double(v);
-            rr += e * e;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            ss += __shfl_xor_sync(0xffffffffu, ss, o);
-            rr += __shfl_xor_sync(0xffffffffu, rr, o);
-        }
+        float nrm, rn;
+        row_bounds(ss, rr, mx > 0.f, xr, d, [&](float v) { return double(v) - double(float(quant(v)) * s); }, &nrm, &rn);
         if (lane == 0) {
-            // fp64 sums of d squares, sqrt, rounded up with room to spare
-            norm[r] = __double2float_ru(sqrt(ss * (1.0 + 1e-12)) * (1.0 + 1e-7));
-            res[r] = __double2float_ru(sqrt(rr * (1.0 + 1e-12)) * (1.0 + 1e-7));
-            if (scale) scale[r] = s;
+            norm[r] = nrm;
+            res[r] = rn;
+            scale[r] = s;
         }
     }
 }
 
 // Compensated fp32 re-check of listed projections: two-product and two-sum
 // per term (one warp per projection), error at most 2^-23 |p| + 2 g(2d)^2 S
-// with S = sum |w x|. Decided bits are set; the rest go to the next list.
-// xr: the entry's row of x (global or shared memory).
+// with S = sum |w x|, in any order of the sums. Decided bits are set; the rest
+// go to the next list. xr: the entry's row of x (global or shared memory). The
+// rows of W are 16-byte aligned (d % 8 == 0).
+template <bool VEC>
 __device__ __forceinline__ void recheck2_entry(const float *xr, const float *__restrict__ Wm, uint32_t d,
                                                uint32_t L, uint32_t K, float g2, float tiny, unsigned long long ent,
                                                uint32_t *__restrict__ codes, unsigned long long *__restrict__ out_list,
@@ -579,26 +682,45 @@ __device__ __forceinline__ void recheck2_entry(const float *xr, const float *__r
     const uint64_t gr = ent_row(ent);
     const uint32_t gc = ent_col(ent);
     const float *wr = Wm + uint64_t(gc) * d;
-    float s = 0.f, c = 0.f, sa = 0.f;
-    for (uint32_t t = lane; t < d; t += 32) {
-        const float xv = xr[t], wv = wr[t];
-        const float h = xv * wv;
-        const float l = fmaf(xv, wv, -h);          // exact product error
-        const float sn = s + h;                     // two-sum
-        const float z = sn - s;
-        c += (s - (sn - z)) + (h - z) + l;
-        s = sn;
-        sa = fmaf(fabsf(xv), fabsf(wv), sa);
+    // four compensated sums per lane (one per component of a 16-byte load): four
+    // independent chains of two-sums
+    float s[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f}, sa = 0.f;
+    auto add = [&](float &sum, float &comp, float h, float l) {
+        const float sn = sum + h;                   // two-sum
+        const float z = sn - sum;
+        comp += (sum - (sn - z)) + (h - z) + l;
+        sum = sn;
+    };
+#pragma unroll 2
+    for (uint32_t t = lane * 4; t < d; t += 128) {
+        float xv[4];                                  // xr may be shared memory: plain loads
+        if constexpr (VEC) {
+            const float4 x4 = *reinterpret_cast<const float4 *>(xr + t);
+            xv[0] = x4.x;
+            xv[1] = x4.y;
+            xv[2] = x4.z;
+            xv[3] = x4.w;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) xv[i] = xr[t + i];
+        }
+        const float4 w4 = load4<true>(wr, t, d, true);
+        const float wv[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float h = xv[i] * wv[i];
+            add(s[i], c[i], h, fmaf(xv[i], wv[i], -h));       // exact product error
+            sa = fmaf(fabsf(xv[i]), fabsf(wv[i]), sa);
+        }
     }
-    // combine the lanes: lane 0 adds the 32 (s, c) pairs with two-sums
-    float ts = 0.f, tc = 0.f;
-    for (int k = 0; k < 32; ++k) {
-        const float sk = __shfl_sync(0xffffffffu, s, k);
-        const float ck = __shfl_sync(0xffffffffu, c, k);
-        const float sn = ts + sk;
-        const float z = sn - ts;
-        tc += (ts - (sn - z)) + (sk - z) + ck;
-        ts = sn;
+#pragma unroll
+    for (int i = 1; i < 4; ++i) add(s[0], c[0], s[i], c[i]);
+    // combine the lanes, halving: each pair by a two-sum
+    float ts = s[0], tc = c[0];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float so = __shfl_down_sync(0xffffffffu, ts, o), co = __shfl_down_sync(0xffffffffu, tc, o);
+        add(ts, tc, so, co);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sa += __shfl_xor_sync(0xffffffffu, sa, o);
@@ -616,7 +738,8 @@ __device__ __forceinline__ void recheck2_entry(const float *xr, const float *__r
     }
 }
 
-__global__ void k_srp_recheck2(const float *__restrict__ X, uint64_t ldx, const float *__restrict__ Wm, uint32_t d,
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_srp_recheck2(const float *__restrict__ X, uint64_t ldx, const float *__restrict__ Wm, uint32_t d,
                                uint32_t L, uint32_t K, float g2, float tiny,
                                const unsigned long long *__restrict__ rlist,
                                const unsigned long long *__restrict__ rcount, uint32_t *__restrict__ codes,
@@ -628,7 +751,7 @@ __global__ void k_srp_recheck2(const float *__restrict__ X, uint64_t ldx, const 
     for (unsigned long long e = (unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
          e < nlist; e += nwarps) {
         const unsigned long long ent = rlist[e];
-        recheck2_entry(X + ent_row(ent) * ldx, Wm, d, L, K, g2, tiny, ent, codes, out_list, out_count, stats);
+        recheck2_entry<VEC>(X + ent_row(ent) * ldx, Wm, d, L, K, g2, tiny, ent, codes, out_list, out_count, stats);
     }
 }
 
@@ -665,7 +788,7 @@ __global__ void k_srp_recheck2_rows(const float *__restrict__ X, uint64_t ldx, c
                                     uint32_t *__restrict__ codes, unsigned long long *__restrict__ out_list,
                                     unsigned long long *__restrict__ out_count, unsigned long long *__restrict__ stats)
 {
-    extern __shared__ float xs[];
+    extern __shared__ __align__(16) float xs[];
     const uint32_t warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (uint32_t r = blockIdx.x; r < rows; r += gridDim.x) {
         const uint32_t e0 = rowoff[r], e1 = rowoff[r + 1];
@@ -674,7 +797,7 @@ __global__ void k_srp_recheck2_rows(const float *__restrict__ X, uint64_t ldx, c
         for (uint32_t t = threadIdx.x; t < d; t += blockDim.x) xs[t] = xg[t];
         __syncthreads();
         for (uint32_t e = e0 + warp; e < e1; e += nw)
-            recheck2_entry(xs, Wm, d, L, K, g2, tiny, sorted[e], codes, out_list, out_count, stats);
+            recheck2_entry<true>(xs, Wm, d, L, K, g2, tiny, sorted[e], codes, out_list, out_count, stats);
         __syncthreads();                              // before the next row overwrites xs
     }
 }
@@ -730,30 +853,48 @@ inline size_t qrow_bytes(uint32_t precision, uint32_t d)
     return precision == FLINNG_PREC_BF16X2 ? size_t(d) * 4 : precision == FLINNG_PREC_BF16 ? size_t(d) * 2 : size_t(d);
 }
 
-int quant_rows(uint32_t precision, const float *x, uint64_t ld, uint64_t n, uint32_t d, void *q, float *norm,
-               float *res, float *scale, cudaStream_t st)
+// A single-term form leaves a share of the projections undecided that grows
+// with its residual norms (about a sixth at d = 4096 in BF16, nearly all in
+// FP8). Re-checked one by one, each streams its row of W from L2 (2.3 ns per
+// projection at d = 4096 with every SM busy); a dense second pass on the
+// two-term split costs 0.05 ns per projection of the batch, decided or not, so
+// it wins from an undecided share of about 2 %: d >= 128 in BF16, any d in FP8,
+// once the batch fills the chip (2^20 projections: 64 tiles of 128 x 128). 8,192
+// embeddings in BF16: 4.04 ms re-checked one by one, 0.77 ms with the second pass.
+inline bool dense_second_pass(uint32_t precision, uint64_t rows, uint32_t P, uint32_t d)
 {
-    if (precision == FLINNG_PREC_BF16X2) {
+    if (precision != FLINNG_PREC_BF16 && precision != FLINNG_PREC_FP8) return false;
+    return rows * P >= (1ull << 20) && (precision == FLINNG_PREC_FP8 || d >= 128);
+}
+
+// two: also x2 behind x1 (the BF16 form's second pass)
+int quant_rows(uint32_t precision, const float *x, uint64_t ld, uint64_t n, uint32_t d, void *q, float *norm,
+               float *res, float *scale, bool two, cudaStream_t st)
+{
+    const bool vec = rows_vec4(x, ld, d);
+    const unsigned grid = warp_grid(n);
+    if (precision != FLINNG_PREC_FP8) {
         __nv_bfloat16 *q1 = static_cast<__nv_bfloat16 *>(q);
-        k_split_rows<<<warp_grid(n), 256, 0, st>>>(x, ld, n, d, q1, q1 + n * d, norm);
-    } else if (precision == FLINNG_PREC_BF16) {
-        k_quant_rows<kFormBf16><<<warp_grid(n), 256, 0, st>>>(x, ld, n, d, q, norm, res, nullptr);
+        auto fn = two ? (vec ? k_split_rows<true, true> : k_split_rows<false, true>)
+                      : (vec ? k_split_rows<true, false> : k_split_rows<false, false>);
+        fn<<<grid, 256, 0, st>>>(x, ld, n, d, q1, q1 + n * d, norm, res);
     } else {
-        k_quant_rows<kFormFp8><<<warp_grid(n), 256, 0, st>>>(x, ld, n, d, q, norm, res, scale);
+        auto fn = vec ? k_quant_rows<true> : k_quant_rows<false>;
+        fn<<<grid, 256, 0, st>>>(x, ld, n, d, static_cast<__nv_fp8_e4m3 *>(q), norm, res, scale);
     }
     count_launch();
     FL_CUDA(cudaGetLastError());
     return FLINNG_OK;
 }
 
-template <int FORM>
+template <int FORM, int MASK>
 int launch_tc(const CUtensorMap &mx1, const CUtensorMap &mx2, const CUtensorMap &mw1, const CUtensorMap &mw2,
               const TcArgs &a, uint64_t rows, cudaStream_t st)
 {
     const size_t smem = tc_smem_bytes<FORM>();
-    FL_TRY(ensure_dyn_smem((const void *)k_srp_tc<FORM>, smem));
+    FL_TRY(ensure_dyn_smem((const void *)k_srp_tc<FORM, MASK>, smem));
     dim3 grid((a.P + kTN - 1) / kTN, (unsigned)((rows + kTM - 1) / kTM));
-    k_srp_tc<FORM><<<grid, kTcThreads, smem, st>>>(mx1, mx2, mw1, mw2, a);
+    k_srp_tc<FORM, MASK><<<grid, kTcThreads, smem, st>>>(mx1, mx2, mw1, mw2, a);
     count_launch();
     FL_CUDA(cudaGetLastError());
     return FLINNG_OK;
@@ -767,22 +908,32 @@ int srp_tc_prepare_weights(flinng_index *ix)
     if (d % (prec == FLINNG_PREC_FP8 ? 16 : 8) != 0)
         return set_error(FLINNG_ERR_INVALID_ARG, "tensor-core SRP: dim %u is not a multiple of %d", d,
                          prec == FLINNG_PREC_FP8 ? 16 : 8);
-    const size_t qb = qrow_bytes(prec, d) * P;
+    // the single-term forms also keep the two-term split, for the dense second pass
+    const size_t split = size_t(P) * d * 4, qb = prec == FLINNG_PREC_FP8 ? split + size_t(P) * d : split;
     FL_CUDA(cudaMalloc(&ix->w_split, qb));
-    FL_CUDA(cudaMalloc(&ix->w_norm, size_t(P) * sizeof(float)));
-    ix->device_bytes += qb + size_t(P) * 4;
+    ix->device_bytes += qb;
     if (prec != FLINNG_PREC_BF16X2) {
         FL_CUDA(cudaMalloc(&ix->w_aux, size_t(P) * 2 * sizeof(float)));
         ix->device_bytes += size_t(P) * 8;
     }
-    return quant_rows(prec, ix->srp_w, d, P, d, ix->w_split, ix->w_norm, ix->w_aux, ix->w_aux ? ix->w_aux + P : nullptr,
-                      ix->stream);
+    FL_TRY(quant_rows(FLINNG_PREC_BF16X2, ix->srp_w, d, P, d, ix->w_split, ix->w_norm, ix->w_aux, nullptr, true,
+                      ix->stream));
+    if (prec != FLINNG_PREC_FP8) return FLINNG_OK;
+    return quant_rows(prec, ix->srp_w, d, P, d, static_cast<char *>(ix->w_split) + split, ix->w_norm, ix->w_aux,
+                      ix->w_aux + P, false, ix->stream);
+}
+
+// bytes per row of the quantised x: the two-term split where a second pass needs it
+static size_t x_bytes(const flinng_index *ix, uint64_t rows)
+{
+    return dense_second_pass(ix->cfg.precision, rows, ix->P, ix->cfg.dim) ? size_t(ix->cfg.dim) * 4
+                                                                          : qrow_bytes(ix->cfg.precision, ix->cfg.dim);
 }
 
 size_t srp_tc_workspace_bytes(const flinng_index *ix, uint64_t n)
 {
     const uint64_t rows = n < kTcChunkRows ? n : kTcChunkRows;
-    return carve_bytes<char>(rows * qrow_bytes(ix->cfg.precision, ix->cfg.dim)) + 3 * carve_bytes<float>(rows) +
+    return carve_bytes<char>(rows * x_bytes(ix, rows)) + 3 * carve_bytes<float>(rows) +
            carve_bytes<unsigned long long>(8) + 2 * carve_bytes<unsigned long long>(rows * ix->P + 1) +
            3 * carve_bytes<uint32_t>(rows + 1) + carve_bytes<char>(scan_workspace_bytes(rows + 1)) + 4096;
 }
@@ -799,7 +950,7 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
     const uint64_t chunk = kTcChunkRows;
     const uint64_t cap = n < chunk ? n : chunk;     // rows the workspace was sized for
     Carver c(ws, ~size_t(0));
-    char *xq = c.take<char>(cap * qrow_bytes(prec, d));
+    char *xq = c.take<char>(cap * x_bytes(ix, cap));
     float *xn = c.take<float>(cap);
     float *xr = c.take<float>(cap);
     float *xsc = c.take<float>(cap);
@@ -816,34 +967,39 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
     FL_CUDA(cudaMemsetAsync(ix->stats, 0, kStats * sizeof(unsigned long long), st));
     if (n == 0) return FLINNG_OK;
     FL_CUDA(cudaMemsetAsync(buckets, 0, n * L * sizeof(uint32_t), st));
-    const char *wq = static_cast<const char *>(ix->w_split);
-    CUtensorMap mw1, mw2;
-    FL_TRY(make_map(&mw1, wq, P, d, bytes));
-    if (prec == FLINNG_PREC_BF16X2) FL_TRY(make_map(&mw2, wq + size_t(P) * d * 2, P, d, false));
-    else mw2 = mw1;
+    const char *w1p = static_cast<const char *>(ix->w_split), *wqp = bytes ? w1p + size_t(P) * d * 4 : w1p;
+    CUtensorMap mw1, mw2, mwq;
+    FL_TRY(make_map(&mw1, w1p, P, d, false));
+    FL_TRY(make_map(&mw2, w1p + size_t(P) * d * 2, P, d, false));
+    if (bytes) FL_TRY(make_map(&mwq, wqp, P, d, true));
+    else mwq = mw1;
     // margin factors (see the header comment), in double then rounded up
     const double u = std::ldexp(1.0, -24), up = std::ldexp(1.0, -22);
     auto g = [](double m, double uu) { return m * uu / (1.0 - m * uu); };
     const double q = (1 + std::ldexp(1.0, -8)) * (1 + std::ldexp(1.0, -8));
     const double kb = prec == FLINNG_PREC_FP8 ? 128.0 : double(kTK);     // products per k-block
     const double m_blocks = std::ceil(double(d) / kb);
-    double f;
-    if (prec == FLINNG_PREC_BF16X2)
-        f = (g(kTK, up) + std::ldexp(1.0, -7) * g(2 * kTK, up)) * q +
-            g(2 * m_blocks, u) * (1 + g(kTK, up)) * (1 + std::ldexp(1.0, -7)) * q + 3.1 * std::ldexp(1.0, -16);
-    else
-        f = g(kb, up) + g(m_blocks, u) * (1 + g(kb, up));    // times (||x|| + ||e_x||)(||w|| + ||e_w||)
-    const float c_norm = std::nextafter(float(f * 1.0001), INFINITY);
+    const double m64 = std::ceil(double(d) / kTK);
+    const double f2 = (g(kTK, up) + std::ldexp(1.0, -7) * g(2 * kTK, up)) * q +
+                      g(2 * m64, u) * (1 + g(kTK, up)) * (1 + std::ldexp(1.0, -7)) * q + 3.1 * std::ldexp(1.0, -16);
+    const double f1 = g(kb, up) + g(m_blocks, u) * (1 + g(kb, up));    // times (||x|| + ||e_x||)(||w|| + ||e_w||)
+    const float c_two = std::nextafter(float(f2 * 1.0001), INFINITY);
+    const float c_norm = prec == FLINNG_PREC_BF16X2 ? c_two : std::nextafter(float(f1 * 1.0001), INFINITY);
     const float c_sub = std::nextafter(float(std::sqrt(double(d)) * std::ldexp(1.0, -125)), INFINITY);
     const float tiny = std::nextafter(float(8.0 * d * std::ldexp(1.0, -126)), INFINITY);
     const double g2d = 2.0 * d * std::ldexp(1.0, -24) / (1.0 - 2.0 * d * std::ldexp(1.0, -24));
     const float g2 = std::nextafter(float(2.0 * g2d * g2d + std::ldexp(1.0, -40)), INFINITY);
     for (uint64_t r0 = 0; r0 < n; r0 += chunk) {
         const uint64_t rows = (n - r0) < chunk ? (n - r0) : chunk;
-        FL_TRY(quant_rows(prec, x + r0 * ld, ld, rows, d, xq, xn, xr, xsc, st));
+        const float *xc = x + r0 * ld;
+        // capped by the rows the workspace was sized for, so that the last, shorter
+        // chunk goes the way its space allows
+        const bool dense = dense_second_pass(prec, cap, P, d) && dense_second_pass(prec, rows, P, d);
+        const bool two = prec == FLINNG_PREC_BF16X2 || (dense && prec == FLINNG_PREC_BF16);
+        FL_TRY(quant_rows(prec, xc, ld, rows, d, xq, xn, prec == FLINNG_PREC_BF16X2 ? nullptr : xr, xsc, two, st));
         CUtensorMap mx1, mx2;
         FL_TRY(make_map(&mx1, xq, rows, d, bytes));
-        if (prec == FLINNG_PREC_BF16X2) FL_TRY(make_map(&mx2, xq + rows * d * 2, rows, d, false));
+        if (two) FL_TRY(make_map(&mx2, xq + rows * d * 2, rows, d, false));
         else mx2 = mx1;
         FL_CUDA(cudaMemsetAsync(cnt, 0, 8 * sizeof(unsigned long long), st));
         TcArgs a{};
@@ -865,13 +1021,32 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
         a.proj = proj ? proj + r0 * P : nullptr;
         a.rlist = list1;
         a.rcount = cnt;
+        a.mask = reinterpret_cast<uint32_t *>(list2);     // free until the list is grouped by row
+        a.nund = cnt + 2;
+        a.stats = ix->stats;
         a.err = ix->tc_err;
         a.wait_ns = ix->tc_wait_ns ? ix->tc_wait_ns - 1 : kWaitNs;
-        if (prec == FLINNG_PREC_BF16X2) FL_TRY(launch_tc<kFormBf16x2>(mx1, mx2, mw1, mw2, a, rows, st));
-        else if (prec == FLINNG_PREC_BF16) FL_TRY(launch_tc<kFormBf16>(mx1, mx2, mw1, mw2, a, rows, st));
-        else FL_TRY(launch_tc<kFormFp8>(mx1, mx2, mw1, mw2, a, rows, st));
-        // stage 2: compensated fp32; stage 3: fp64 / exact
-        if (rows_staged) {
+        if (prec == FLINNG_PREC_BF16X2) FL_TRY((launch_tc<kFormBf16x2, 0>(mx1, mx2, mw1, mw2, a, rows, st)));
+        else if (!dense && prec == FLINNG_PREC_BF16) FL_TRY((launch_tc<kFormBf16, 0>(mx1, mx1, mwq, mwq, a, rows, st)));
+        else if (!dense) FL_TRY((launch_tc<kFormFp8, 0>(mx1, mx1, mwq, mwq, a, rows, st)));
+        else if (prec == FLINNG_PREC_BF16) FL_TRY((launch_tc<kFormBf16, 1>(mx1, mx1, mwq, mwq, a, rows, st)));
+        else FL_TRY((launch_tc<kFormFp8, 1>(mx1, mx1, mwq, mwq, a, rows, st)));
+        if (dense) {
+            // the marked projections again on the two-term split, whose margin
+            // leaves a few in a thousand
+            if (bytes) {
+                FL_TRY(quant_rows(FLINNG_PREC_BF16X2, xc, ld, rows, d, xq, xn, nullptr, nullptr, true, st));
+                FL_TRY(make_map(&mx1, xq, rows, d, false));
+                FL_TRY(make_map(&mx2, xq + rows * d * 2, rows, d, false));
+            }
+            a.c_norm = c_two;
+            a.proj = nullptr;
+            FL_TRY((launch_tc<kFormBf16x2, 2>(mx1, mx2, mw1, mw2, a, rows, st)));
+        }
+        // stage 2: compensated fp32; stage 3: fp64 / exact. A list of a sixth of
+        // the projections or more is grouped by row, so that each row of x is
+        // staged once; a short one is not worth the passes.
+        if (rows_staged && !dense && prec != FLINNG_PREC_BF16X2) {
             // the list grouped by row into list2; stage 2 lists what stays undecided in list1
             FL_CUDA(cudaMemsetAsync(rowcnt, 0, (rows + 1) * sizeof(uint32_t), st));
             FL_CUDA(cudaMemsetAsync(fill, 0, (rows + 1) * sizeof(uint32_t), st));
@@ -890,13 +1065,14 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
             FL_CUDA(cudaGetLastError());
             FL_TRY(srp_recheck_list(ix, x + r0 * ld, ld, list1, cnt + 1, buckets + r0 * L));
         } else {
-            k_srp_recheck2<<<152 * 4, 256, 0, st>>>(x + r0 * ld, ld, ix->srp_w, d, L, K, g2, tiny, list1, cnt,
+            auto fn = rows_vec4(xc, ld, d) ? k_srp_recheck2<true> : k_srp_recheck2<false>;
+            fn<<<152 * 8, 256, 0, st>>>(x + r0 * ld, ld, ix->srp_w, d, L, K, g2, tiny, list1, cnt,
                                                    buckets + r0 * L, list2, cnt + 1, ix->stats);
             count_launch();
             FL_CUDA(cudaGetLastError());
             FL_TRY(srp_recheck_list(ix, x + r0 * ld, ld, list2, cnt + 1, buckets + r0 * L));
         }
-        FL_TRY(add_counter(ix->stats, cnt, st));            // undecided after the tensor-core pass
+        FL_TRY(add_counter(ix->stats, dense ? cnt + 2 : cnt, st));     // undecided after the first pass
     }
     // no synchronisation here (servers hash on their own streams): the flag
     // lands in pinned memory and the next call on this index reports it
