@@ -258,6 +258,59 @@ bool pinned_points(const flinng_index *ix, const flinng_points *pts, uint64_t n,
     return true;
 }
 
+// A small fused query from host memory: inputs memcpy'd into the index's pinned
+// staging, read and written there in place by the kernel over the host link, and
+// the results memcpy'd out after one wait. For a few KB this replaces up to five
+// asynchronous copies of pageable memory and the buffers' pointer queries, which
+// cost more than the query (1 genomic read: 59 -> 31 us a call). Larger batches
+// move at copy-engine rates instead. The staging is in use only within a call,
+// which waits for the kernel; calls on one index do not overlap.
+int query_small_host(flinng_index *ix, const flinng_points *q, uint32_t nq, const uint32_t *k, uint32_t k_max,
+                     uint32_t *out_ids, uint16_t *out_scores, bool *done)
+{
+    *done = false;
+    const bool srp = ix->cfg.metric == FLINNG_COSINE_SRP;
+    const uint64_t ne = srp ? uint64_t(nq) * ix->cfg.dim : q->off[nq];
+    // bounded before it is added up: nq and ne may be anything here
+    if (nq > kSmallStage / 8 || ne > kSmallStage / 4) return FLINNG_OK;
+    size_t need = carve_bytes<float>(ne) + carve_bytes<uint64_t>(nq + 1) + carve_bytes<uint32_t>(nq) +
+                  carve_bytes<uint32_t>(uint64_t(nq) * k_max) + carve_bytes<uint16_t>(uint64_t(nq) * k_max);
+    if (need > kSmallStage) return FLINNG_OK;
+    Carver c(reinterpret_cast<char *>(ix->h_flag) + 256, kSmallStage);
+    FusedQuery fq{nq, nullptr, ix->cfg.dim, nullptr, nullptr};
+    if (srp) {
+        float *x = c.take<float>(ne);
+        for (uint32_t i = 0; i < nq; ++i)
+            std::memcpy(x + size_t(i) * ix->cfg.dim, q->x + size_t(i) * q->ld, ix->cfg.dim * sizeof(float));
+        fq.x = x;
+    } else {
+        uint64_t *off = c.take<uint64_t>(nq + 1);
+        uint32_t *el = c.take<uint32_t>(ne);
+        std::memcpy(off, q->off, (nq + 1) * sizeof(uint64_t));
+        if (ne) std::memcpy(el, q->elems, ne * sizeof(uint32_t));
+        fq.off = off;
+        fq.elems = el;
+    }
+    uint32_t *kk = nullptr;
+    if (k) {
+        kk = c.take<uint32_t>(nq);
+        std::memcpy(kk, k, nq * sizeof(uint32_t));
+    }
+    uint32_t *ids = c.take<uint32_t>(uint64_t(nq) * k_max);
+    uint16_t *sc = out_scores ? c.take<uint16_t>(uint64_t(nq) * k_max) : nullptr;
+    uint32_t bucket = 0;
+    while ((1u << bucket) < nq) ++bucket;
+    const QueryTuning *tune = ix->tuning[bucket].valid ? &ix->tuning[bucket] : nullptr;
+    if (ix->query_mode == FLINNG_QUERY_GRAPH) FL_TRY(query_graph_launch(ix, fq, kk, k_max, ids, sc, tune));
+    else FL_TRY(query_fused_launch(ix, fq, kk, k_max, ids, sc, tune));
+    FL_CUDA(cudaStreamSynchronize(ix->stream));
+    std::memcpy(out_ids, ids, size_t(nq) * k_max * sizeof(uint32_t));
+    if (out_scores) std::memcpy(out_scores, sc, size_t(nq) * k_max * sizeof(uint16_t));
+    *done = true;
+    if (ix->h_flag[3]) return set_error(FLINNG_ERR_TIMEOUT, "tensor-core SRP: a pipeline wait timed out");
+    return FLINNG_OK;
+}
+
 int hash_staged(flinng_index *ix, const Staged &s, uint64_t n, uint32_t *buckets, uint32_t *values,
                 float *proj, void *hws, size_t hws_bytes)
 {
@@ -410,7 +463,8 @@ int flinng_create(const flinng_config *cfg, const flinng_params *params, void *s
     ALLOC(tc_err, 4);
 #undef ALLOC
     if (rc == FLINNG_OK) {
-        cudaError_t e = cudaMallocHost((void **)&ix->h_flag, 16);
+        // status words, then the staging of small host queries
+        cudaError_t e = cudaMallocHost((void **)&ix->h_flag, kSmallStage + 256);
         if (e != cudaSuccess) rc = cuda_error(e, "cudaMallocHost");
         else std::memset(ix->h_flag, 0, 16);
     }
@@ -683,6 +737,16 @@ static int query_common(flinng_index *idx, const flinng_points *q, const uint32_
     const cudaStream_t st = idx->stream;
     const uint32_t L = idx->cfg.L;
     const bool probe = idx->probes > 1;
+    // Per-CTA hashing reads all L*K projection rows for every query: for a
+    // large projection matrix the batched GEMM (plain form) hashes far better.
+    const bool big_srp = idx->cfg.metric == FLINNG_COSINE_SRP && uint64_t(idx->P) * idx->cfg.dim > (1ull << 18);
+    const bool fused = q && !big_srp && !probe &&
+                       (idx->query_mode == FLINNG_QUERY_FUSED || idx->query_mode == FLINNG_QUERY_GRAPH);
+    if (fused && !on_device) {
+        bool done = false;
+        FL_TRY(query_small_host(idx, q, nq, k, k_max, out_ids, out_scores, &done));
+        if (done) return FLINNG_OK;
+    }
     size_t need = 4096 + carve_bytes<uint32_t>(uint64_t(nq) * L);
     if (probe) need += carve_bytes<uint16_t>(uint64_t(nq) * idx->BR);
     if (q) need += stage_bytes(idx, q, nq, on_device) + hash_ws_bytes(idx, nq);
@@ -692,11 +756,6 @@ static int query_common(flinng_index *idx, const flinng_points *q, const uint32_
     FL_TRY(ws_reserve(idx, need));
     Carver c(idx->ws.ptr, idx->ws.bytes);
     uint32_t *qb = nullptr;
-    // Per-CTA hashing reads all L*K projection rows for every query: for a
-    // large projection matrix the batched GEMM (plain form) hashes far better.
-    const bool big_srp = idx->cfg.metric == FLINNG_COSINE_SRP && uint64_t(idx->P) * idx->cfg.dim > (1ull << 18);
-    const bool fused = q && !big_srp && !probe &&
-                       (idx->query_mode == FLINNG_QUERY_FUSED || idx->query_mode == FLINNG_QUERY_GRAPH);
     Staged fs;
     if (fused) {
         if (on_device || !pinned_points(idx, q, nq, fs)) FL_TRY(stage_points(idx, q, nq, on_device, c, fs));

@@ -30,6 +30,9 @@ constexpr uint64_t kMg1Pad = 16;
 // the same for the cell lists (read eight aligned cells at a time)
 constexpr uint64_t kCellPad = 8;
 
+// pinned bytes per index for the inputs and outputs of small host queries
+constexpr size_t kSmallStage = 64 * 1024;
+
 // Error plumbing: every internal step returns an int status and leaves a
 // message in the thread-local buffer.
 int set_error(int code, const char *fmt, ...);
@@ -147,7 +150,7 @@ struct flinng_index {
     uint32_t *cell_cnt;    // BR + 1 (build scratch)
     uint32_t *flag;        // device status word
     uint32_t *qnext;       // query counter of the fused kernel
-    uint32_t *h_flag;      // pinned host copy
+    uint32_t *h_flag;      // pinned: status words, from byte 256 the staging of small host queries
     unsigned long long *stats;   // [recheck, exact]
     uint64_t last_recheck, last_exact;
 

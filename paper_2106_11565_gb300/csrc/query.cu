@@ -232,6 +232,8 @@ static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t 
     uint64_t grid = uint64_t(sms) * want;
     if (grid > grid_for) grid = grid_for;
     P->grid = uint32_t(grid ? grid : 1);
+    // every query has a CTA of its own: no counter to clear and draw from
+    if (P->grid == nq && grid_for == nq) h.qnext = nullptr;
     P->args[0] = &P->a;
     P->args[1] = &P->h;
     return FLINNG_OK;
@@ -245,7 +247,7 @@ int query_fused_launch(flinng_index *ix, const FusedQuery &fq, const uint32_t *k
     FL_TRY(fused_prepare(ix, fq, k, k_max, out_ids, out_scores, tune, fq.nq, &P));
     if (ix->cfg.metric == FLINNG_COSINE_SRP)
         FL_CUDA(cudaMemsetAsync(ix->stats, 0, kStats * sizeof(unsigned long long), ix->stream));
-    FL_CUDA(cudaMemsetAsync(ix->qnext, 0, sizeof(uint32_t), ix->stream));
+    if (P.h.qnext) FL_CUDA(cudaMemsetAsync(ix->qnext, 0, sizeof(uint32_t), ix->stream));
     FL_CUDA(cudaLaunchKernel(P.fn, dim3(P.grid), dim3(P.threads), P.args, P.smem, ix->stream));
     count_launch();
     return FLINNG_OK;

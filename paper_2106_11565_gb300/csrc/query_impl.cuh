@@ -1058,7 +1058,7 @@ struct HArgs {
     float gamma2, tiny;
     double gamma64;
     unsigned long long *stats;
-    uint32_t *qnext;    // next query to hand out (zeroed before each launch)
+    uint32_t *qnext;    // next query to hand out (zeroed before each launch), or null: one per CTA
     uint32_t K;
     size_t hash_off;    // byte offset of the hash region in shared memory (0: inside the
                         // candidate buffer, which is free until the decode)
@@ -1252,10 +1252,12 @@ k_query_fused(QArgs a, HArgs h)
     uint32_t *hs = qslot + 4;
     // queries are handed out one at a time from a counter (zeroed before the
     // launch), so CTAs that drew cheap queries take more of them
-    for (;;) {
-        if (threadIdx.x == 0) qslot[0] = atomicAdd(h.qnext, 1u);
-        __syncthreads();
-        const uint32_t q = qslot[0];
+    for (uint32_t q = blockIdx.x;;) {
+        if (h.qnext) {
+            if (threadIdx.x == 0) qslot[0] = atomicAdd(h.qnext, 1u);
+            __syncthreads();
+            q = qslot[0];
+        }
         if (q >= a.nq) break;
         uint32_t kq = a.k ? a.k[q] : a.k_max;
         if (kq > a.k_max) kq = a.k_max;
@@ -1268,6 +1270,7 @@ k_query_fused(QArgs a, HArgs h)
             __syncthreads();
         }
         decode_topk<NT, RW, CW>(a, s, q, kq);
+        if (!h.qnext) break;
     }
 }
 
