@@ -179,12 +179,12 @@ static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t 
     hash_bytes = (hash_bytes + 15) & ~size_t(15);
     // The hash region (query buckets, hash scratch, the query slot) is live
     // only before the decode keeps candidates, so it shares the candidate
-    // buffer with the gather's heavy-table list (the buffer's last NT words)
+    // buffer with the gather's heavy-table list (the buffer's last 2 NT words)
     // when both fit; otherwise it follows the query state.
     auto shape = [&](int nt) {
         size_t qbytes;
         pick_buffer(a, nt, tune, 0, &qbytes, int(ix->cw));
-        if (hash_bytes + size_t(nt) * 4 <= size_t(a.cap) * 8) {
+        if (hash_bytes + size_t(nt) * 8 <= size_t(a.cap) * 8) {
             h.hash_off = 0;
             P->smem = qbytes;
         } else {
@@ -202,18 +202,26 @@ static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t 
     // against 45), else 512.
     int NT = tune && tune->threads ? int(tune->threads) : 512;
     shape(NT);
+    auto fit = [&]() { return uint32_t(228 * 1024 / (P->smem + 1024)); };
+    // Threads per SM by registers: with 16-bit counts 1,024 where shared memory
+    // (or the batch) fills no more of the SM, since 64 registers then cost nothing
+    // (4,000 recall-target queries: 382 -> 363 us; at 2,048 possible threads, 349
+    // tables in 2,000 cells, they cost 187 -> 231 us).
+    uint32_t sm_threads = srp ? 1024 : 2048;
+    const bool both = !srp && ix->cw == 2;
     if (!tune || !tune->threads) {
-        const uint32_t sm_threads = srp ? 1024 : 2048;     // the kernels' register bounds
-        const uint32_t fit = std::min(uint32_t(228 * 1024 / (P->smem + 1024)), sm_threads / 512);
-        if (fq.nq > uint32_t(sms) * fit) {
+        if (both && nq <= uint32_t(sms) * std::min(fit(), 2u)) {
+            sm_threads = 1024;
+        } else if (nq > uint32_t(sms) * std::min(fit(), sm_threads / 512)) {
             shape(256);
-            if (228 * 1024 / (P->smem + 1024) >= 4) NT = 256;
+            if (fit() >= 4) NT = 256;
             else shape(512);
         }
     }
+    if (both && fit() * uint32_t(NT) <= 1024) sm_threads = 1024;
     if (P->smem > 227 * 1024)
         return set_error(FLINNG_ERR_INVALID_ARG, "fused query: %zu bytes of shared memory needed (> 227 KB)", P->smem);
-    P->fn = ix->cw == 1 ? fused_kernel_c1(NT, ix->rw, srp) : fused_kernel_c2(NT, ix->rw, srp);
+    P->fn = ix->cw == 1 ? fused_kernel_c1(NT, ix->rw, srp, sm_threads) : fused_kernel_c2(NT, ix->rw, srp, sm_threads);
     P->threads = NT;
     FL_TRY(ensure_dyn_smem(P->fn, P->smem));
     int per_sm = 0;
@@ -319,7 +327,7 @@ int counts_launch(flinng_index *ix, const uint32_t *qbuckets, uint32_t nq,
 {
     if (nq == 0) return FLINNG_OK;
     QArgs a = make_args(ix, qbuckets, nq);
-    a.cap = kQTmax / 2;      // the heavy-table list takes the buffer's last kQTmax words
+    a.cap = kQTmax;          // the heavy-table list takes the buffer's last 2 kQTmax words
     a.kp = 2;
     a.out_counts = out_counts;
     const size_t smem = qsmem_bytes(a.cap, a.kp, a.BR, a.lcap, kQTmax, a.L, int(ix->cw));
@@ -332,7 +340,10 @@ int counts_launch(flinng_index *ix, const uint32_t *qbuckets, uint32_t nq,
 }
 
 const void *plain_kernel_c1(int NT, uint32_t rw) { return plain_kernel_t<1>(NT, rw); }
-const void *fused_kernel_c1(int NT, uint32_t rw, bool srp) { return fused_kernel_t<1>(NT, rw, srp); }
+const void *fused_kernel_c1(int NT, uint32_t rw, bool srp, uint32_t sm_threads)
+{
+    return fused_kernel_t<1>(NT, rw, srp, sm_threads);
+}
 const void *counts_kernel_c1() { return (const void *)k_counts<1>; }
 
 }  // namespace flinng

@@ -6,7 +6,10 @@
 namespace flinng {
 
 const void *plain_kernel_c2(int NT, uint32_t rw) { return plain_kernel_t<2>(NT, rw); }
-const void *fused_kernel_c2(int NT, uint32_t rw, bool srp) { return fused_kernel_t<2>(NT, rw, srp); }
+const void *fused_kernel_c2(int NT, uint32_t rw, bool srp, uint32_t sm_threads)
+{
+    return fused_kernel_t<2>(NT, rw, srp, sm_threads);
+}
 const void *counts_kernel_c2() { return (const void *)k_counts<2>; }
 
 }  // namespace flinng

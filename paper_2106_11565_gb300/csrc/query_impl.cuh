@@ -53,10 +53,9 @@ template <> struct CountWidth<2> {
     static constexpr uint64_t kKeyBits = (1ull << 60) - 1;
 };
 
-// cells per chunk of the walk; the gather keeps two words for each of its NT
-// tables in the same space
+// cells per chunk of the walk, tables per chunk of the gather
 template <int NT> constexpr uint32_t kChunkCells = 2 * NT;
-constexpr uint32_t kWarpQueue = 64;      // filtered members a warp holds back
+constexpr uint32_t kWarpQueue = 64;      // filtered members a warp holds back (2 NT words in all)
 
 struct QArgs {
     const uint32_t *qb;
@@ -92,16 +91,18 @@ struct QSmem {
     uint32_t *u;         // 8 scalars: nbuf, nkeep, digit / k-th score, rank / found, whole / count,
                          // heavy tables, bound (u[6..7])
     uint32_t *lvl_n;     // nlev: repetition-0 cells per count, then cells at levels >= v
-    uint32_t *lvl_cur;   // nlev: placement cursors of the level list
     uint32_t *shist;     // nlev: candidates in buf per score
     uint32_t *rhist;     // 256: radix histogram
     uint32_t *c_pre;     // kChunkCells + 4: exclusive prefix of unit counts, closed by ~0
-    uint32_t *c_ms;      // kChunkCells: first member of each cell of a chunk
-    uint2 *g_rec;        // NT (in c_ms): per table of the gather its list's cells {first, end}
-    uint32_t *g_hl;      // NT: bitmap indices of the heavy tables of a chunk of tables (the last
-                         // NT words of buf: the gather runs before any candidate is kept)
+    uint32_t *c_ms;      // kChunkCells: first member of each cell of a chunk; in the gather, first
+                         // cell of each of 2 NT tables' lists
+    uint32_t *lvl_cur;   // nlev: placement cursors of the level list (in c_pre and c_ms, which hold
+                         // nothing while cells are placed)
+    uint32_t *g_hl;      // 2 NT: bitmap indices of the heavy tables of a chunk of tables (the last
+                         // words of buf: the gather runs before any candidate is kept)
     uint32_t *wsum;      // NT / 32: block-scan scratch
-    uint32_t *q_m;       // kWarpQueue per warp: members that passed the filter
+    uint32_t *q_m;       // kWarpQueue per warp: members that passed the filter; in the gather, the
+                         // lengths of the 2 NT tables' lists
     uint16_t *q_c;       // their cells
     uint32_t *cntw;      // count words: 4 byte counts (CW = 1) or 2 16-bit counts (CW = 2) each
     uint16_t *lvl_cells; // lcap
@@ -115,9 +116,9 @@ __host__ __device__ inline uint32_t q_count_words(uint32_t BR, int cw) { return 
 __host__ __device__ inline size_t qsmem_bytes(uint32_t cap, uint32_t kp, uint32_t BR, uint32_t lcap, int NT,
                                               uint32_t L, int cw)
 {
-    const uint32_t ch = 2 * NT;       // kChunkCells
-    size_t b = size_t(cap) * 8 + size_t(kp) * 8 + 8 * 4 + 3 * size_t(q_nlev(L)) * 4 + 256 * 4 +
-               (ch + 4) * 4 + ch * 4 + (NT / 32) * 4 + size_t(NT / 32) * kWarpQueue * 6;
+    const uint32_t ch = 2 * NT, chunk = 2 * ch + 4;      // kChunkCells; c_pre and c_ms
+    size_t b = size_t(cap) * 8 + size_t(kp) * 8 + 8 * 4 + 2 * size_t(q_nlev(L)) * 4 + 256 * 4 +
+               size_t(chunk > q_nlev(L) ? chunk : q_nlev(L)) * 4 + (NT / 32) * 4 + size_t(NT / 32) * kWarpQueue * 6;
     b = (b + 15) & ~size_t(15);
     b += size_t(q_count_words(BR, cw)) * 4 + size_t(lcap) * 2;
     return (b + 15) & ~size_t(15);
@@ -132,14 +133,13 @@ __device__ inline QSmem carve_q(unsigned char *sm, uint32_t cap, uint32_t kp, ui
     s.keep = s.buf + cap;
     s.u = (uint32_t *)(s.keep + kp);
     s.lvl_n = s.u + 8;
-    s.lvl_cur = s.lvl_n + nlev;
-    s.shist = s.lvl_cur + nlev;
+    s.shist = s.lvl_n + nlev;
     s.rhist = s.shist + nlev;
     s.c_pre = s.rhist + 256;
     s.c_ms = s.c_pre + kChunkCells<NT> + 4;
-    s.g_rec = reinterpret_cast<uint2 *>(s.c_ms);               // 8-byte aligned: offsets are even
-    s.g_hl = reinterpret_cast<uint32_t *>(s.buf + cap) - NT;   // needs 2 cap >= NT
-    s.wsum = s.c_ms + kChunkCells<NT>;
+    s.lvl_cur = s.c_pre;
+    s.g_hl = reinterpret_cast<uint32_t *>(s.buf + cap) - 2 * NT;   // needs cap >= NT
+    s.wsum = s.c_pre + (2 * kChunkCells<NT> + 4 > nlev ? 2 * kChunkCells<NT> + 4 : nlev);
     s.q_m = s.wsum + NT / 32;
     s.q_c = reinterpret_cast<uint16_t *>(s.q_m + NT / 32 * kWarpQueue);
     size_t o = (size_t)((unsigned char *)(s.q_c + NT / 32 * kWarpQueue) - sm);
@@ -427,7 +427,8 @@ __device__ __forceinline__ void planes_to_bytes(uint32_t (&pl)[8], uint32_t (&ou
     }
 }
 
-// Per-cell collision counts of one query (Sec. 5), NT tables at a time.
+// Per-cell collision counts of one query (Sec. 5), 2 NT tables at a time (a
+// thread's two offset pairs are in flight together).
 // Tables whose bucket is heavy contribute their cell bitmap: each thread owns
 // one bitmap word position (32 cells) and sums it over the heavy tables in
 // bit-sliced form, then adds the sums to its counter words without atomics. The
@@ -441,28 +442,39 @@ template <int NT, int CW>
 __device__ void gather_counts(const QArgs &a, const QSmem &s, const uint32_t *qb)
 {
     const int tid = threadIdx.x;
-    for (uint32_t l0 = 0; l0 < a.L; l0 += NT) {
-        const uint32_t l = l0 + tid;
-        uint32_t beg = 0, end = 0;
-        if (l < a.L) {
-            const uint64_t slot = (uint64_t(l) << a.W) | qb[l];
+    constexpr uint32_t kTab = 2 * NT;
+    for (uint32_t l0 = 0; l0 < a.L; l0 += kTab) {
+        uint32_t o0[2] = {0u, 0u}, o1[2] = {0u, 0u}, units[2];
+        uint64_t slot[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const uint32_t l = l0 + tid * 2 + i;
+            if (l < a.L) {
+                slot[i] = (uint64_t(l) << a.W) | qb[l];
+                o0[i] = a.off[slot[i]];
+                o1[i] = a.off[slot[i] + 1];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
             // the list's length decides whether the slot is heavy, so the
             // bitmap index (another random DRAM access) is read for heavy
             // slots only
-            const uint32_t o0 = a.off[slot], o1 = a.off[slot + 1];
-            if (o1 - o0 >= a.heavy_min) {
-                s.g_hl[atomicAdd(&s.u[5], 1u)] = a.hidx[slot];
-            } else {
-                beg = o0;
-                end = o1;
+            if (o1[i] - o0[i] >= a.heavy_min) {
+                s.g_hl[atomicAdd(&s.u[5], 1u)] = a.hidx[slot[i]];
+                o1[i] = o0[i];
             }
+            units[i] = o1[i] > o0[i] ? ((o1[i] - 1) >> 3) - (o0[i] >> 3) + 1 : 0u;
         }
-        if (tid == 0) s.c_pre[NT] = ~0u;   // ends every forward search of c_pre
-        const uint32_t units = end > beg ? ((end - 1) >> 3) - (beg >> 3) + 1 : 0u;
+        if (tid == 0) s.c_pre[kTab] = ~0u;   // ends every forward search of c_pre
         uint32_t total;
-        const uint32_t pre = block_excl_scan<NT>(units, s.wsum, &total);
-        s.g_rec[tid] = make_uint2(beg, end);
-        s.c_pre[tid] = pre;
+        const uint32_t pre = block_excl_scan<NT>(units[0] + units[1], s.wsum, &total);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            s.c_pre[tid * 2 + i] = pre + (i ? units[0] : 0u);
+            s.c_ms[tid * 2 + i] = o0[i];
+            s.q_m[tid * 2 + i] = o1[i] - o0[i];
+        }
         __syncthreads();
         const uint32_t nh = s.u[5];
         if (nh > 0) {
@@ -528,10 +540,10 @@ __device__ void gather_counts(const QArgs &a, const QSmem &s, const uint32_t *qb
             }
             __syncthreads();
         }
-        const uint32_t nl = min(uint32_t(NT), a.L - l0);
+        const uint32_t nl = min(kTab, a.L - l0);
         // each warp counts a contiguous slice of the flattened units, so a lane's
         // table index moves forward by a few tables per step (c_pre is total
-        // past the last table and ~0 at NT, which ends the search)
+        // past the last table and ~0 at the end, which ends the search)
         const uint32_t per = ((total + NT / 32 - 1) / (NT / 32) + 31) & ~31u;
         const uint32_t eb = min(uint32_t(tid >> 5) * per, total);
         const uint32_t ee = min(eb + per, total);
@@ -545,9 +557,8 @@ __device__ void gather_counts(const QArgs &a, const QSmem &s, const uint32_t *qb
                 }
                 ++t;
             }
-            const uint2 r = s.g_rec[t];
-            const uint32_t u = (r.x >> 3) + (e - s.c_pre[t]), m0 = u << 3;
-            const uint32_t lo = r.x > m0 ? r.x - m0 : 0u, hi = min(r.y - m0, 8u);
+            const uint32_t beg = s.c_ms[t], u = (beg >> 3) + (e - s.c_pre[t]), m0 = u << 3;
+            const uint32_t lo = beg > m0 ? beg - m0 : 0u, hi = min(beg + s.q_m[t] - m0, 8u);
             const uint4 v = __ldg(reinterpret_cast<const uint4 *>(a.cells) + u);
             const uint32_t cv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -1236,13 +1247,13 @@ __device__ void cta_srp(const QArgs &a, const HArgs &h, uint32_t q, uint32_t *qb
 // Bound by latency and instruction issue, not by DRAM: at the recall-target
 // genomic shape a query's 8,000 cycles of hashing, 20,000 of gathering and
 // 60,000 of decoding are chains of dependent L2 and DRAM loads and barriers, which
-// four to eight resident CTAs per SM overlap (32 registers a thread; 48 and 64
-// with fewer CTAs measured slower on most shapes). Default launch shapes, same
+// four to eight resident CTAs per SM overlap (32 registers a thread; with 16-bit
+// counts also 64, where shared memory admits no more than 1,024 threads anyway). Default launch shapes, same
 // box, before the walk's filter, the gather's 16-byte units and the score
 // histogram, and after: 1,000 genomic queries 197 -> 121 us, 10^4 URL queries
 // 2.66 -> 1.54 ms, the plain form's 10^4 embedding queries 2.95 -> 1.49 ms.
-template <int NT, int RW, int HASH, int CW>
-__global__ void __launch_bounds__(NT, (HASH == 2 ? 1024 : 2048) / NT)
+template <int NT, int RW, int HASH, int CW, int FT>
+__global__ void __launch_bounds__(NT, FT / NT)
 k_query_fused(QArgs a, HArgs h)
 {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -1310,23 +1321,29 @@ const void *plain_kernel_t(int NT, uint32_t rw)
 #undef FL_PLAIN
 }
 
+// sm_threads: the threads per SM that the kernel's registers allow: 1,024 (64
+// registers) or 2,048 (32). The SRP hash needs the former; with 8-bit counts the
+// latter is compiled alone.
 template <int CW>
-const void *fused_kernel_t(int NT, uint32_t rw, bool srp)
+const void *fused_kernel_t(int NT, uint32_t rw, bool srp, uint32_t sm_threads)
 {
-#define FL_FUSED(N) \
-    switch ((srp ? 10 : 0) + rw) { \
-    case 1: return (const void *)k_query_fused<N, 1, 1, CW>; \
-    case 2: return (const void *)k_query_fused<N, 2, 1, CW>; \
-    case 4: return (const void *)k_query_fused<N, 4, 1, CW>; \
-    case 8: return (const void *)k_query_fused<N, 8, 1, CW>; \
-    case 11: return (const void *)k_query_fused<N, 1, 2, CW>; \
-    case 12: return (const void *)k_query_fused<N, 2, 2, CW>; \
-    case 14: return (const void *)k_query_fused<N, 4, 2, CW>; \
-    default: return (const void *)k_query_fused<N, 8, 2, CW>; \
+#define FL_FUSED(N, H, FT) \
+    switch (rw) { \
+    case 1: return (const void *)k_query_fused<N, 1, H, CW, FT>; \
+    case 2: return (const void *)k_query_fused<N, 2, H, CW, FT>; \
+    case 4: return (const void *)k_query_fused<N, 4, H, CW, FT>; \
+    default: return (const void *)k_query_fused<N, 8, H, CW, FT>; \
     }
-    if (NT == 128) { FL_FUSED(128) }
-    if (NT == 512) { FL_FUSED(512) }
-    FL_FUSED(256)
+#define FL_FUSED_N(H, FT) \
+    if (NT == 128) { FL_FUSED(128, H, FT) } \
+    if (NT == 512) { FL_FUSED(512, H, FT) } \
+    FL_FUSED(256, H, FT)
+    if (srp) { FL_FUSED_N(2, 1024) }
+    if constexpr (CW == 2) {
+        if (sm_threads == 1024) { FL_FUSED_N(1, 1024) }
+    }
+    FL_FUSED_N(1, 2048)
+#undef FL_FUSED_N
 #undef FL_FUSED
 }
 
@@ -1335,10 +1352,10 @@ const void *fused_kernel_t(int NT, uint32_t rw, bool srp)
 // Per count width: the plain, fused and counts kernels (query.cu: CW = 1,
 // query_c16.cu: CW = 2).
 const void *plain_kernel_c1(int NT, uint32_t rw);
-const void *fused_kernel_c1(int NT, uint32_t rw, bool srp);
+const void *fused_kernel_c1(int NT, uint32_t rw, bool srp, uint32_t sm_threads);
 const void *counts_kernel_c1();
 const void *plain_kernel_c2(int NT, uint32_t rw);
-const void *fused_kernel_c2(int NT, uint32_t rw, bool srp);
+const void *fused_kernel_c2(int NT, uint32_t rw, bool srp, uint32_t sm_threads);
 const void *counts_kernel_c2();
 
 }  // namespace flinng
