@@ -650,15 +650,16 @@ size_t insert_workspace_bytes(const flinng_index *ix, uint64_t n, bool reset)
     if ((reset || ix->n_points == 0) && part_build_applies(ix, n))
         return carve_bytes<uint32_t>(ix->BR + 1) +
                std::max(part_workspace_bytes(ix, n), scan_workspace_bytes(size_t(ix->BR) + 1)) + 256;
-    if (!reset && delta_insert_applies(ix, n))
-        return carve_bytes<uint32_t>(ix->BR + 1) +
-               std::max(delta_workspace_bytes(ix, n), scan_workspace_bytes(size_t(ix->BR) + 1)) + 256;
+    const size_t delta = carve_bytes<uint32_t>(ix->BR + 1) +
+                         std::max(delta_workspace_bytes(ix, n), scan_workspace_bytes(size_t(ix->BR) + 1)) + 256;
+    if (!reset && delta_insert_applies(ix, n)) return delta;
     const size_t ns = ix->nslot + 1;
     const size_t big = ns > size_t(ix->BR) + 1 ? ns : size_t(ix->BR) + 1;
     const uint64_t D = n * ix->cfg.L * ix->cfg.R;
-    return 2 * carve_bytes<uint32_t>(ns) + carve_bytes<uint32_t>(ix->BR + 1) +
-           carve_bytes<uint32_t>(worklist_entries(ix, n, reset)) + carve_bytes<uint32_t>(4) +
-           (reset ? 0 : carve_bytes<uint16_t>(D)) + scan_workspace_bytes(big);
+    const size_t full = 2 * carve_bytes<uint32_t>(ns) + carve_bytes<uint32_t>(ix->BR + 1) +
+                        carve_bytes<uint32_t>(worklist_entries(ix, n, reset)) + carve_bytes<uint32_t>(4) +
+                        (reset ? 0 : carve_bytes<uint16_t>(D)) + scan_workspace_bytes(big);
+    return !reset && delta_part_applies(ix, n) ? std::max(delta, full) : full;
 }
 
 int check_groups(flinng_index *ix, const uint16_t *groups, uint64_t n)
@@ -735,15 +736,17 @@ int insert_hashed(flinng_index *ix, uint32_t *buckets, const uint32_t *perm, con
     const uint64_t n_old = ix->n_points, N = n_old + n, nslot = ix->nslot;
     const bool have_old = ix->n_cells > 0;
     const uint64_t D = n * L * R;   // new (table, cell) entries before deduplication
-    const bool delta = delta_insert_applies(ix, n);
+    const bool delta = delta_insert_applies(ix, n) || delta_part_applies(ix, n);
     Carver c(ws, ~size_t(0));
     uint32_t *mcur = c.take<uint32_t>(BR + 1);
     if (delta) {
-        // a small batch: only the slots that gain cells are merged
+        // only the slots that gain cells are merged
         void *dws = c.base + ((c.used + 255) & ~size_t(255));
         FL_TRY(member_stage(ix, perm, groups, n, mcur, dws));
         TraceRange stage2("reverse index (delta)");
-        return insert_delta(ix, buckets, n, dws);
+        bool done = false;
+        FL_TRY(insert_delta(ix, buckets, n, dws, &done));
+        if (done) return FLINNG_OK;
     }
     if (n_old == 0 && part_build_applies(ix, n)) {
         // from scratch: sorted partition by partition in shared memory
@@ -771,7 +774,7 @@ int insert_hashed(flinng_index *ix, uint32_t *buckets, const uint32_t *perm, con
     uint16_t *dbuf = have_old ? c.take<uint16_t>(D) : ix->cells_tmp;
     void *scan_ws = c.base + ((c.used + 255) & ~size_t(255));
 
-    FL_TRY(member_stage(ix, perm, groups, n, mcur, scan_ws));
+    if (!delta) FL_TRY(member_stage(ix, perm, groups, n, mcur, scan_ws));
 
     TraceRange stage2("reverse index");    // 1. the new entries by slot: counting sort (histogram, scan, scatter)
     uint32_t *hist = ix->slot_a;

@@ -749,6 +749,34 @@ bool plan_for(const flinng_index *ix, uint64_t n, PartPlan *pl)
 
 }  // namespace
 
+// Steps 1 and 2 for n new points: part (n x L entries) grouped by (table, top C
+// bucket bits) with the groups' bases in pbase (L << C of them, the total last);
+// bt: room for L x n buckets (dead afterwards; may be anything but buckets and
+// part), pcur: L << C words of scratch.
+int partition_entries(flinng_index *ix, const uint32_t *buckets, uint64_t n, uint32_t C, uint32_t idbits, uint32_t *bt,
+                      uint32_t *part, uint32_t *pbase, uint32_t *pcur, void *scan_ws)
+{
+    const cudaStream_t st = ix->stream;
+    const uint32_t L = ix->cfg.L, low = ix->cfg.range_bits - C;
+    const uint64_t parts = uint64_t(L) << C;
+    FL_CUDA(cudaMemsetAsync(pcur, 0, parts * sizeof(uint32_t), st));
+    k_transpose<<<dim3(unsigned((n + 31) / 32), (L + 31) / 32), 256, 0, st>>>(buckets, n, L, bt);
+    count_launch();
+    FL_CUDA(cudaGetLastError());
+    const dim3 tiles(unsigned((n + kTile - 1) / kTile), L);
+    k_part_count<<<tiles, kT, sizeof(uint32_t) << C, st>>>(bt, n, C, low, pcur);
+    count_launch();
+    FL_CUDA(cudaGetLastError());
+    FL_TRY(scan_exclusive(pcur, pbase, parts, scan_ws, st));
+    FL_CUDA(cudaMemcpyAsync(pcur, pbase, parts * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st));
+    const size_t ssm = (sizeof(uint32_t) * 2 << C) + kTile * 6 + (kT / 32) * 4;
+    FL_TRY(ensure_dyn_smem((const void *)k_part_scatter, ssm));
+    k_part_scatter<<<tiles, kT, ssm, st>>>(bt, n, C, low, idbits, pcur, part);
+    count_launch();
+    FL_CUDA(cudaGetLastError());
+    return FLINNG_OK;
+}
+
 // The build scratch and the list array double as the pass buffers (four
 // bytes per entry), which takes R >= 2; the general path of build.cu covers
 // the rest. heavy_min >= 32 and the list in shared memory bound R and B*R no
@@ -792,22 +820,8 @@ int part_build(flinng_index *ix, uint32_t *buckets, uint64_t n, void *ws, uint32
     // array (2 R bytes per entry), which receives the lists only at the end
     uint32_t *bt = reinterpret_cast<uint32_t *>(ix->cells);
     uint32_t *part = buckets;
-    FL_CUDA(cudaMemsetAsync(pcur, 0, (pl.parts + 1) * sizeof(uint32_t), st));
     FL_CUDA(cudaMemsetAsync(cnt, 0, 4 * sizeof(uint32_t), st));
-    k_transpose<<<dim3(unsigned((n + 31) / 32), (L + 31) / 32), 256, 0, st>>>(buckets, n, L, bt);
-    count_launch();
-    FL_CUDA(cudaGetLastError());
-    const dim3 tiles(unsigned((n + kTile - 1) / kTile), L);
-    k_part_count<<<tiles, kT, sizeof(uint32_t) << pl.C, st>>>(bt, n, pl.C, pl.low, pcur);
-    count_launch();
-    FL_CUDA(cudaGetLastError());
-    FL_TRY(scan_exclusive(pcur, pbase, pl.parts, scan_ws, st));
-    FL_CUDA(cudaMemcpyAsync(pcur, pbase, pl.parts * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st));
-    const size_t ssm = (sizeof(uint32_t) * 2 << pl.C) + kTile * 6 + (kT / 32) * 4;
-    FL_TRY(ensure_dyn_smem((const void *)k_part_scatter, ssm));
-    k_part_scatter<<<tiles, kT, ssm, st>>>(bt, n, pl.C, pl.low, pl.idbits, pcur, part);
-    count_launch();
-    FL_CUDA(cudaGetLastError());
+    FL_TRY(partition_entries(ix, buckets, n, pl.C, pl.idbits, bt, part, pbase, pcur, scan_ws));
     FineArgs a{};
     a.part = part;
     a.pbase = pbase;

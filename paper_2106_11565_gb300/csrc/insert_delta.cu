@@ -5,7 +5,10 @@
 // array each take one streaming pass, and no work runs per slot of the whole
 // index (L * 2^W slots, most of them untouched by a batch).
 //
-//  1. k_delta_table, one CTA per table: the batch's (bucket, cell) entries of
+//  0. A batch of more than kDeltaMaxKeys cells per table: the entries
+//     partitioned by the top bits of their bucket (build_part.cu); below, a
+//     segment is a table, or such a partition of it.
+//  1. k_delta_table, one CTA per segment: the batch's (bucket, cell) entries of
 //     table l (n * R of them) sorted in shared memory, deduplicated (a filter
 //     bit is set once, Sec. 3.3), and stripped of the cells the slot's list
 //     already holds; what remains is "added". The table's touched slots
@@ -100,27 +103,46 @@ __device__ __forceinline__ uint32_t rank_u16(const uint16_t *a, uint32_t n, uint
 }
 
 // Step 1. Keys are (bucket << CB) | cell (CB bits hold a cell id), 32-bit
-// when W + CB <= 31; P2 (a power of two, 32 .. 32 E blockDim, >= n R) of
-// them in shared memory, E = max(1, P2 / blockDim) per thread.
+// when W + CB <= 31; P2 (a power of two, 32 .. E blockDim, >= the segment's
+// cells) of them in shared memory, E per thread. Segment l is table l, or with
+// pbase partition l: W is then the bits below the partition's, part its packed
+// entries, and a partition of more than P2max cells only sets *over.
 template <class KT, int E>
 __global__ void __launch_bounds__(kDeltaThreads)
 k_delta_table(const uint32_t *__restrict__ buckets, const uint16_t *__restrict__ gid, uint64_t n_old, uint32_t n,
-              uint32_t L, uint32_t W, uint32_t R, uint32_t B, uint32_t rp, uint32_t P2, uint32_t CB,
+              uint32_t L, uint32_t W, uint32_t R, uint32_t B, uint32_t rp, uint32_t P2max, uint32_t CB,
               const uint32_t *__restrict__ off, const uint16_t *__restrict__ cells, uint16_t *__restrict__ rcell,
-              uint2 *__restrict__ rt, uint32_t *__restrict__ A, uint32_t *__restrict__ T)
+              uint2 *__restrict__ rt, uint32_t *__restrict__ A, uint32_t *__restrict__ T,
+              const uint32_t *__restrict__ pbase, const uint32_t *__restrict__ part, uint32_t idbits,
+              uint32_t *__restrict__ over)
 {
     constexpr KT kNone = ~KT(0);
     extern __shared__ __align__(16) unsigned char dsm[];
     KT *key = reinterpret_cast<KT *>(dsm);
-    uint32_t *wsum = reinterpret_cast<uint32_t *>(key + P2);
-    const uint32_t l = blockIdx.x, nR = n * R, tid = threadIdx.x, nt = blockDim.x;
+    uint32_t *wsum = reinterpret_cast<uint32_t *>(key + P2max);
+    const uint32_t l = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
+    const uint32_t e0 = pbase ? pbase[l] : 0u, nR = (pbase ? pbase[l + 1] - e0 : n) * R;
+    const uint64_t seg = pbase ? uint64_t(e0) * R : uint64_t(l) * nR;      // where this segment's results go
+    uint32_t P2 = P2max;
+    if (pbase) {
+        if (nR == 0 || nR > P2max) {
+            if (tid == 0) {
+                A[l] = T[l] = 0u;
+                if (nR) atomicOr(over, 1u);
+            }
+            return;
+        }
+        for (P2 = 32 * E; P2 < nR; P2 <<= 1) {}
+    }
     const KT cmask = (KT(1) << CB) - 1;
     for (uint32_t i = tid; i < P2; i += nt) {
         KT k = kNone;
         if (i < nR) {
             const uint32_t x = i / R, r = i - x * R;
-            const uint32_t b = buckets[uint64_t(x) * L + l];
-            const uint32_t c = r * B + gid[(n_old + x) * rp + r];
+            const uint32_t ent = pbase ? part[e0 + x] : 0u;
+            const uint32_t b = pbase ? ent >> idbits : buckets[uint64_t(x) * L + l];
+            const uint32_t id = pbase ? ent & ((1u << idbits) - 1u) : x;
+            const uint32_t c = r * B + gid[(n_old + id) * rp + r];
             k = (KT(b) << CB) | KT(c);
         }
         key[i] = k;
@@ -232,7 +254,7 @@ k_delta_table(const uint32_t *__restrict__ buckets, const uint16_t *__restrict__
         if (e >= E) break;
         const uint32_t i = i0 + e;
         if (i >= nA) break;
-        rcell[uint64_t(l) * nR + i] = uint16_t(key[i] & cmask);
+        rcell[seg + i] = uint16_t(key[i] & cmask);
         if (i == 0 || (key[i] >> CB) != (key[i - 1] >> CB)) {
             tm |= 1u << e;
             ++tcnt;
@@ -242,17 +264,18 @@ k_delta_table(const uint32_t *__restrict__ buckets, const uint16_t *__restrict__
     uint32_t tp = cta_excl_scan(tcnt, wsum, &nT);
 #pragma unroll
     for (uint32_t e = 0; e < 8; ++e)
-        if ((tm >> e) & 1u) rt[uint64_t(l) * nR + tp++] = make_uint2(uint32_t(key[i0 + e] >> CB), i0 + e);
+        if ((tm >> e) & 1u) rt[seg + tp++] = make_uint2(uint32_t(key[i0 + e] >> CB), i0 + e);
     if (tid == 0) {
         A[l] = nA;
         T[l] = nT;
     }
 }
 
-// Step 2. Apre, Tpre: exclusive prefixes of A, T over the tables (L + 1
+// Step 2. Apre, Tpre: exclusive prefixes of A, T over the L segments (L + 1
 // entries, totals last). Sentinels close gslot / gdbeg / gend.
 __global__ void k_delta_flatten(const uint32_t *__restrict__ Apre, const uint32_t *__restrict__ Tpre, uint32_t L,
-                                uint32_t W, uint32_t nR, const uint16_t *__restrict__ rcell,
+                                uint32_t W, uint32_t nR, const uint32_t *__restrict__ pbase, uint32_t R,
+                                const uint16_t *__restrict__ rcell,
                                 const uint2 *__restrict__ rt, const uint32_t *__restrict__ off,
                                 uint32_t *__restrict__ gslot, uint32_t *__restrict__ gdbeg,
                                 uint32_t *__restrict__ gbeg, uint32_t *__restrict__ gend,
@@ -260,9 +283,10 @@ __global__ void k_delta_flatten(const uint32_t *__restrict__ Apre, const uint32_
 {
     const uint32_t l = blockIdx.x;
     const uint32_t a0 = Apre[l], na = Apre[l + 1] - a0, t0 = Tpre[l], ntt = Tpre[l + 1] - t0;
-    for (uint32_t i = threadIdx.x; i < na; i += blockDim.x) gdcell[a0 + i] = rcell[uint64_t(l) * nR + i];
+    const uint64_t seg = pbase ? uint64_t(pbase[l]) * R : uint64_t(l) * nR;
+    for (uint32_t i = threadIdx.x; i < na; i += blockDim.x) gdcell[a0 + i] = rcell[seg + i];
     for (uint32_t j = threadIdx.x; j < ntt; j += blockDim.x) {
-        const uint2 t = rt[uint64_t(l) * nR + j];
+        const uint2 t = rt[seg + j];
         const uint32_t slot = (l << W) | t.x;
         gslot[t0 + j] = slot;
         gdbeg[t0 + j] = a0 + t.y;
@@ -487,22 +511,22 @@ inline unsigned blocks_of(uint64_t items, uint64_t per)
 }
 
 template <class KT, int E, class... Args>
-int launch_table_e(uint32_t grid, uint32_t P2, cudaStream_t st, Args... args)
+int launch_table_e(uint32_t grid, uint32_t threads, uint32_t P2, cudaStream_t st, Args... args)
 {
     const size_t smem = size_t(P2) * sizeof(KT) + 32 * 4;
     FL_TRY(ensure_dyn_smem((const void *)k_delta_table<KT, E>, smem));
-    k_delta_table<KT, E><<<grid, kDeltaThreads, smem, st>>>(args...);
+    k_delta_table<KT, E><<<grid, threads, smem, st>>>(args...);
     return FLINNG_OK;
 }
 
 template <class KT, class... Args>
-int launch_table(int E, uint32_t grid, uint32_t P2, cudaStream_t st, Args... args)
+int launch_table(int E, uint32_t grid, uint32_t threads, uint32_t P2, cudaStream_t st, Args... args)
 {
     switch (E) {
-    case 8: return launch_table_e<KT, 8>(grid, P2, st, args...);
-    case 4: return launch_table_e<KT, 4>(grid, P2, st, args...);
-    case 2: return launch_table_e<KT, 2>(grid, P2, st, args...);
-    default: return launch_table_e<KT, 1>(grid, P2, st, args...);
+    case 8: return launch_table_e<KT, 8>(grid, threads, P2, st, args...);
+    case 4: return launch_table_e<KT, 4>(grid, threads, P2, st, args...);
+    case 2: return launch_table_e<KT, 2>(grid, threads, P2, st, args...);
+    default: return launch_table_e<KT, 1>(grid, threads, P2, st, args...);
     }
 }
 
@@ -513,24 +537,72 @@ bool delta_insert_applies(const flinng_index *ix, uint64_t n)
     return ix->n_cells > 0 && n > 0 && n * ix->cfg.R <= kDeltaMaxKeys;
 }
 
-size_t delta_workspace_bytes(const flinng_index *ix, uint64_t n)
+namespace {
+
+// Partitioned batches: coarse bits so that a partition's cells average at most
+// kPartCells, a third of what its CTA sorts (kPartThreads x 8).
+constexpr uint32_t kPartCells = 640, kPartThreads = 256;
+
+struct DeltaPlan {
+    uint32_t C, low, idbits;
+    uint64_t segs;             // tables or partitions
+};
+
+bool delta_plan(const flinng_index *ix, uint64_t n, bool part, DeltaPlan *pl)
 {
-    const uint64_t L = ix->cfg.L, nR = n * ix->cfg.R, D = L * nR;
-    return carve_bytes<uint16_t>(D) + carve_bytes<uint2>(D) + 4 * carve_bytes<uint32_t>(L + 1) +
-           4 * carve_bytes<uint32_t>(D + 1) + carve_bytes<uint16_t>(D) + carve_bytes<uint32_t>(D + 1) +
-           carve_bytes<uint32_t>(4) + scan_workspace_bytes(L + 1) +
-           2 * carve_bytes<uint32_t>(std::max(ix->nslot + 1, ix->n_cells + n * L * ix->cfg.R) / kChunk + 3);
+    const uint32_t W = ix->cfg.range_bits;
+    uint32_t C = 0, idbits = 1;
+    if (part) {
+        while (C < 11 && C < W && ((n * ix->cfg.R) >> C) > kPartCells) ++C;
+        while (idbits < 32 && (n - 1) >> idbits) ++idbits;
+    }
+    *pl = DeltaPlan{C, W - C, idbits, uint64_t(ix->cfg.L) << C};
+    return !part || pl->low + idbits <= 32;
 }
 
-int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws)
+}  // namespace
+
+// A larger batch, partitioned, while its cells are at most a third of the
+// index's: into 20,000 reads at the recall-target parameters, 6,000 more take
+// 1.40 ms against 2.14 with the full merge's six passes over all 67 M slots,
+// 19,000 more 3.30 against 2.78; into 100,000, 10,000 take 2.34 against 3.42,
+// 20,000 3.79 against 4.00. At most 2^25 cells (32 bytes of workspace each).
+// R >= 2: the list scratch has room for the transposed buckets.
+bool delta_part_applies(const flinng_index *ix, uint64_t n)
 {
+    const uint64_t D = n * ix->cfg.L * ix->cfg.R;
+    DeltaPlan pl;
+    return ix->n_cells > 0 && ix->cfg.R >= 2 && n * ix->cfg.R > kDeltaMaxKeys && 3 * D <= ix->n_cells &&
+           D <= (1ull << 25) && delta_plan(ix, n, true, &pl);
+}
+
+size_t delta_workspace_bytes(const flinng_index *ix, uint64_t n)
+{
+    const bool part = delta_part_applies(ix, n);
+    DeltaPlan pl;
+    if (!part && !delta_insert_applies(ix, n)) return 0;
+    delta_plan(ix, n, part, &pl);
+    const uint64_t D = n * ix->cfg.L * ix->cfg.R;
+    return carve_bytes<uint16_t>(D) + carve_bytes<uint2>(D) + 4 * carve_bytes<uint32_t>(pl.segs + 1) +
+           4 * carve_bytes<uint32_t>(D + 1) + carve_bytes<uint16_t>(D) + carve_bytes<uint32_t>(D + 1) +
+           carve_bytes<uint32_t>(4) + scan_workspace_bytes(pl.segs + 1) +
+           2 * carve_bytes<uint32_t>(std::max(ix->nslot + 1, ix->n_cells + D) / kChunk + 3) +
+           (part ? carve_bytes<uint32_t>(n * ix->cfg.L) + 2 * carve_bytes<uint32_t>(pl.segs + 1) : 0);
+}
+
+int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws, bool *done)
+{
+    *done = false;
     const cudaStream_t st = ix->stream;
-    const uint32_t R = ix->cfg.R, B = ix->cfg.B, L = ix->cfg.L, W = ix->cfg.range_bits;
+    const uint32_t R = ix->cfg.R, B = ix->cfg.B, W = ix->cfg.range_bits;
     const uint64_t n_old = ix->n_points, nslot = ix->nslot, n_cells = ix->n_cells;
-    const uint32_t nR = uint32_t(n * R);
-    const uint64_t D = uint64_t(L) * nR;
-    if (!delta_insert_applies(ix, n))
+    const uint64_t D = n * ix->cfg.L * R;
+    const bool part = !delta_insert_applies(ix, n);
+    DeltaPlan pl;
+    if ((part && !delta_part_applies(ix, n)) || !delta_plan(ix, n, part, &pl))
         return set_error(FLINNG_ERR_INVALID_ARG, "internal: delta insert of %llu points", (unsigned long long)n);
+    const uint32_t L = uint32_t(pl.segs), low = part ? pl.low : W;       // L: segments from here on
+    const uint32_t nR = part ? 0u : uint32_t(n * R);
     Carver c(ws, ~size_t(0));
     uint16_t *rcell = c.take<uint16_t>(D);
     uint2 *rt = c.take<uint2>(D);
@@ -543,23 +615,42 @@ int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws
     const uint64_t nchunk = std::max(nslot + 1, n_cells) / kChunk + 2;
     uint32_t *off_j = c.take<uint32_t>(nchunk + 1), *mov_lo = c.take<uint32_t>(nchunk);
     uint32_t *cnt = c.take<uint32_t>(4);
+    uint32_t *ent = nullptr, *pbase = nullptr, *pcur = nullptr;
+    if (part) {
+        ent = c.take<uint32_t>(n * ix->cfg.L);
+        pbase = c.take<uint32_t>(L + 1);
+        pcur = c.take<uint32_t>(L + 1);
+    }
     void *scan_ws = c.base + ((c.used + 255) & ~size_t(255));
 
-    const uint32_t P2 = pow2_ceil(nR < 32 ? 32u : nR);
+    FL_CUDA(cudaMemsetAsync(cnt, 0, 4 * sizeof(uint32_t), st));
+    // the transposed buckets pass through the list scratch, written only by the merge
+    if (part) FL_TRY(partition_entries(ix, buckets, n, pl.C, pl.idbits, reinterpret_cast<uint32_t *>(ix->cells_tmp), ent,
+                                       pbase, pcur, scan_ws));
+    const uint32_t P2 = part ? kPartThreads * 8 : pow2_ceil(nR < 32 ? 32u : nR);
     uint32_t CB = 1;
     while ((1u << CB) < ix->BR) ++CB;
-    const int E = P2 >= 8192 ? 8 : P2 >= 4096 ? 4 : P2 >= 2048 ? 2 : 1;
-    if (W + CB <= 31)        // all-ones marks padding: real keys stay below it
-        FL_TRY(launch_table<uint32_t>(E, L, P2, st, buckets, ix->gid, n_old, uint32_t(n), L, W, R, B, ix->rp, P2,
-                                      CB, ix->off, ix->cells, rcell, rt, A, T));
+    const int E = part ? 8 : P2 >= 8192 ? 8 : P2 >= 4096 ? 4 : P2 >= 2048 ? 2 : 1;
+    const uint32_t threads = part ? kPartThreads : uint32_t(kDeltaThreads);
+    if (low + CB <= 31)        // all-ones marks padding: real keys stay below it
+        FL_TRY(launch_table<uint32_t>(E, L, threads, P2, st, buckets, ix->gid, n_old, uint32_t(n), L, low, R, B, ix->rp,
+                                      P2, CB, ix->off, ix->cells, rcell, rt, A, T, pbase, ent, pl.idbits, cnt + 1));
     else
-        FL_TRY(launch_table<uint64_t>(E, L, P2, st, buckets, ix->gid, n_old, uint32_t(n), L, W, R, B, ix->rp, P2,
-                                      CB, ix->off, ix->cells, rcell, rt, A, T));
+        FL_TRY(launch_table<uint64_t>(E, L, threads, P2, st, buckets, ix->gid, n_old, uint32_t(n), L, low, R, B, ix->rp,
+                                      P2, CB, ix->off, ix->cells, rcell, rt, A, T, pbase, ent, pl.idbits, cnt + 1));
     count_launch();
     FL_CUDA(cudaGetLastError());
+    if (part) {
+        // a partition past what a CTA sorts (buckets that many points share): the
+        // full merge, before anything of the index changes
+        FL_CUDA(cudaMemcpyAsync(ix->h_flag, cnt + 1, 4, cudaMemcpyDeviceToHost, st));
+        FL_CUDA(cudaStreamSynchronize(st));
+        if (ix->h_flag[0]) return FLINNG_OK;
+    }
     FL_TRY(scan_exclusive(A, Apre, L, scan_ws, st));
     FL_TRY(scan_exclusive(T, Tpre, L, scan_ws, st));
-    k_delta_flatten<<<L, 256, 0, st>>>(Apre, Tpre, L, W, nR, rcell, rt, ix->off, gslot, gdbeg, gbeg, gend, gdcell);
+    k_delta_flatten<<<L, part ? 128 : 256, 0, st>>>(Apre, Tpre, L, low, nR, pbase, R, rcell, rt, ix->off, gslot, gdbeg,
+                                                    gbeg, gend, gdcell);
     count_launch();
     FL_CUDA(cudaGetLastError());
     uint32_t *noff = ix->slot_b;
@@ -570,7 +661,6 @@ int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws
     FL_CUDA(cudaGetLastError());
     // the merge writes only the touched slots' new lists, the streaming passes
     // only the other lists and the offsets: the merge runs beside them
-    FL_CUDA(cudaMemsetAsync(cnt, 0, 4 * sizeof(uint32_t), st));
     if (!ix->side) {
         FL_CUDA(cudaStreamCreateWithFlags(&ix->side, cudaStreamNonBlocking));
         FL_CUDA(cudaEventCreateWithFlags(&ix->ev_fork, cudaEventDisableTiming));
@@ -623,6 +713,7 @@ int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws
     ix->n_cells = n_cells + added;
     ix->n_heavy += nh_new;
     ix->n_points = n_old + n;
+    *done = true;
     return FLINNG_OK;
 }
 

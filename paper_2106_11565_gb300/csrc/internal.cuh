@@ -226,6 +226,8 @@ int heavy_bitmaps(flinng_index *ix, const uint32_t *list, const uint32_t *count)
 // ---- build_part.cu
 // A build from scratch sorts its entries partition by partition in shared
 // memory where part_build_applies.
+int partition_entries(flinng_index *ix, const uint32_t *buckets, uint64_t n, uint32_t C, uint32_t idbits, uint32_t *bt,
+                      uint32_t *part, uint32_t *pbase, uint32_t *pcur, void *scan_ws);
 bool part_build_applies(const flinng_index *ix, uint64_t n);
 size_t part_workspace_bytes(const flinng_index *ix, uint64_t n);
 int part_build(flinng_index *ix, uint32_t *buckets, uint64_t n, void *ws, uint32_t **list_out, uint32_t **count_out);
@@ -259,12 +261,16 @@ int counts_launch(flinng_index *ix, const uint32_t *qbuckets, uint32_t nq,
 // ---- insert_delta.cu
 // An insert of n points into a built index merges only the slots that gain
 // cells when n * R <= kDeltaMaxKeys (the batch's entries of one table are
-// sorted in shared memory); larger batches take the full merge of build.cu.
+// sorted in shared memory) or delta_part_applies (a table's entries are first
+// partitioned by bucket); other batches take the full merge of build.cu.
 constexpr uint32_t kDeltaMaxKeys = 8192;
 bool delta_insert_applies(const flinng_index *ix, uint64_t n);
+bool delta_part_applies(const flinng_index *ix, uint64_t n);
 size_t delta_workspace_bytes(const flinng_index *ix, uint64_t n);
 // After insert_hashed's group and member-list stage: the reverse index.
-int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws);
+// *done stays false, and the index as it was, when a partition of a
+// partitioned batch was too large (the caller takes the full merge).
+int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws, bool *done);
 
 // ---- probe.cu
 // Multi-probe counts (probes P >= 1 per table): nq x B*R uint16, each <= L.

@@ -58,3 +58,33 @@ def test_csr_equals_oracle(F, n, L, W, R, B, kind):
     for i in range(12):
         assert np.array_equal(got[i], O.counts(off, cells, L, W, q[i], B * R))
     ix.close()
+
+
+@pytest.mark.parametrize("universe,W,R,B", [(50_000, 14, 3, 300), (50_000, 20, 2, 5000), (400, 5, 4, 60), (3, 9, 3, 500),
+                                            (9000, 9, 1, 200)])
+def test_large_inserts_equal_oracle(F, universe, W, R, B):
+    """Batches past the one-CTA-per-table limit: partitioned where their buckets
+    spread, the full merge where many points share a bucket (a universe of three
+    elements) or the batch outnumbers the index, R = 1 always."""
+    L = 9
+    sizes = [24_000, 5000, 9001, 30_000]
+    N = sum(sizes)
+    off, el = WL.random_sets(70 + W, N, universe, 1, min(universe, 40))
+    dp = WL.doph_params(71, L, 1)
+    ix = F.Index("jaccard", R, B, L, 1, capacity=N, params=dp, W=W)
+    o = O.OracleIndex("jaccard", R, B, L, 1, W, doph=dp)
+    lo = 0
+    for step, n in enumerate(sizes):
+        part = (off[lo:lo + n + 1] - off[lo]).astype(np.uint64), np.ascontiguousarray(el[off[lo]:off[lo + n]])
+        perm = WL.group_permutations(72, R, n, batch=step)
+        (ix.build if step == 0 else ix.insert)(part, perm)
+        o.insert(part, perm)
+        lo += n
+        ex = ix.export()
+        assert np.array_equal(ex["gid"], o.gid), step
+        assert np.array_equal(ex["off"], o.off) and np.array_equal(ex["cells"], o.cells), step
+        q = o.buckets[:: max(1, lo // 7)]
+        got = ix.counts(q)
+        for i in range(len(q)):
+            assert np.array_equal(got[i], O.counts(o.off, o.cells, L, W, q[i], B * R)), step
+    ix.close()
