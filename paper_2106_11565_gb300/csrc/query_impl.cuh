@@ -634,10 +634,9 @@ __device__ __forceinline__ void for_level_cells(const QArgs &a, const QSmem &s, 
 // groups of its unit's members with one 16-byte load and drops those whose
 // repetition-1 cell is below the admission bound; of the thousands of members
 // a query walks almost all go there, at 2 bytes and about five instructions
-// each instead of a record of 8 to 32 bytes and a key. The few that pass are
-// queued and decoded 32 at a time; a step with many (no bound yet) decodes
-// them at once. VS = 0, for cells of a few members, or while most would pass
-// the filter: one member per lane.
+// each instead of a record of 8 to 32 bytes and a key. Those that pass are
+// queued and decoded 32 at a time. VS = 0, for cells of a few members, or while
+// most would pass the filter: one member per lane, decoded at once.
 //
 // Candidates are appended without reservations: a warp reads the buffer fill
 // first and appends (at most 32 keys) only while it is at or below hwm. Above
@@ -666,8 +665,9 @@ __device__ void walk_members(const QArgs &a, const QSmem &s, const uint16_t *cel
     for (;;) {
         const uint32_t smin = max(a.t_min, bscore);   // lower scores cannot enter
         for (;;) {
-            const bool dense = __any_sync(0xffffffffu, pend != 0u);
-            if (!dense && qn < 32u && jb < je) {
+            const bool more = __any_sync(0xffffffffu, pend != 0u);
+            const bool dense = VS == 0 && more;
+            if (!more && qn < 32u && jb < je) {
                 // lanes to cells: one warp-uniform pass over the cell boundaries
                 // inside this step; c_pre is M past the chunk's last cell and ~0 at
                 // the array's end, so the pass stops at the step's last unit
@@ -704,27 +704,29 @@ __device__ void walk_members(const QArgs &a, const QSmem &s, const uint16_t *cel
                         }
                     }
                 }
-                if constexpr (VS == 3) {
-                    const uint32_t np = __popc(pend), total = __reduce_add_sync(0xffffffffu, np);
-                    if (total > 0u && total <= 32u) {          // qn + total <= kWarpQueue
-                        uint32_t x = np;
+                if constexpr (VS == 0) continue;
+            }
+            if (VS == 3 && qn < 32u && __any_sync(0xffffffffu, pend != 0u)) {
+                // the members that passed go to the queue, as many as fit; the
+                // others wait in pend, so that 32 are always decoded together
+                const uint32_t np = __popc(pend);
+                uint32_t x = np;
 #pragma unroll
-                        for (int d = 1; d < 32; d <<= 1) {
-                            const uint32_t y = __shfl_up_sync(0xffffffffu, x, d);
-                            if (lane >= d) x += y;
-                        }
-                        uint32_t at = qn + x - np;
-                        for (; pend; pend &= pend - 1u, ++at) {
-                            qm[at] = m0 + __ffs(pend) - 1;
-                            qc[at] = uint16_t(my_cell);
-                        }
-                        qn += total;
-                        __syncwarp();
-                    }
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xffffffffu, x, d);
+                    if (lane >= d) x += y;
                 }
+                uint32_t at = qn + x - np;
+                for (; pend && at < kWarpQueue; pend &= pend - 1u, ++at) {
+                    qm[at] = m0 + __ffs(pend) - 1;
+                    qc[at] = uint16_t(my_cell);
+                }
+                qn = min(qn + __shfl_sync(0xffffffffu, x, 31), kWarpQueue);
+                __syncwarp();
                 continue;
             }
-            // decode one member per lane: of the step's pending ones, or the queue's last
+            if (VS == 3 && qn < 32u && jb < je) continue;      // nothing passed: the next step
+            // decode one member per lane: the step's (VS = 0), or the queue's last
             uint32_t m = 0, last = 0, qb = 0;
             bool has;
             if (dense) {
@@ -886,9 +888,11 @@ __device__ void decode_topk(const QArgs &a, const QSmem &s, uint32_t q, uint32_t
                     __syncthreads();
                     nc = s.lvl_cur[t];
                 }
-                // the filter pays while few members pass it: about the share of cells
-                // that reach the admission bound (any repetition's counts are alike)
-                const bool wide = a.wide && s.lvl_n[max(a.t_min, bscore)] * 4u < a.B;
+                // the filter pays while fewer than half the members pass it: about the
+                // share of cells that reach the admission bound (any repetition's counts
+                // are alike). 1,528 queries of 568,482 URL sets in 17 tables, whose
+                // scores mostly tie: 378 us, 500 with the line at a quarter
+                const bool wide = a.wide && s.lvl_n[max(a.t_min, bscore)] * 2u < a.B;
                 for (uint32_t c0 = 0; c0 < nc; c0 += kCh) {
                     constexpr uint32_t kPer = kCh / NT;
                     uint32_t ms[kPer], units[kPer], mine = 0;
