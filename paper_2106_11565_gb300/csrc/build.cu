@@ -517,33 +517,35 @@ __global__ void k_heavy_collect(const uint32_t *__restrict__ off, uint64_t nslot
     }
 }
 
-// Warp per heavy slot: its cell bitmap, collected in shared memory (the list's
-// cells are random words of the row) and written as one coalesced row.
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+// CTA per heavy slot: its cell bitmap, collected in shared memory (the list's
+// cells are random words of the row) and written as one coalesced row. A warp
+// per slot left the chip to the longest lists (tens of thousands of cells).
+constexpr int kFillThreads = 128;
+
+__global__ void __launch_bounds__(kFillThreads)
 k_heavy_fill(const uint32_t *__restrict__ off, const uint16_t *__restrict__ cells,
              const uint32_t *__restrict__ list, uint32_t nh, uint32_t BRw, uint32_t *__restrict__ hbm)
 {
-    extern __shared__ uint32_t bm_all[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t *bm = bm_all + warp * BRw;
-    constexpr uint32_t kU = 4;                       // cells in flight per lane
-    for (uint32_t i = blockIdx.x * kWarpsPerBlock + warp; i < nh; i += gridDim.x * kWarpsPerBlock) {
+    extern __shared__ uint32_t bm[];                 // BRw
+    constexpr uint32_t kU = 4;                       // cells in flight per thread
+    for (uint32_t i = blockIdx.x; i < nh; i += gridDim.x) {
         const uint32_t s = list[i];
-        for (uint32_t w = lane; w < BRw; w += 32) bm[w] = 0u;
+        for (uint32_t w = threadIdx.x; w < BRw; w += kFillThreads) bm[w] = 0u;
         const uint32_t beg = off[s], end = off[s + 1];
-        __syncwarp();
-        for (uint32_t t = beg + lane; t < end; t += 32 * kU) {
+        __syncthreads();
+        for (uint32_t t = beg + threadIdx.x; t < end; t += kFillThreads * kU) {
             uint32_t c[kU];
 #pragma unroll
-            for (uint32_t u = 0; u < kU; ++u) c[u] = t + 32 * u < end ? uint32_t(cells[t + 32 * u]) : 0u;
+            for (uint32_t u = 0; u < kU; ++u)
+                c[u] = t + kFillThreads * u < end ? uint32_t(cells[t + kFillThreads * u]) : 0u;
 #pragma unroll
             for (uint32_t u = 0; u < kU; ++u)
-                if (t + 32 * u < end) atomicOr(&bm[c[u] >> 5], 1u << (c[u] & 31));
+                if (t + kFillThreads * u < end) atomicOr(&bm[c[u] >> 5], 1u << (c[u] & 31));
         }
-        __syncwarp();
+        __syncthreads();
         uint32_t *row = hbm + uint64_t(i) * BRw;
-        for (uint32_t w = lane; w < BRw; w += 32) row[w] = bm[w];
-        __syncwarp();
+        for (uint32_t w = threadIdx.x; w < BRw; w += kFillThreads) row[w] = bm[w];
+        __syncthreads();
     }
 }
 
@@ -590,9 +592,8 @@ int heavy_bitmaps(flinng_index *ix, const uint32_t *list, const uint32_t *count)
     if (nh > 0 && (!ix->hbm || ix->hbm_words < words))
         return set_error(FLINNG_ERR_OOM, "internal: no storage for %u cell bitmaps", nh);
     if (nh > 0) {
-        const size_t smem = size_t(kWarpsPerBlock) * ix->BRw * sizeof(uint32_t);
-        FL_TRY(ensure_dyn_smem((const void *)k_heavy_fill, smem));
-        k_heavy_fill<<<warp_blocks(nh), kWarpsPerBlock * 32, smem, st>>>(ix->off, ix->cells, list, nh, ix->BRw, ix->hbm);
+        k_heavy_fill<<<std::min(nh, 152u * 16u), kFillThreads, ix->BRw * sizeof(uint32_t), st>>>(
+            ix->off, ix->cells, list, nh, ix->BRw, ix->hbm);
         count_launch();
         FL_CUDA(cudaGetLastError());
     }

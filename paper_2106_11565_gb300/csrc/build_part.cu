@@ -19,20 +19,23 @@
 //     written compactly to the build scratch, their offsets within the
 //     partition to the offset array and the partition's total.
 //  4. Partitions too large for shared memory (a bucket that many points
-//     share): k_big_group groups the partition's points by bucket in global
-//     memory, k_big_lists (a warp per list) and k_big_hot (a CTA per list of
-//     more than kHotPoints points) build each list through a bitmap over the
-//     B*R cells, k_big_scan makes their offsets.
+//     share): k_big_count, k_big_starts and k_big_scatter group the partition's
+//     points by bucket in global memory, kBigChunk entries a CTA; k_big_lists (a
+//     warp per list), k_big_hot (a CTA per list of more than kHotPoints points)
+//     and k_big_wide (kBigChunk points a CTA, then k_big_wide_list) build each
+//     list through a bitmap over the B*R cells, k_big_scan makes their offsets.
+//     Chunks, because a single CTA on the half million points of one bucket is
+//     what the others would wait for.
 //  5. A scan of the partitions' totals, and k_part_finish: final offsets, the
 //     heavy slots' list and bitmap rows, and the lists moved to their place.
 //
 // Bound by the passes over the entries and slots (about 12 bytes per entry and
 // list cell, 8 per slot) and by the lists' sorts in shared memory. Measured,
 // general path -> this one, whole build with hashing: recall-target genomic
-// index (100,000 reads, 512 tables, 67 M slots, 154 M cells) 5.08 -> 2.11 ms, of
-// which k_part_fine 0.94, k_part_finish 0.39, k_doph 0.22; URL index (10^6 sets,
-// 64 tables, 136 M cells, buckets of up to 10^5 points) 28.2 -> 4.7 ms, where the
-// general path's warp per slot walked the hot buckets alone.
+// index (100,000 reads, 512 tables, 67 M slots, 154 M cells) 5.08 -> 1.88 ms, of
+// which k_part_fine 0.87, k_part_finish 0.24, k_doph 0.20; URL index (10^6 sets,
+// 64 tables, 136 M cells, buckets of up to half the points) 28.2 -> 3.3 ms, where
+// the general path's warp per slot walked the hot buckets alone.
 #include <algorithm>
 
 #include "internal.cuh"
@@ -50,6 +53,7 @@ constexpr uint32_t kMaxLow = 12;           // bucket bits within a partition
 constexpr uint32_t kThreadList = 16;       // cells a single thread sorts
 constexpr uint32_t kWarpList = 128;        // cells a warp sorts
 constexpr uint32_t kHotPoints = 512;       // points of a list that one warp still handles
+constexpr uint32_t kBigChunk = 8192;       // entries of a big partition, points of a wide list per CTA
 
 // Exclusive prefix of v over the CTA of NT threads; total in *total.
 template <int NT>
@@ -230,32 +234,32 @@ __device__ __forceinline__ uint32_t thread_sort_unique(uint16_t *list, uint32_t 
     return m;
 }
 
-// Exclusive prefix over the CTA of nb values given by get(b), handed to put(b,
-// prefix): four consecutive values per thread and round, so that shared-memory
-// accesses stay spread. Returns the total. Contains __syncthreads; nb is a power
-// of two. get(b) is read before any put.
+// Exclusive prefix over the CTA of nb values, four consecutive ones per thread
+// and round: get(b, v) reads values b .. b + 3 (nb of them or fewer), put(b, pre,
+// v) receives their prefixes. With nb a power of two of at least four both move
+// all four at once. Returns the total. Contains __syncthreads; a round is read
+// before it is written.
 template <class Get, class Put>
 __device__ uint32_t scan_buckets(uint32_t nb, uint32_t *wsum, Get get, Put put)
 {
     uint32_t base = 0;
     for (uint32_t b0 = 0; b0 < nb; b0 += 4 * kT) {
         const uint32_t b = b0 + threadIdx.x * 4;
-        uint32_t v[4], sum = 0, total;
-#pragma unroll
-        for (uint32_t j = 0; j < 4; ++j) {
-            v[j] = b + j < nb ? get(b + j) : 0u;
-            sum += v[j];
-        }
-        uint32_t run = base + excl_scan<kT>(sum, wsum, &total);
-#pragma unroll
-        for (uint32_t j = 0; j < 4; ++j) {
-            if (b + j < nb) put(b + j, run, v[j]);
-            run += v[j];
-        }
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (b < nb) v = get(b);
+        uint32_t total;
+        uint4 pre;
+        pre.x = base + excl_scan<kT>(v.x + v.y + v.z + v.w, wsum, &total);
+        pre.y = pre.x + v.x;
+        pre.z = pre.y + v.y;
+        pre.w = pre.z + v.z;
+        if (b < nb) put(b, pre, v);
         base += total;
     }
     return base;
 }
+
+__device__ __forceinline__ uint2 pack16x4(const uint4 &v) { return make_uint2(v.x | v.y << 16, v.z | v.w << 16); }
 
 // A list of len <= 32 K cells sorted by one warp in registers and
 // deduplicated in place; returns the distinct cells.
@@ -319,12 +323,16 @@ struct FineArgs {
     uint32_t *ptot;            // per partition: its list cells
     uint32_t *big;             // partitions of more than kFinePoints points
     uint32_t *nbig;
+    uint2 *chunks;             // their chunks {partition, first entry of the chunk within it}
+    uint32_t *nchunks;
 };
 
 __host__ __device__ inline size_t fine_smem(uint32_t low, uint32_t R, uint32_t BRw)
 {
     const size_t nb = size_t(1) << low;
-    return nb * 4 + size_t(BRw) * 4 + 64 + size_t(kFinePoints) * R * 4 + (nb + 2) * 2 + nb * 2 + kFinePoints * 2;
+    const size_t nb4 = nb < 4 ? 4 : nb;                // the scans move four buckets at a time
+    return nb4 * 4 + (size_t(BRw) + 3) / 4 * 16 + 64 + size_t(kFinePoints) * R * 4 + (nb4 + 4) * 2 + nb4 * 2 +
+           kFinePoints * 2;
 }
 
 // Bound by issue and shared-memory latency over the lists: per list of two or
@@ -334,18 +342,19 @@ template <int RP>
 __global__ void __launch_bounds__(kT) k_part_fine(FineArgs a)
 {
     extern __shared__ __align__(16) unsigned char raw[];
-    const uint32_t nb = 1u << a.low, tid = threadIdx.x, lane = tid & 31, R = a.R;
-    uint32_t *cnt = reinterpret_cast<uint32_t *>(raw);            // nb: cells per bucket, later list offsets
-    uint32_t *bm = cnt + nb;                                      // BRw
-    uint32_t *wsum = bm + a.BRw;                                  // 8
+    const uint32_t nb = 1u << a.low, nb4 = max(nb, 4u), tid = threadIdx.x, lane = tid & 31, R = a.R;
+    // every array below starts at a multiple of 8 bytes (cnt of 16)
+    uint32_t *cnt = reinterpret_cast<uint32_t *>(raw);            // nb4: cells per bucket, later list offsets
+    uint32_t *bm = cnt + nb4;                                     // BRw
+    uint32_t *wsum = bm + (a.BRw + 3) / 4 * 4;                    // 8
     uint32_t *nwl = wsum + 8;                                     // lists for threads, warps, the CTA; next warp list
     uint16_t *cells = reinterpret_cast<uint16_t *>(nwl + 4);      // kFinePoints R
     uint16_t *owner = cells + kFinePoints * R;                    // their buckets
-    uint16_t *start = owner + kFinePoints * R;                    // nb + 1
-    uint16_t *dlen = start + nb + 2;                              // nb: distinct cells
+    uint16_t *start = owner + kFinePoints * R;                    // nb4 + 1
+    uint16_t *dlen = start + nb4 + 4;                             // nb4: distinct cells
     // worklists of buckets with two points or more: for threads from the front
     // and for warps from the back of the first half, for the CTA in the second
-    uint16_t *wl = dlen + nb, *wc = wl + kFinePoints / 2;
+    uint16_t *wl = dlen + nb4, *wc = wl + kFinePoints / 2;
     const uint64_t p = blockIdx.x;
     const uint32_t e0 = a.pbase[p], E = a.pbase[p + 1] - e0;
     uint32_t *noff = a.noff + (p << a.low);
@@ -355,7 +364,12 @@ __global__ void __launch_bounds__(kT) k_part_fine(FineArgs a)
         return;
     }
     if (E > kFinePoints) {
-        if (tid == 0) a.big[atomicAdd(a.nbig, 1u)] = uint32_t(p);
+        for (uint32_t b = tid; b < nb; b += kT) noff[b] = 0u;      // k_big_count adds up here
+        if (tid == 0) {
+            a.big[atomicAdd(a.nbig, 1u)] = uint32_t(p);
+            uint32_t at = atomicAdd(a.nchunks, (E + kBigChunk - 1) / kBigChunk);
+            for (uint32_t t = 0; t < E; t += kBigChunk) a.chunks[at++] = make_uint2(uint32_t(p), t);
+        }
         return;
     }
     constexpr int kPer = kFinePoints / kT;
@@ -364,7 +378,7 @@ __global__ void __launch_bounds__(kT) k_part_fine(FineArgs a)
     uint16_t rk[kPer];
 #pragma unroll
     for (int i = 0; i < kPer; ++i) e[i] = tid + i * kT < E ? a.part[e0 + tid + i * kT] : 0u;
-    for (uint32_t b = tid; b < nb; b += kT) cnt[b] = 0u;
+    for (uint32_t b = tid * 4; b < nb4; b += 4 * kT) *reinterpret_cast<uint4 *>(cnt + b) = make_uint4(0u, 0u, 0u, 0u);
     if (tid < 4) nwl[tid] = 0u;
     __syncthreads();
 #pragma unroll
@@ -372,12 +386,12 @@ __global__ void __launch_bounds__(kT) k_part_fine(FineArgs a)
         if (tid + i * kT < E) rk[i] = uint16_t(atomicAdd(&cnt[e[i] >> a.idbits], R));
     __syncthreads();
     const uint32_t total = scan_buckets(
-        nb, wsum, [&](uint32_t b) { return cnt[b]; },
-        [&](uint32_t b, uint32_t pre, uint32_t v) {
-            start[b] = uint16_t(pre);
-            dlen[b] = uint16_t(v);
+        nb4, wsum, [&](uint32_t b) { return *reinterpret_cast<const uint4 *>(cnt + b); },
+        [&](uint32_t b, const uint4 &pre, const uint4 &v) {
+            *reinterpret_cast<uint2 *>(start + b) = pack16x4(pre);
+            *reinterpret_cast<uint2 *>(dlen + b) = pack16x4(v);
         });
-    if (tid == 0) start[nb] = uint16_t(total);
+    if (tid == 0) start[nb4] = uint16_t(total);           // start[nb .. nb4) are the total already
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
@@ -441,11 +455,22 @@ __global__ void __launch_bounds__(kT) k_part_fine(FineArgs a)
     __syncthreads();
     // offsets within the partition, then the lists behind one another
     const uint32_t kept = scan_buckets(
-        nb, wsum, [&](uint32_t b) { return uint32_t(dlen[b]); },
-        [&](uint32_t b, uint32_t pre, uint32_t) { cnt[b] = pre; });
+        nb4, wsum,
+        [&](uint32_t b) {
+            const uint2 v = *reinterpret_cast<const uint2 *>(dlen + b);
+            return make_uint4(v.x & 0xFFFFu, v.x >> 16, v.y & 0xFFFFu, v.y >> 16);
+        },
+        [&](uint32_t b, const uint4 &pre, const uint4 &) {
+            *reinterpret_cast<uint4 *>(cnt + b) = pre;
+            if (nb >= 4) {
+                *reinterpret_cast<uint4 *>(noff + b) = pre;
+            } else {
+                noff[0] = pre.x;
+                if (nb > 1) noff[1] = pre.y;
+            }
+        });
     if (tid == 0) a.ptot[p] = kept;
     __syncthreads();
-    for (uint32_t b = tid; b < nb; b += kT) noff[b] = cnt[b];
     uint16_t *out = a.tmp + uint64_t(e0) * R;
     for (uint32_t q = tid; q < total; q += kT) {
         const uint32_t b = owner[q], j = q - start[b];
@@ -453,66 +478,116 @@ __global__ void __launch_bounds__(kT) k_part_fine(FineArgs a)
     }
 }
 
-// A big partition's points grouped by bucket: part2, first entry (sstart) and
-// number (noff) of each slot; slots of more than kHotPoints are listed.
-__global__ void __launch_bounds__(1024) k_big_group(FineArgs a, uint32_t *__restrict__ part2,
-                                                    uint32_t *__restrict__ sstart, uint32_t *__restrict__ hot,
-                                                    uint32_t *__restrict__ nhot)
+// Points per slot of the big partitions (added up in noff), a chunk per CTA.
+__global__ void __launch_bounds__(kT) k_big_count(FineArgs a)
 {
     extern __shared__ uint32_t cur[];                 // nb
-    __shared__ uint32_t wsum[32];
-    const uint32_t nb = 1u << a.low, tid = threadIdx.x, lane = tid & 31, nbig = *a.nbig;
-    const uint32_t idmask = (1u << a.idbits) - 1u;
-    for (uint32_t i = blockIdx.x; i < nbig; i += gridDim.x) {
-        const uint64_t p = a.big[i];
-        const uint32_t e0 = a.pbase[p], E = a.pbase[p + 1] - e0;
-        const uint64_t slot0 = p << a.low;
-        for (uint32_t b = tid; b < nb; b += 1024) cur[b] = 0u;
+    const uint32_t nb = 1u << a.low, tid = threadIdx.x, nch = *a.nchunks;
+    for (uint32_t i = blockIdx.x; i < nch; i += gridDim.x) {
+        const uint2 ch = a.chunks[i];
+        const uint32_t e0 = a.pbase[ch.x] + ch.y, m = min(kBigChunk, a.pbase[ch.x + 1] - e0);
+        for (uint32_t b = tid; b < nb; b += kT) cur[b] = 0u;
         __syncthreads();
-        constexpr int kU = 4;                         // entries in flight per thread
-        for (uint32_t t0 = tid; t0 < E; t0 += 1024 * kU) {
+        constexpr int kU = 8;                         // entries in flight per thread
+        for (uint32_t t0 = tid; t0 < m; t0 += kT * kU) {
             uint32_t v[kU];
 #pragma unroll
-            for (int u = 0; u < kU; ++u) v[u] = t0 + u * 1024 < E ? a.part[e0 + t0 + u * 1024] : 0u;
+            for (int u = 0; u < kU; ++u) v[u] = t0 + u * kT < m ? a.part[e0 + t0 + u * kT] : 0u;
 #pragma unroll
             for (int u = 0; u < kU; ++u)
-                if (t0 + u * 1024 < E) atomicAdd(&cur[v[u] >> a.idbits], 1u);
+                if (t0 + u * kT < m) atomicAdd(&cur[v[u] >> a.idbits], 1u);
         }
         __syncthreads();
-        const uint32_t per = (nb + 1023) / 1024;
+        uint32_t *noff = a.noff + (uint64_t(ch.x) << a.low);
+        for (uint32_t b = tid; b < nb; b += kT)
+            if (cur[b]) atomicAdd(&noff[b], cur[b]);
+        __syncthreads();
+    }
+}
+
+struct BigLists {
+    uint32_t *sstart;          // per slot of the big partitions: its first entry in part2
+    uint32_t *scur;            // and its scatter cursor
+    uint32_t *hot;             // slots of more than kHotPoints points
+    uint2 *wide;               // of more than kBigChunk: {slot, points}
+    uint2 *wchunk;             // chunks of the wide slots {wide index, first point}
+    uint32_t *n;               // counts of hot, wide, wchunk
+};
+
+// First entry and cursor of every slot of a big partition; hot and wide slots
+// listed.
+__global__ void __launch_bounds__(kT) k_big_starts(FineArgs a, BigLists g)
+{
+    __shared__ uint32_t wsum[kT / 32];
+    const uint32_t nb = 1u << a.low, tid = threadIdx.x, nbig = *a.nbig, per = (nb + kT - 1) / kT;
+    for (uint32_t i = blockIdx.x; i < nbig; i += gridDim.x) {
+        const uint64_t p = a.big[i], slot0 = p << a.low;
         uint32_t sum = 0, total;
         for (uint32_t j = 0; j < per; ++j)
-            if (tid * per + j < nb) sum += cur[tid * per + j];
-        uint32_t run = excl_scan<1024>(sum, wsum, &total);
+            if (tid * per + j < nb) sum += a.noff[slot0 + tid * per + j];
+        uint32_t run = a.pbase[p] + excl_scan<kT>(sum, wsum, &total);
         for (uint32_t j = 0; j < per; ++j) {
             const uint32_t b = tid * per + j;
             if (b >= nb) break;
-            const uint32_t c = cur[b];
-            cur[b] = run;
-            sstart[slot0 + b] = e0 + run;
-            a.noff[slot0 + b] = c;
-            if (c > kHotPoints) hot[atomicAdd(nhot, 1u)] = uint32_t(slot0 + b);
+            const uint32_t c = a.noff[slot0 + b];
+            g.sstart[slot0 + b] = g.scur[slot0 + b] = run;
+            if (c > kBigChunk) {
+                const uint32_t w = atomicAdd(&g.n[1], 1u);
+                g.wide[w] = make_uint2(uint32_t(slot0 + b), c);
+                uint32_t at = atomicAdd(&g.n[2], (c + kBigChunk - 1) / kBigChunk);
+                for (uint32_t t = 0; t < c; t += kBigChunk) g.wchunk[at++] = make_uint2(w, t);
+            } else if (c > kHotPoints) {
+                g.hot[atomicAdd(&g.n[0], 1u)] = uint32_t(slot0 + b);
+            }
             run += c;
         }
+    }
+}
+
+// The big partitions' points grouped by bucket in part2, a chunk per CTA: its
+// run of each bucket reserved with one atomic, places within it drawn in shared
+// memory, one atomic for the lanes of a bucket.
+__global__ void __launch_bounds__(kT) k_big_scatter(FineArgs a, BigLists g, uint32_t *__restrict__ part2)
+{
+    extern __shared__ uint32_t cur[];                 // nb
+    const uint32_t nb = 1u << a.low, tid = threadIdx.x, lane = tid & 31, nch = *a.nchunks;
+    const uint32_t idmask = (1u << a.idbits) - 1u;
+    for (uint32_t i = blockIdx.x; i < nch; i += gridDim.x) {
+        const uint2 ch = a.chunks[i];
+        const uint32_t e0 = a.pbase[ch.x] + ch.y, m = min(kBigChunk, a.pbase[ch.x + 1] - e0);
+        for (uint32_t b = tid; b < nb; b += kT) cur[b] = 0u;
         __syncthreads();
-        for (uint32_t t0 = tid - lane; t0 < E; t0 += 1024 * kU) {
+        constexpr int kU = 8;
+        for (uint32_t t0 = tid; t0 < m; t0 += kT * kU) {
+            uint32_t v[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) v[u] = t0 + u * kT < m ? a.part[e0 + t0 + u * kT] : 0u;
+#pragma unroll
+            for (int u = 0; u < kU; ++u)
+                if (t0 + u * kT < m) atomicAdd(&cur[v[u] >> a.idbits], 1u);
+        }
+        __syncthreads();
+        uint32_t *scur = g.scur + (uint64_t(ch.x) << a.low);
+        for (uint32_t b = tid; b < nb; b += kT)
+            if (cur[b]) cur[b] = atomicAdd(&scur[b], cur[b]);
+        __syncthreads();
+        for (uint32_t t0 = tid - lane; t0 < m; t0 += kT * kU) {
             uint32_t v[kU];
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
-                const uint32_t t = t0 + lane + u * 1024;
-                v[u] = t < E ? a.part[e0 + t] : 0u;
+                const uint32_t t = t0 + lane + u * kT;
+                v[u] = t < m ? a.part[e0 + t] : 0u;
             }
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
-                const bool in = t0 + lane + u * 1024 < E;
+                const bool in = t0 + lane + u * kT < m;
                 const uint32_t b = in ? v[u] >> a.idbits : 0xFFFFFFFFu;
-                // lanes of one bucket take their places with one atomic
                 const uint32_t same = __match_any_sync(0xffffffffu, b);
                 const uint32_t lead = __ffs(same) - 1;
                 uint32_t at = 0;
                 if (in && lane == lead) at = atomicAdd(&cur[b], __popc(same));
                 at = __shfl_sync(0xffffffffu, at, lead) + __popc(same & ((1u << lane) - 1u));
-                if (in) part2[e0 + at] = v[u] & idmask;
+                if (in) part2[at] = v[u] & idmask;
             }
         }
         __syncthreads();
@@ -586,48 +661,107 @@ __global__ void __launch_bounds__(kT) k_big_lists(FineArgs a, const uint32_t *__
     }
 }
 
-// A CTA per hot slot.
+// The cells of points part2[s0 .. s0 + m) set in the CTA's bitmap bm.
 template <int RP>
-__global__ void __launch_bounds__(1024) k_big_hot(FineArgs a, const uint32_t *__restrict__ part2,
-                                                  const uint32_t *__restrict__ sstart,
-                                                  const uint32_t *__restrict__ hot, const uint32_t *__restrict__ nhot)
+__device__ __forceinline__ void set_cells(const FineArgs &a, const uint32_t *__restrict__ part2, uint32_t s0, uint32_t m,
+                                          uint32_t *bm)
+{
+    constexpr int kU = 4;                             // points in flight per thread
+    for (uint32_t t0 = threadIdx.x; t0 < m; t0 += kT * kU) {
+        uint32_t id[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) id[u] = t0 + u * kT < m ? part2[s0 + t0 + u * kT] : 0u;
+        uint32_t c[kU][RP];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) point_cells<RP>(a.gid, id[u], a.R, a.B, c[u]);
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            if (t0 + u * kT >= m) break;
+#pragma unroll
+            for (int r = 0; r < RP; ++r)
+                if (r < int(a.R)) atomicOr(&bm[c[u][r] >> 5], 1u << (c[u][r] & 31));
+        }
+    }
+}
+
+// The set bits of a bitmap (BRw words) as an ascending list at out, by the CTA:
+// prefixes per word (pre: BRw words of shared memory), then a warp per word, a
+// lane per bit, so that a word's cells are one coalesced store. Returns their
+// number. Contains __syncthreads.
+__device__ __forceinline__ uint32_t cta_bitmap_list(const uint32_t *bm, uint32_t BRw, uint32_t *wsum, uint32_t *pre,
+                                                    uint16_t *out)
+{
+    const uint32_t tid = threadIdx.x, lane = tid & 31, per = (BRw + kT - 1) / kT;
+    uint32_t bits = 0, len;
+    for (uint32_t j = 0; j < per; ++j)
+        if (tid * per + j < BRw) bits += __popc(bm[tid * per + j]);
+    uint32_t at = excl_scan<kT>(bits, wsum, &len);
+    for (uint32_t j = 0; j < per; ++j) {
+        const uint32_t w = tid * per + j;
+        if (w >= BRw) break;
+        pre[w] = at;
+        at += __popc(bm[w]);
+    }
+    __syncthreads();
+    for (uint32_t w = tid >> 5; w < BRw; w += kT / 32) {
+        const uint32_t x = bm[w];
+        if ((x >> lane) & 1u) out[pre[w] + __popc(x & ((1u << lane) - 1u))] = uint16_t(w * 32 + lane);
+    }
+    return len;
+}
+
+// A CTA per hot slot; eight of them per SM overlap their chains of loads and
+// barriers.
+template <int RP>
+__global__ void __launch_bounds__(kT)
+k_big_hot(FineArgs a, const uint32_t *__restrict__ part2, BigLists g)
+{
+    extern __shared__ uint32_t bm[];                  // BRw, then as many prefixes
+    __shared__ uint32_t wsum[kT / 32];
+    const uint32_t nh = g.n[0];
+    for (uint32_t i = blockIdx.x; i < nh; i += gridDim.x) {
+        const uint32_t slot = g.hot[i], s0 = g.sstart[slot];
+        for (uint32_t w = threadIdx.x; w < a.BRw; w += kT) bm[w] = 0u;
+        __syncthreads();
+        set_cells<RP>(a, part2, s0, a.noff[slot], bm);
+        __syncthreads();
+        const uint32_t len = cta_bitmap_list(bm, a.BRw, wsum, bm + a.BRw, a.tmp + uint64_t(s0) * a.R);
+        if (threadIdx.x == 0) a.noff[slot] = len;
+        __syncthreads();
+    }
+}
+
+// A chunk of a wide slot per CTA: its cells OR'ed into the slot's row of wbm
+// (zeroed).
+template <int RP>
+__global__ void __launch_bounds__(kT)
+k_big_wide(FineArgs a, const uint32_t *__restrict__ part2, BigLists g, uint32_t *__restrict__ wbm)
 {
     extern __shared__ uint32_t bm[];                  // BRw
-    __shared__ uint32_t wsum[32];
-    const uint32_t tid = threadIdx.x, R = a.R, nh = *nhot;
-    for (uint32_t i = blockIdx.x; i < nh; i += gridDim.x) {
-        const uint32_t slot = hot[i], m = a.noff[slot], s0 = sstart[slot];
-        for (uint32_t w = tid; w < a.BRw; w += 1024) bm[w] = 0u;
+    const uint32_t nch = g.n[2];
+    for (uint32_t i = blockIdx.x; i < nch; i += gridDim.x) {
+        const uint2 ch = g.wchunk[i], ws = g.wide[ch.x];
+        for (uint32_t w = threadIdx.x; w < a.BRw; w += kT) bm[w] = 0u;
         __syncthreads();
-        constexpr int kU = 4;                         // points in flight per thread
-        for (uint32_t t0 = tid; t0 < m; t0 += 1024 * kU) {
-            uint32_t id[kU];
-#pragma unroll
-            for (int u = 0; u < kU; ++u) id[u] = t0 + u * 1024 < m ? part2[s0 + t0 + u * 1024] : 0u;
-            uint32_t c[kU][RP];
-#pragma unroll
-            for (int u = 0; u < kU; ++u) point_cells<RP>(a.gid, id[u], R, a.B, c[u]);
-#pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                if (t0 + u * 1024 >= m) break;
-#pragma unroll
-                for (int r = 0; r < RP; ++r)
-                    if (r < int(R)) atomicOr(&bm[c[u][r] >> 5], 1u << (c[u][r] & 31));
-            }
-        }
+        set_cells<RP>(a, part2, g.sstart[ws.x] + ch.y, min(kBigChunk, ws.y - ch.y), bm);
         __syncthreads();
-        const uint32_t wper = (a.BRw + 1023) / 1024;
-        uint32_t bits = 0, len;
-        for (uint32_t j = 0; j < wper; ++j)
-            if (tid * wper + j < a.BRw) bits += __popc(bm[tid * wper + j]);
-        uint16_t *out = a.tmp + uint64_t(s0) * R;
-        uint32_t at = excl_scan<1024>(bits, wsum, &len);
-        for (uint32_t j = 0; j < wper; ++j) {
-            const uint32_t w = tid * wper + j;
-            if (w >= a.BRw) break;
-            for (uint32_t x = bm[w]; x; x &= x - 1) out[at++] = uint16_t(w * 32 + __ffs(x) - 1);
-        }
-        if (tid == 0) a.noff[slot] = len;
+        for (uint32_t w = threadIdx.x; w < a.BRw; w += kT)
+            if (bm[w]) atomicOr(&wbm[uint64_t(ch.x) * a.BRw + w], bm[w]);
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kT) k_big_wide_list(FineArgs a, BigLists g, const uint32_t *__restrict__ wbm)
+{
+    extern __shared__ uint32_t bm[];                  // BRw, then as many prefixes
+    __shared__ uint32_t wsum[kT / 32];
+    const uint32_t nw = g.n[1];
+    for (uint32_t i = blockIdx.x; i < nw; i += gridDim.x) {
+        const uint32_t slot = g.wide[i].x;
+        for (uint32_t w = threadIdx.x; w < a.BRw; w += kT) bm[w] = wbm[uint64_t(i) * a.BRw + w];
+        __syncthreads();
+        const uint32_t len = cta_bitmap_list(bm, a.BRw, wsum, bm + a.BRw, a.tmp + uint64_t(g.sstart[slot]) * a.R);
+        if (threadIdx.x == 0) a.noff[slot] = len;
         __syncthreads();
     }
 }
@@ -656,8 +790,46 @@ __global__ void __launch_bounds__(kT) k_big_scan(FineArgs a)
     }
 }
 
+// n cells from src to dst (anywhere, not overlapping) by lanes t of nt: 16-byte
+// stores at dst's alignment, each from two aligned 16-byte loads of src shifted
+// by their distance. Reads up to 15 bytes past src's end (kCellPad).
+template <int Q>
+__device__ __forceinline__ uint4 shifted(const uint4 &x, const uint4 &y, bool half)
+{
+    const uint32_t w[9] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w, 0u};
+    uint4 o;
+    o.x = half ? __funnelshift_r(w[Q], w[Q + 1], 16) : w[Q];
+    o.y = half ? __funnelshift_r(w[Q + 1], w[Q + 2], 16) : w[Q + 1];
+    o.z = half ? __funnelshift_r(w[Q + 2], w[Q + 3], 16) : w[Q + 2];
+    o.w = half ? __funnelshift_r(w[Q + 3], w[Q + 4], 16) : w[Q + 3];
+    return o;
+}
+
+__device__ __forceinline__ void copy_cells(uint16_t *__restrict__ dst, const uint16_t *__restrict__ src, uint32_t n,
+                                           uint32_t t, uint32_t nt)
+{
+    const uint32_t head = min(n, uint32_t((16u - (reinterpret_cast<uintptr_t>(dst) & 15u)) & 15u) / 2);
+    const uint32_t body = (n - head) / 8, tail = head + body * 8;
+    if (t < head) dst[t] = src[t];
+    if (tail + t < n && t < 8) dst[tail + t] = src[tail + t];
+    const uint32_t by = uint32_t(reinterpret_cast<uintptr_t>(src + head) & 15u);
+    const uint4 *s4 = reinterpret_cast<const uint4 *>(reinterpret_cast<uintptr_t>(src + head) - by);
+    uint4 *d4 = reinterpret_cast<uint4 *>(dst + head);
+    const bool half = (by & 2u) != 0u;
+    for (uint32_t i = t; i < body; i += nt) {
+        const uint4 x = s4[i], y = by ? s4[i + 1] : x;
+        switch (by >> 2) {                       // uniform over the copy
+        case 0: d4[i] = shifted<0>(x, y, half); break;
+        case 1: d4[i] = shifted<1>(x, y, half); break;
+        case 2: d4[i] = shifted<2>(x, y, half); break;
+        default: d4[i] = shifted<3>(x, y, half); break;
+        }
+    }
+}
+
 // A CTA per partition: its slots' final offsets and bitmap rows, its lists to
-// their place.
+// their place. Bound by memory: 1.4 GB in 237 us at the recall-target index (385
+// us with 2-byte copies).
 __global__ void __launch_bounds__(kT) k_part_finish(FineArgs a, uint64_t nparts, const uint32_t *__restrict__ tbase,
                                                     const uint32_t *__restrict__ sstart, uint32_t heavy_min,
                                                     uint32_t *__restrict__ hidx, uint32_t *__restrict__ list,
@@ -713,15 +885,13 @@ __global__ void __launch_bounds__(kT) k_part_finish(FineArgs a, uint64_t nparts,
     }
     if (p + 1 == nparts && tid == 0) noff[nb] = base + total;
     if (E <= kFinePoints) {
-        const uint16_t *src = a.tmp + uint64_t(e0) * a.R;
-        for (uint32_t i = tid; i < total; i += kT) cells[base + i] = src[i];
+        copy_cells(cells + base, a.tmp + uint64_t(e0) * a.R, total, tid, kT);
     } else {
         __syncthreads();                    // the final offsets, read back by the warps
         for (uint32_t b = warp; b < nb; b += kT / 32) {
             const uint32_t o0 = noff[b], o1 = b + 1 < nb ? noff[b + 1] : base + total;
             if (o0 == o1) continue;
-            const uint16_t *src = a.tmp + uint64_t(sstart[slot0 + b]) * a.R;
-            for (uint32_t i = lane; i < o1 - o0; i += 32) cells[o0 + i] = src[i];
+            copy_cells(cells + o0, a.tmp + uint64_t(sstart[slot0 + b]) * a.R, o1 - o0, lane, 32);
         }
     }
 }
@@ -791,9 +961,10 @@ size_t part_workspace_bytes(const flinng_index *ix, uint64_t n)
 {
     PartPlan pl;
     if (!plan_for(ix, n, &pl)) return 0;
-    const uint64_t entries = n * ix->cfg.L;
-    return 4 * carve_bytes<uint32_t>(pl.parts + 1) + carve_bytes<uint32_t>(entries / kHotPoints + 1) +
-           carve_bytes<uint32_t>(entries * ix->cfg.R / ix->heavy_min + 2) + carve_bytes<uint32_t>(4) +
+    const uint64_t entries = n * ix->cfg.L, ch = 2 * (entries / kFinePoints) + 1, wide = entries / kBigChunk + 1;
+    return 4 * carve_bytes<uint32_t>(pl.parts + 1) + carve_bytes<uint2>(ch) + carve_bytes<uint32_t>(entries / kHotPoints + 1) +
+           3 * carve_bytes<uint2>(wide) + carve_bytes<uint32_t>(wide * ix->BRw) +
+           carve_bytes<uint32_t>(entries * ix->cfg.R / ix->heavy_min + 2) + carve_bytes<uint32_t>(8) +
            carve_bytes<char>(scan_workspace_bytes(pl.parts + 1));
 }
 
@@ -812,15 +983,24 @@ int part_build(flinng_index *ix, uint32_t *buckets, uint64_t n, void *ws, uint32
     uint32_t *pcur = c.take<uint32_t>(pl.parts + 1);       // counts, cursors, then the partitions' totals
     uint32_t *tbase = c.take<uint32_t>(pl.parts + 1);
     uint32_t *big = c.take<uint32_t>(pl.parts + 1);
-    uint32_t *hot = c.take<uint32_t>(entries / kHotPoints + 1);
+    // a big partition of E > kFinePoints entries has at most 2 E / kFinePoints
+    // chunks, a wide slot of c > kBigChunk points at most 2 c / kBigChunk
+    const uint64_t nch = 2 * (entries / kFinePoints) + 1, nwide = entries / kBigChunk + 1;
+    uint2 *chunks = c.take<uint2>(nch);
+    BigLists g{};
+    g.hot = c.take<uint32_t>(entries / kHotPoints + 1);
+    g.wide = c.take<uint2>(nwide);
+    g.wchunk = c.take<uint2>(2 * nwide);
+    uint32_t *wbm = c.take<uint32_t>(nwide * ix->BRw);
     uint32_t *list = c.take<uint32_t>(entries * R / ix->heavy_min + 2);
-    uint32_t *cnt = c.take<uint32_t>(4);                   // big partitions, hot slots, heavy slots
+    uint32_t *cnt = c.take<uint32_t>(8);                   // big partitions, chunks, heavy slots; hot, wide slots, their chunks
     void *scan_ws = c.take<char>(scan_workspace_bytes(pl.parts + 1));
     // L x n buckets, later the big partitions' points by bucket, in the list
     // array (2 R bytes per entry), which receives the lists only at the end
     uint32_t *bt = reinterpret_cast<uint32_t *>(ix->cells);
     uint32_t *part = buckets;
-    FL_CUDA(cudaMemsetAsync(cnt, 0, 4 * sizeof(uint32_t), st));
+    FL_CUDA(cudaMemsetAsync(cnt, 0, 8 * sizeof(uint32_t), st));
+    FL_CUDA(cudaMemsetAsync(wbm, 0, nwide * ix->BRw * sizeof(uint32_t), st));
     FL_TRY(partition_entries(ix, buckets, n, pl.C, pl.idbits, bt, part, pbase, pcur, scan_ws));
     FineArgs a{};
     a.part = part;
@@ -836,7 +1016,12 @@ int part_build(flinng_index *ix, uint32_t *buckets, uint64_t n, void *ws, uint32
     a.ptot = pcur;
     a.big = big;
     a.nbig = cnt;
-    uint32_t *part2 = bt, *sstart = ix->slot_a;
+    a.chunks = chunks;
+    a.nchunks = cnt + 1;
+    uint32_t *part2 = bt;
+    g.sstart = ix->slot_a;
+    g.scur = ix->hidx;          // rewritten as a whole at the end
+    g.n = cnt + 4;
     const size_t fsm = fine_smem(pl.low, R, ix->BRw), gsm = sizeof(uint32_t) << pl.low;
     const size_t lsm = size_t(kT / 32) * ix->BRw * 4, hsm = size_t(ix->BRw) * 4;
 #define FL_RP(call) \
@@ -850,20 +1035,30 @@ int part_build(flinng_index *ix, uint32_t *buckets, uint64_t n, void *ws, uint32
     FL_TRY(ensure_dyn_smem(ix->rp == 2 ? (const void *)k_part_fine<2> : ix->rp == 4 ? (const void *)k_part_fine<4>
                                                                                      : (const void *)k_part_fine<8>, fsm));
     FL_RP((k_part_fine<RP><<<(unsigned)pl.parts, kT, fsm, st>>>(a)));
-    k_big_group<<<152 * 2, 1024, gsm, st>>>(a, part2, sstart, hot, cnt + 1);
+    k_big_count<<<152 * 8, kT, gsm, st>>>(a);
+    count_launch();
+    FL_CUDA(cudaGetLastError());
+    k_big_starts<<<152 * 8, kT, 0, st>>>(a, g);
+    count_launch();
+    FL_CUDA(cudaGetLastError());
+    k_big_scatter<<<152 * 8, kT, gsm, st>>>(a, g, part2);
     count_launch();
     FL_CUDA(cudaGetLastError());
     FL_TRY(ensure_dyn_smem(ix->rp == 2 ? (const void *)k_big_lists<2> : ix->rp == 4 ? (const void *)k_big_lists<4>
                                                                                      : (const void *)k_big_lists<8>, lsm));
     // k_big_lists first: it tells the hot slots by their number of points, which
-    // k_big_hot replaces with the length of the list
-    FL_RP((k_big_lists<RP><<<152 * 8, kT, lsm, st>>>(a, part2, sstart)));
-    FL_RP((k_big_hot<RP><<<152 * 2, 1024, hsm, st>>>(a, part2, sstart, hot, cnt + 1)));
+    // the others replace with the length of the list
+    FL_RP((k_big_lists<RP><<<152 * 8, kT, lsm, st>>>(a, part2, g.sstart)));
+    FL_RP((k_big_hot<RP><<<152 * 8, kT, 2 * hsm, st>>>(a, part2, g)));
+    FL_RP((k_big_wide<RP><<<152 * 8, kT, hsm, st>>>(a, part2, g, wbm)));
+    k_big_wide_list<<<152 * 8, kT, 2 * hsm, st>>>(a, g, wbm);
+    count_launch();
+    FL_CUDA(cudaGetLastError());
     k_big_scan<<<152 * 8, kT, 0, st>>>(a);
     count_launch();
     FL_CUDA(cudaGetLastError());
     FL_TRY(scan_exclusive(pcur, tbase, pl.parts, scan_ws, st));
-    k_part_finish<<<(unsigned)pl.parts, kT, 0, st>>>(a, pl.parts, tbase, sstart, ix->heavy_min, ix->hidx, list, cnt + 2,
+    k_part_finish<<<(unsigned)pl.parts, kT, 0, st>>>(a, pl.parts, tbase, g.sstart, ix->heavy_min, ix->hidx, list, cnt + 2,
                                                      ix->cells);
     count_launch();
     FL_CUDA(cudaGetLastError());

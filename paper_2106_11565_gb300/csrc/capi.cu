@@ -441,7 +441,10 @@ int flinng_create(const flinng_config *cfg, const flinng_params *params, void *s
         ALLOC(srp_w, size_t(ix->P) * cfg->dim + ix->P);     // then the rows' norms
         if (rc == FLINNG_OK) ix->w_norm = ix->srp_w + size_t(ix->P) * cfg->dim;
     } else {
-        ALLOC(bucket_a, size_t(ix->P));
+        // then each bin's first densification draws (16-byte aligned: P rows of 16 bytes after P of 8)
+        const size_t words = (size_t(ix->P) + 1) & ~size_t(1);
+        ALLOC(bucket_a, words + size_t(ix->P) * kDophTable * sizeof(uint16_t) / sizeof(uint64_t));
+        if (rc == FLINNG_OK) ix->doph_draw = reinterpret_cast<uint16_t *>(ix->bucket_a + words);
         ALLOC(bucket_c, size_t(L));
     }
     ALLOC(gid, size_t(cfg->capacity) * ix->rp);
@@ -502,6 +505,7 @@ int flinng_create(const flinng_config *cfg, const flinng_params *params, void *s
         chk(cudaEventCreateWithFlags(&ix->ev_join, cudaEventDisableTiming), "create event");
         if (rc == FLINNG_OK && cfg->metric == FLINNG_COSINE_SRP)
             rc = cfg->precision != FLINNG_PREC_FP32 ? srp_tc_prepare_weights(ix) : srp_weight_norms(ix);
+        if (rc == FLINNG_OK && cfg->metric == FLINNG_JACCARD_DOPH) rc = doph_draws(ix);
         chk(cudaStreamSynchronize(st), "create sync");
     }
     if (rc != FLINNG_OK) {

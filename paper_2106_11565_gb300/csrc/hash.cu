@@ -17,6 +17,7 @@
 #include <cmath>
 
 #include "internal.cuh"
+#include "doph.cuh"
 #include "srp_rows.cuh"
 
 namespace flinng {
@@ -404,12 +405,11 @@ __global__ void k_add_counter(unsigned long long *dst, const unsigned long long 
 constexpr int kDophWarps = 8;
 constexpr int kDophUnroll = 4;     // element loads in flight per lane
 
-__device__ __forceinline__ uint64_t splitmix64(uint64_t z)
+// The table of each bin's first densification draws.
+__global__ void k_doph_draws(uint32_t nb, uint64_t seed, uint16_t *__restrict__ draw)
 {
-    z += 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < nb * kDophTable) draw[t] = uint16_t(doph_draw_of(t / kDophTable, t % kDophTable + 1, nb, seed));
 }
 
 // 32-bit words of shared memory per set: bin minima, occupancy, empty bins
@@ -419,8 +419,8 @@ __global__ void __launch_bounds__(kDophWarps * 32)
 k_doph(const uint64_t *__restrict__ off, const uint32_t *__restrict__ elems,
        uint64_t n, uint32_t nb, uint32_t a, uint32_t b, uint64_t seed, uint32_t L,
        uint32_t K, uint32_t W, const uint64_t *__restrict__ ba,
-       const uint64_t *__restrict__ bc, uint32_t *__restrict__ buckets,
-       uint32_t *__restrict__ values)
+       const uint64_t *__restrict__ bc, const uint16_t *__restrict__ draw,
+       uint32_t *__restrict__ buckets, uint32_t *__restrict__ values)
 {
     extern __shared__ uint32_t sm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -465,36 +465,18 @@ k_doph(const uint64_t *__restrict__ off, const uint32_t *__restrict__ elems,
             if (lane == 0) occ[k0 >> 5] = bits;
             // the empty bins listed: a third to a seventh of them, so a loop over
             // the list keeps the lanes busy where one over all bins left most
-            // idle through the other lanes' draws (100,000 genomic reads, 512
-            // bins: 300 -> 221 us; 10^6 URL sets, 64 bins: 801 -> 710 us)
+            // idle through the other lanes' draws (with doph_source's table,
+            // 100,000 genomic reads, 512 bins: 300 -> 200 us; 10^6 URL sets, 64
+            // bins: 801 -> 461 us)
             const uint32_t none = ~bits & (nb - k0 >= 32 ? 0xffffffffu : (1u << (nb - k0)) - 1u);
             if ((none >> lane) & 1u) empty[ne + __popc(none & ((1u << lane) - 1u))] = uint16_t(k);
             ne += __popc(none);
         }
         __syncwarp();
         if (end > beg) {
-            const bool pow2 = (nb & (nb - 1u)) == 0u;     // z mod nb is a mask then
             for (uint32_t i = lane; i < ne; i += 32) {
                 const uint32_t k = empty[i];
-                bool found = false;
-                for (uint32_t att = 1; att <= kDophMaxAttempts; ++att) {
-                    const uint64_t z = splitmix64(seed ^ ((uint64_t(k) << 32) | att));
-                    const uint32_t j = pow2 ? uint32_t(z) & (nb - 1u) : uint32_t(z % nb);
-                    if ((occ[j >> 5] >> (j & 31)) & 1u) {
-                        val[k] = val[j];
-                        found = true;
-                        break;
-                    }
-                }
-                if (!found) {
-                    for (uint32_t s = 1; s <= nb; ++s) {
-                        const uint32_t j = (k + s) % nb;
-                        if ((occ[j >> 5] >> (j & 31)) & 1u) {
-                            val[k] = val[j];
-                            break;
-                        }
-                    }
-                }
+                val[k] = val[doph_source(k, nb, seed, draw, occ)];
             }
         }
         __syncwarp();
@@ -614,6 +596,15 @@ int srp_hash(flinng_index *ix, const float *x, uint64_t ld, uint64_t n,
     return FLINNG_OK;
 }
 
+int doph_draws(flinng_index *ix)
+{
+    const uint32_t nb = ix->P;
+    k_doph_draws<<<(nb * kDophTable + 255) / 256, 256, 0, ix->stream>>>(nb, ix->doph_seed, ix->doph_draw);
+    count_launch();
+    FL_CUDA(cudaGetLastError());
+    return FLINNG_OK;
+}
+
 int doph_hash(flinng_index *ix, const uint64_t *off, const uint32_t *elems,
               uint64_t n, uint32_t *buckets, uint32_t *values)
 {
@@ -625,7 +616,7 @@ int doph_hash(flinng_index *ix, const uint64_t *off, const uint32_t *elems,
     if (blocks > 152ull * 64) blocks = 152ull * 64;
     k_doph<<<(unsigned)blocks, kDophWarps * 32, smem, ix->stream>>>(
         off, elems, n, nb, ix->doph_a, ix->doph_b, ix->doph_seed, ix->cfg.L, ix->cfg.K,
-        ix->cfg.range_bits, ix->bucket_a, ix->bucket_c, buckets, values);
+        ix->cfg.range_bits, ix->bucket_a, ix->bucket_c, ix->doph_draw, buckets, values);
     count_launch();
     FL_CUDA(cudaGetLastError());
     return FLINNG_OK;

@@ -14,6 +14,7 @@ constexpr uint64_t kKeyNone = ~0ull;
 constexpr uint32_t kMaxKMax = 1024;
 constexpr uint32_t kMaxL = 4095;          // 12-bit scores in the query keys
 constexpr uint32_t kDophMaxAttempts = 4096;
+constexpr uint32_t kDophTable = 8;        // densification draws per bin laid out at create time
 // hash counters: [0] undecided after the first pass, [1] exact accumulator,
 // [2] fp64 re-checks, [3] compensated fp32 re-checks, [4] first-pass signs
 // that a re-check reversed (flips)
@@ -110,6 +111,7 @@ struct flinng_index {
     uint64_t *bucket_c;    // L
     uint32_t doph_a, doph_b;
     uint64_t doph_seed;
+    uint16_t *doph_draw;      // P x kDophTable: bin k's first draws (they depend on the seed and k alone)
     float srp_margin_gamma;   // 2 * gamma_d in fp32, rounded up
     double srp_gamma64;       // 2 * gamma_d for the fp64 recheck
     void *w_split;            // tensor-core precision: bf16 w1 then w2, P x dim each
@@ -189,6 +191,8 @@ int scan_exclusive(const uint32_t *in, uint32_t *out, size_t n, void *ws,
 size_t srp_workspace_bytes(const flinng_index *ix, uint64_t n);
 int srp_hash(flinng_index *ix, const float *x, uint64_t ld, uint64_t n,
              uint32_t *buckets, float *proj, void *ws, size_t ws_bytes);
+// Fills doph_draw.
+int doph_draws(flinng_index *ix);
 // DOPH + bucket combine: buckets n x L; values (optional) n x P.
 int doph_hash(flinng_index *ix, const uint64_t *off, const uint32_t *elems,
               uint64_t n, uint32_t *buckets, uint32_t *values);

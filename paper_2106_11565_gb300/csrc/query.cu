@@ -174,6 +174,7 @@ static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t 
         h.seed = ix->doph_seed;
         h.ba = ix->bucket_a;
         h.bc = ix->bucket_c;
+        h.draw = ix->doph_draw;
         hash_bytes += size_t(h.nb + (h.nb + 31) / 32) * 4;
     }
     hash_bytes = (hash_bytes + 15) & ~size_t(15);

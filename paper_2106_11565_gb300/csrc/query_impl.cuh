@@ -34,6 +34,7 @@
 // The kernels are templates on the count width; query.cu instantiates CW = 1
 // and query_c16.cu CW = 2, each in its own translation unit.
 #pragma once
+#include "doph.cuh"
 #include "internal.cuh"
 
 namespace flinng {
@@ -1065,6 +1066,7 @@ struct HArgs {
     uint64_t seed;
     const uint64_t *ba;
     const uint64_t *bc;
+    const uint16_t *draw;     // densification draws
     // cosine
     const float *x;
     uint64_t ldx;
@@ -1078,14 +1080,6 @@ struct HArgs {
     size_t hash_off;    // byte offset of the hash region in shared memory (0: inside the
                         // candidate buffer, which is free until the decode)
 };
-
-__device__ __forceinline__ uint64_t splitmix64_q(uint64_t z)
-{
-    z += 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
 
 // DOPH of query q into qb[0..L) (shared memory). Contains __syncthreads.
 template <int NT>
@@ -1106,29 +1100,8 @@ __device__ void cta_doph(const QArgs &a, const HArgs &h, uint32_t q, uint32_t *q
     }
     __syncthreads();
     if (end > beg) {
-        const bool pow2 = (nb & (nb - 1u)) == 0u;     // z mod nb is a mask then
-        for (uint32_t k = tid; k < nb; k += NT) {
-            if ((occ[k >> 5] >> (k & 31)) & 1u) continue;
-            bool found = false;
-            for (uint32_t att = 1; att <= kDophMaxAttempts; ++att) {
-                const uint64_t z = splitmix64_q(h.seed ^ ((uint64_t(k) << 32) | att));
-                const uint32_t j = pow2 ? uint32_t(z) & (nb - 1u) : uint32_t(z % nb);
-                if ((occ[j >> 5] >> (j & 31)) & 1u) {
-                    val[k] = val[j];
-                    found = true;
-                    break;
-                }
-            }
-            if (!found) {
-                for (uint32_t s2 = 1; s2 <= nb; ++s2) {
-                    const uint32_t j = (k + s2) % nb;
-                    if ((occ[j >> 5] >> (j & 31)) & 1u) {
-                        val[k] = val[j];
-                        break;
-                    }
-                }
-            }
-        }
+        for (uint32_t k = tid; k < nb; k += NT)
+            if (!((occ[k >> 5] >> (k & 31)) & 1u)) val[k] = val[doph_source(k, nb, h.seed, h.draw, occ)];
     }
     __syncthreads();
     for (uint32_t l = tid; l < a.L; l += NT) {
