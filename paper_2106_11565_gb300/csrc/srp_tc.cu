@@ -216,6 +216,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t r[32])
         : "r"(taddr));
 }
 
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t r[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+}
+
 __device__ __forceinline__ void tmem_wait_ld()
 {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -231,6 +241,7 @@ struct TcArgs {
     const float *xscale;   // FP8: n row scales s_x (powers of two)
     const float *wscale;   // FP8: P row scales s_w
     float c_norm;          // margin factor on ||x|| ||w||
+    float c_one;           // MASK = 3: that of the first pass
     float c_sub;           // margin factor on ||x|| + ||w|| (subnormal flushes)
     float tiny;            // absolute margin (underflow)
     uint32_t *codes;       // n x L (zeroed)
@@ -251,9 +262,12 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 }
 
 // MASK: 0 undecided projections are listed; 1 they are marked in a.mask (the
-// first pass of a single-term form whose undecided share is large); 2 only the
-// marked ones are decided (its second pass, on the two-term split), the rest
-// listed.
+// first pass of the FP8 form whose undecided share is large); 2 only the marked
+// ones are decided (its second pass, on the two-term split), the rest listed; 3
+// both passes of the BF16 form at once, whose first pass is the split's x1 w1
+// half: the sums of that half are kept beside the full ones (128 accumulators a
+// thread, which the 320 threads' registers hold), so the second pass costs the
+// split's two extra MMAs per step and no second reading of the operands.
 template <int FORM, int MASK>
 __global__ void __launch_bounds__(kTcThreads, 1)
 k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtensorMap mx2,
@@ -372,8 +386,11 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
         const uint32_t half = uint32_t(warp - 2) >> 2;
         const uint32_t tbase = tmem + (quarter << 16) + 64u * half;
         float acc[64];
+        float one[MASK == 3 ? 64 : 1];       // the first pass's sums
 #pragma unroll
         for (int j = 0; j < 64; ++j) acc[j] = 0.f;
+#pragma unroll
+        for (int j = 0; j < (MASK == 3 ? 64 : 1); ++j) one[j] = 0.f;
         bool abort = false;
         for (uint32_t kb = 0; kb < nkb; ++kb) {
             const uint32_t b = kb & 1u;
@@ -386,7 +403,26 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if constexpr (FORM == kFormBf16x2) {
+            if constexpr (MASK == 3) {
+                // four quarters: 128 accumulators leave room for 32 values in flight
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    uint32_t hv[16], lv[16];
+                    tmem_ld16(tbase + kBuf * b + 16 * q, hv);
+                    tmem_ld16(tbase + kBuf * b + kTN + 16 * q, lv);
+                    tmem_wait_ld();
+                    if (q == 3) {
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&tempty[b]);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        acc[16 * q + j] += __uint_as_float(hv[j]) + __uint_as_float(lv[j]);
+                        one[16 * q + j] += __uint_as_float(hv[j]);
+                    }
+                }
+            } else if constexpr (FORM == kFormBf16x2) {
                 // two halves of 32 columns: hi and lo loads in flight together, one
                 // wait each; the buffer goes back to the MMA issuer before the
                 // second half is added
@@ -425,13 +461,13 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
         if (!abort && row < a.n) {
             const float xn = a.xnorm[row];
             float xr = 0.f, xs = 1.f;
-            if constexpr (FORM != kFormBf16x2) xr = a.xres[row];
+            if constexpr (FORM != kFormBf16x2 || MASK == 3) xr = a.xres[row];
             if constexpr (FORM == kFormFp8) xs = a.xscale[row];
             uint32_t cur_l = 0xFFFFFFFFu, cur_bits = 0u;
             // this thread's two words of the masks: undecided, first-pass signs
             const uint32_t pw = (a.P + 31) / 32, w0 = (col0 + 64u * half) / 32;
-            uint32_t und[2] = {0u, 0u}, sgn[2] = {0u, 0u}, decided = 0u, flips = 0u;
-            uint32_t *mrow = MASK ? a.mask + row * (2 * pw) + w0 : nullptr;
+            uint32_t und[2] = {0u, 0u}, sgn[2] = {0u, 0u}, decided = 0u, flips = 0u, open = 0u;
+            uint32_t *mrow = MASK == 1 || MASK == 2 ? a.mask + row * (2 * pw) + w0 : nullptr;
             if constexpr (MASK == 2) {
 #pragma unroll
                 for (int i = 0; i < 2; ++i)
@@ -448,23 +484,35 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
                 float p = acc[j];
                 if constexpr (FORM == kFormFp8) p *= xs * a.wscale[col];    // powers of two: exact
                 const float wn = a.wnorm[col];
-                if (a.proj) a.proj[row * a.P + col] = p;
+                if (a.proj) a.proj[row * a.P + col] = MASK == 3 ? one[MASK == 3 ? j : 0] : p;
+                // residual term (Cauchy-Schwarz on the quantisation errors) plus
+                // accumulation on the quantised operands' norms, then slack
+                auto single_margin = [&](float v, float c) {
+                    const float wr = a.wres[col];
+                    const float resid = fmaf(xn, wr, fmaf(xr, wn, 3.f * xr * wr));
+                    const float accum = c * (xn + xr) * (wn + wr);
+                    return (resid + accum + fmaf(ldexpf(1.f, -23), fabsf(v), fmaf(a.c_sub, xn + wn, a.tiny))) *
+                           (1.f + ldexpf(1.f, -20));
+                };
+                bool first_pos = p > 0.f, again = MASK == 2;       // again: this is a second look
                 float margin;
                 if constexpr (FORM == kFormBf16x2) {
                     margin = fmaf(a.c_norm * xn, wn, fmaf(ldexpf(1.f, -23), fabsf(p), fmaf(a.c_sub, xn + wn, a.tiny)));
                 } else {
-                    // residual term (Cauchy-Schwarz on the quantisation errors) plus
-                    // accumulation on the quantised operands' norms, then slack
-                    const float wr = a.wres[col];
-                    const float resid = fmaf(xn, wr, fmaf(xr, wn, 3.f * xr * wr));
-                    const float accum = a.c_norm * (xn + xr) * (wn + wr);
-                    margin = (resid + accum + fmaf(ldexpf(1.f, -23), fabsf(p), fmaf(a.c_sub, xn + wn, a.tiny))) *
-                             (1.f + ldexpf(1.f, -20));
+                    margin = single_margin(p, a.c_norm);
+                }
+                if constexpr (MASK == 2) first_pos = ((sgn[j / 32] >> (j % 32)) & 1u) != 0u;
+                if constexpr (MASK == 3) {
+                    const float v = one[j];
+                    first_pos = v > 0.f;
+                    again = !(fabsf(v) > single_margin(v, a.c_one));
+                    if (again) ++open;
+                    else p = v, margin = 0.f;                    // decided by the first pass (|v| > 0)
                 }
                 if (fabsf(p) > margin) {
-                    if constexpr (MASK == 2) {
+                    if (MASK >= 2 && again) {
                         ++decided;
-                        flips += (p > 0.f) != (((sgn[j / 32] >> (j % 32)) & 1u) != 0u) ? 1u : 0u;
+                        flips += (p > 0.f) != first_pos ? 1u : 0u;
                     }
                     if (p > 0.f) {
                         const uint32_t l = col / a.K;
@@ -480,9 +528,8 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
                     if (p > 0.f) sgn[j / 32] |= 1u << (j % 32);
                 } else {
                     // the tentative sign a later re-check may reverse is the first pass's
-                    const bool pos = MASK == 2 ? ((sgn[j / 32] >> (j % 32)) & 1u) != 0u : p > 0.f;
                     const unsigned long long slot = atomicAdd(a.rcount, 1ull);
-                    a.rlist[slot] = (pos ? kEntSign : 0ull) | ((unsigned long long)row << 20) | col;
+                    a.rlist[slot] = (first_pos ? kEntSign : 0ull) | ((unsigned long long)row << 20) | col;
                 }
             }
             if (cur_bits) atomicOr(&a.codes[row * a.L + cur_l], cur_bits);
@@ -496,7 +543,10 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
                 const uint32_t c = __popc(und[0]) + __popc(und[1]);
                 if (c) atomicAdd(a.nund, (unsigned long long)c);
             }
-            if constexpr (MASK == 2) {
+            if constexpr (MASK == 3) {
+                if (open) atomicAdd(a.nund, (unsigned long long)open);
+            }
+            if constexpr (MASK >= 2) {
                 if (decided) atomicAdd(&a.stats[3], (unsigned long long)decided);
                 if (flips) atomicAdd(&a.stats[4], (unsigned long long)flips);
             }
@@ -860,7 +910,8 @@ inline size_t qrow_bytes(uint32_t precision, uint32_t d)
 // two-term split costs 0.05 ns per projection of the batch, decided or not, so
 // it wins from an undecided share of about 2 %: d >= 128 in BF16, any d in FP8,
 // once the batch fills the chip (2^20 projections: 64 tiles of 128 x 128). 8,192
-// embeddings in BF16: 4.04 ms re-checked one by one, 0.77 ms with the second pass.
+// embeddings in BF16: 4.04 ms re-checked one by one, 0.76 ms with a second pass,
+// 0.57 ms with both passes in one kernel (MASK = 3).
 inline bool dense_second_pass(uint32_t precision, uint64_t rows, uint32_t P, uint32_t d)
 {
     if (precision != FLINNG_PREC_BF16 && precision != FLINNG_PREC_FP8) return false;
@@ -1029,16 +1080,17 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
         if (prec == FLINNG_PREC_BF16X2) FL_TRY((launch_tc<kFormBf16x2, 0>(mx1, mx2, mw1, mw2, a, rows, st)));
         else if (!dense && prec == FLINNG_PREC_BF16) FL_TRY((launch_tc<kFormBf16, 0>(mx1, mx1, mwq, mwq, a, rows, st)));
         else if (!dense) FL_TRY((launch_tc<kFormFp8, 0>(mx1, mx1, mwq, mwq, a, rows, st)));
-        else if (prec == FLINNG_PREC_BF16) FL_TRY((launch_tc<kFormBf16, 1>(mx1, mx1, mwq, mwq, a, rows, st)));
-        else FL_TRY((launch_tc<kFormFp8, 1>(mx1, mx1, mwq, mwq, a, rows, st)));
-        if (dense) {
-            // the marked projections again on the two-term split, whose margin
+        else if (prec == FLINNG_PREC_BF16) {
+            a.c_one = c_norm;
+            a.c_norm = c_two;
+            FL_TRY((launch_tc<kFormBf16x2, 3>(mx1, mx2, mw1, mw2, a, rows, st)));
+        } else {
+            // FP8: the marked projections again on the two-term split, whose margin
             // leaves a few in a thousand
-            if (bytes) {
-                FL_TRY(quant_rows(FLINNG_PREC_BF16X2, xc, ld, rows, d, xq, xn, nullptr, nullptr, true, st));
-                FL_TRY(make_map(&mx1, xq, rows, d, false));
-                FL_TRY(make_map(&mx2, xq + rows * d * 2, rows, d, false));
-            }
+            FL_TRY((launch_tc<kFormFp8, 1>(mx1, mx1, mwq, mwq, a, rows, st)));
+            FL_TRY(quant_rows(FLINNG_PREC_BF16X2, xc, ld, rows, d, xq, xn, nullptr, nullptr, true, st));
+            FL_TRY(make_map(&mx1, xq, rows, d, false));
+            FL_TRY(make_map(&mx2, xq + rows * d * 2, rows, d, false));
             a.c_norm = c_two;
             a.proj = nullptr;
             FL_TRY((launch_tc<kFormBf16x2, 2>(mx1, mx2, mw1, mw2, a, rows, st)));

@@ -8,6 +8,7 @@ import pytest
 
 from oracle import oracle as O
 from paper_2106_11565_gb300 import workloads as WL
+from test_gpu_tc_single import worst_case_error
 
 pytestmark = pytest.mark.gpu
 
@@ -64,4 +65,10 @@ def test_tensor_core_codes(F, form, n, d, L, K):
     assert cnt["undecided"] >= 1 and cnt["flips"] <= cnt["undecided"]
     if n > 96:
         assert cnt["compensated"] == cnt["undecided"]
+    # projections, from the dense pass's kernel too: within the formats' worst case
+    codes, _, proj = ix.hash(x, proj=True)
+    ocodes, oproj, _ = O.srp_codes(x, w, L, K, want_proj=True)
+    assert np.array_equal(codes, ocodes)
+    if form != "BF16X2":
+        assert np.all(np.abs(proj - oproj) <= worst_case_error(x, w, form.lower()) * 1.01)
     ix.close()
