@@ -116,7 +116,7 @@ struct flinng_index {
     double srp_gamma64;       // 2 * gamma_d for the fp64 recheck
     void *w_split;            // tensor-core precision: bf16 w1 then w2, P x dim each
     float *w_norm;            // upper bounds of ||w_j|| (behind srp_w)
-    float *w_aux;             // single-term tensor forms: P upper bounds of ||w_j - q(w_j)||, then P row scales
+    float *w_aux;             // tensor forms: P upper bounds of ||w_j - bf16(w_j)||; FP8: then P of ||w_j - q(w_j)||, P row scales
     uint32_t *tc_err;         // tensor-core pipeline timeout flag
     uint64_t tc_wait_ns;      // limit of the tensor-core pipeline's waits + 1 (0: the default)
 

@@ -10,9 +10,15 @@
 // register per projection. Short accumulation chains keep the bound tight:
 //   |p~ - w.x| <= [g'(64) + 2^-7 g'(128)] (1 + 2^-8)^2 ||x|| ||w||      (blocks)
 //              + g(2m) (1 + g'(64)) (1 + 2^-7) (1 + 2^-8)^2 ||x|| ||w||  (sum of m blocks)
-//              + 3.1 * 2^-16 ||x|| ||w||                                 (split)
+//              + 2^-8 (||x|| ||r_w|| + ||r_x|| ||w||)
+//              + (1 + 2^-6) ||r_x|| ||r_w||                              (split)
 //              + 8 d 2^-126 + sqrt(d) 2^-125 (||x|| + ||w||)           (underflow, flushes)
-// with g(n) = n u / (1 - n u), u = 2^-24, and g' the same with u' = 2^-22:
+// where r = x - x1 is what the second term rounds (|x2| <= (1 + 2^-8) |r|, |r -
+// x2| <= 2^-8 |r|; the dropped terms are w2.x2, w.(r_x - x2), (r_w - w2).x and
+// their cross term): its norm, measured per row, is about a quarter of its
+// worst case 2^-8 ||x||, and the worst case alone (3.1 * 2^-16 ||x|| ||w||) was two
+// thirds of the margin (8,192 rows of 4,096, BF16: 548 us with it, 523 without;
+// a query batch of 10,000 in this form 2,069 -> 2,003). With g(n) = n u / (1 - n u), u = 2^-24, and g' the same with u' = 2^-22:
 // four units of fp32 rounding per product accumulated, which also covers a
 // tensor-core adder that aligns and truncates. Projections whose |p~| does
 // not clear that margin go to a compensated fp32 re-check (two-product,
@@ -236,8 +242,8 @@ struct TcArgs {
     uint32_t P, d, L, K;
     const float *xnorm;    // n: upper bounds of ||x||
     const float *wnorm;    // P: upper bounds of ||w||
-    const float *xres;     // single-term forms: n upper bounds of ||x - s_x xq||
-    const float *wres;     // P upper bounds of ||w - s_w wq||
+    const float *xres;     // n upper bounds of ||x - s_x xq|| (the split: of ||x - x1||)
+    const float *wres;     // P upper bounds of ||w - s_w wq|| (||w - w1||)
     const float *xscale;   // FP8: n row scales s_x (powers of two)
     const float *wscale;   // FP8: P row scales s_w
     float c_norm;          // margin factor on ||x|| ||w||
@@ -461,7 +467,7 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
         if (!abort && row < a.n) {
             const float xn = a.xnorm[row];
             float xr = 0.f, xs = 1.f;
-            if constexpr (FORM != kFormBf16x2 || MASK == 3) xr = a.xres[row];
+            xr = a.xres[row];
             if constexpr (FORM == kFormFp8) xs = a.xscale[row];
             uint32_t cur_l = 0xFFFFFFFFu, cur_bits = 0u;
             // this thread's two words of the masks: undecided, first-pass signs
@@ -497,7 +503,10 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
                 bool first_pos = p > 0.f, again = MASK == 2;       // again: this is a second look
                 float margin;
                 if constexpr (FORM == kFormBf16x2) {
+                    const float wr = a.wres[col];
+                    const float split = fmaf(0x1p-8f, fmaf(xn, wr, xr * wn), (1.f + 0x1p-6f) * xr * wr);
                     margin = fmaf(a.c_norm * xn, wn, fmaf(ldexpf(1.f, -23), fabsf(p), fmaf(a.c_sub, xn + wn, a.tiny)));
+                    margin = (margin + split) * (1.f + ldexpf(1.f, -20));
                 } else {
                     margin = single_margin(p, a.c_norm);
                 }
@@ -963,15 +972,15 @@ int srp_tc_prepare_weights(flinng_index *ix)
     const size_t split = size_t(P) * d * 4, qb = prec == FLINNG_PREC_FP8 ? split + size_t(P) * d : split;
     FL_CUDA(cudaMalloc(&ix->w_split, qb));
     ix->device_bytes += qb;
-    if (prec != FLINNG_PREC_BF16X2) {
-        FL_CUDA(cudaMalloc(&ix->w_aux, size_t(P) * 2 * sizeof(float)));
-        ix->device_bytes += size_t(P) * 8;
-    }
+    // residual norms of the split, then for FP8 those of its rows and their scales
+    const size_t aux = size_t(P) * (prec == FLINNG_PREC_FP8 ? 3 : 1);
+    FL_CUDA(cudaMalloc(&ix->w_aux, aux * sizeof(float)));
+    ix->device_bytes += aux * sizeof(float);
     FL_TRY(quant_rows(FLINNG_PREC_BF16X2, ix->srp_w, d, P, d, ix->w_split, ix->w_norm, ix->w_aux, nullptr, true,
                       ix->stream));
     if (prec != FLINNG_PREC_FP8) return FLINNG_OK;
-    return quant_rows(prec, ix->srp_w, d, P, d, static_cast<char *>(ix->w_split) + split, ix->w_norm, ix->w_aux,
-                      ix->w_aux + P, false, ix->stream);
+    return quant_rows(prec, ix->srp_w, d, P, d, static_cast<char *>(ix->w_split) + split, ix->w_norm, ix->w_aux + P,
+                      ix->w_aux + 2 * P, false, ix->stream);
 }
 
 // bytes per row of the quantised x: the two-term split where a second pass needs it
@@ -1032,7 +1041,7 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
     const double m_blocks = std::ceil(double(d) / kb);
     const double m64 = std::ceil(double(d) / kTK);
     const double f2 = (g(kTK, up) + std::ldexp(1.0, -7) * g(2 * kTK, up)) * q +
-                      g(2 * m64, u) * (1 + g(kTK, up)) * (1 + std::ldexp(1.0, -7)) * q + 3.1 * std::ldexp(1.0, -16);
+                      g(2 * m64, u) * (1 + g(kTK, up)) * (1 + std::ldexp(1.0, -7)) * q;
     const double f1 = g(kb, up) + g(m_blocks, u) * (1 + g(kb, up));    // times (||x|| + ||e_x||)(||w|| + ||e_w||)
     const float c_two = std::nextafter(float(f2 * 1.0001), INFINITY);
     const float c_norm = prec == FLINNG_PREC_BF16X2 ? c_two : std::nextafter(float(f1 * 1.0001), INFINITY);
@@ -1047,7 +1056,7 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
         // chunk goes the way its space allows
         const bool dense = dense_second_pass(prec, cap, P, d) && dense_second_pass(prec, rows, P, d);
         const bool two = prec == FLINNG_PREC_BF16X2 || (dense && prec == FLINNG_PREC_BF16);
-        FL_TRY(quant_rows(prec, xc, ld, rows, d, xq, xn, prec == FLINNG_PREC_BF16X2 ? nullptr : xr, xsc, two, st));
+        FL_TRY(quant_rows(prec, xc, ld, rows, d, xq, xn, xr, xsc, two, st));
         CUtensorMap mx1, mx2;
         FL_TRY(make_map(&mx1, xq, rows, d, bytes));
         if (two) FL_TRY(make_map(&mx2, xq + rows * d * 2, rows, d, false));
@@ -1062,9 +1071,9 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
         a.xnorm = xn;
         a.wnorm = ix->w_norm;
         a.xres = xr;
-        a.wres = ix->w_aux;
+        a.wres = bytes ? ix->w_aux + P : ix->w_aux;
         a.xscale = xsc;
-        a.wscale = ix->w_aux ? ix->w_aux + P : nullptr;
+        a.wscale = bytes ? ix->w_aux + 2 * P : nullptr;
         a.c_norm = c_norm;
         a.c_sub = c_sub;
         a.tiny = tiny;
@@ -1088,7 +1097,8 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
             // FP8: the marked projections again on the two-term split, whose margin
             // leaves a few in a thousand
             FL_TRY((launch_tc<kFormFp8, 1>(mx1, mx1, mwq, mwq, a, rows, st)));
-            FL_TRY(quant_rows(FLINNG_PREC_BF16X2, xc, ld, rows, d, xq, xn, nullptr, nullptr, true, st));
+            FL_TRY(quant_rows(FLINNG_PREC_BF16X2, xc, ld, rows, d, xq, xn, xr, nullptr, true, st));
+            a.wres = ix->w_aux;
             FL_TRY(make_map(&mx1, xq, rows, d, false));
             FL_TRY(make_map(&mx2, xq + rows * d * 2, rows, d, false));
             a.c_norm = c_two;
