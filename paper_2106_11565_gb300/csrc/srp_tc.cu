@@ -40,7 +40,7 @@
 // ||e_x||) (||w|| + ||e_w||), 2^-23 |p~|, the underflow terms above, and a
 // 2^-20 relative slack for evaluating the margin itself in fp32.
 //
-// Kernel layout (one CTA per 128 points x 128 projections, 320 threads):
+// Kernel layout (one CTA per 128 points x 128 projections, 576 threads):
 //   warp 0     TMA producer: 3-stage ring of {X1, X2, W1, W2} tiles of 128 rows
 //              x 64 bf16 (128-byte swizzle), one mbarrier per stage (single-term
 //              forms: a 6-stage ring of {X, W} tiles of 128 rows x 128 bytes);
@@ -50,8 +50,8 @@
 //              x2 w1 (N=128, into lo) - then commits the stage back to the
 //              producer and the buffer to the epilogue (single-term forms: one
 //              N=128 MMA per 32-byte step into a 128-column buffer);
-//   warps 2-9  epilogue: warp w reads TMEM lanes 32 (w % 4) .. +32 (one point per
-//              thread) and 64 of the 128 columns, drains each buffer into fp32
+//   warps 2-17 epilogue: warp w reads TMEM lanes 32 (w % 4) .. +32 (one point per
+//              thread) and 32 of the 128 columns, drains each buffer into fp32
 //              registers and hands it back; at the end decides the signs,
 //              writes the codes and lists ambiguous projections.
 // Every wait on an mbarrier is bounded; on timeout the CTA sets an error flag,
@@ -86,7 +86,7 @@ template <> struct TcForm<kFormFp8> {
 };
 template <int FORM>
 constexpr size_t tc_smem_bytes() { return size_t(TcForm<FORM>::kStages) * TcForm<FORM>::kTiles * kTileBytes + 1024 + 256; }
-constexpr int kEpiWarps = 8;                      // two per TMEM lane quarter, 64 columns each
+constexpr int kEpiWarps = 16;                     // four per TMEM lane quarter, 32 columns each
 constexpr int kTcThreads = 64 + 32 * kEpiWarps;
 constexpr uint64_t kWaitNs = 1000000000ull;       // bounded mbarrier waits: 1 s
 constexpr uint64_t kTcChunkRows = 16384;          // rows split and hashed per launch
@@ -207,9 +207,28 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar)
                  ::"r"(smem_u32(bar)) : "memory");
 }
 
-// 32 consecutive fp32 columns of this warp's 32 TMEM lanes; the caller waits
+// N consecutive fp32 columns of this warp's 32 TMEM lanes; the caller waits
 // (tmem_wait_ld) before reading the registers.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t r[32])
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[8])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+        : "r"(taddr));
+}
+
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+}
+
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[32])
 {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -219,16 +238,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t r[32])
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
           "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t r[16])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
 }
 
@@ -271,8 +280,8 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 // first pass of the FP8 form whose undecided share is large); 2 only the marked
 // ones are decided (its second pass, on the two-term split), the rest listed; 3
 // both passes of the BF16 form at once, whose first pass is the split's x1 w1
-// half: the sums of that half are kept beside the full ones (128 accumulators a
-// thread, which the 320 threads' registers hold), so the second pass costs the
+// half: the sums of that half are kept beside the full ones (64 accumulators a
+// thread), so the second pass costs the
 // split's two extra MMAs per step and no second reading of the operands.
 template <int FORM, int MASK>
 __global__ void __launch_bounds__(kTcThreads, 1)
@@ -387,16 +396,21 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
         }
     } else {
         // epilogue: TMEM lanes [32 (warp % 4), +32) = one point per thread;
-        // columns [64 half, +64) of the tile
+        // columns [32 group, +32) of the tile. Each warp's drain of a k-block is a
+        // chain (barrier, TMEM loads, adds): four warps per scheduler overlap theirs
+        // and add in pairs. With two (64 columns each) and single adds it took 1.03
+        // us a k-block in the two-term form and 1.49 with both passes' sums, against
+        // 0.61 for operands and MMAs alone; now 0.68 and 0.70 (0.77 and 0.86 with
+        // single adds). 10,000 rows of 4,096: 329 -> 268 us, 8,192 in BF16: 374 -> 228.
         const uint32_t quarter = (warp & 3) * 32;
-        const uint32_t half = uint32_t(warp - 2) >> 2;
-        const uint32_t tbase = tmem + (quarter << 16) + 64u * half;
-        float acc[64];
-        float one[MASK == 3 ? 64 : 1];       // the first pass's sums
+        const uint32_t group = uint32_t(warp - 2) >> 2;
+        const uint32_t tbase = tmem + (quarter << 16) + 32u * group;
+        float acc[32];
+        float one[MASK == 3 ? 32 : 1];       // the first pass's sums
 #pragma unroll
-        for (int j = 0; j < 64; ++j) acc[j] = 0.f;
+        for (int j = 0; j < 32; ++j) acc[j] = 0.f;
 #pragma unroll
-        for (int j = 0; j < (MASK == 3 ? 64 : 1); ++j) one[j] = 0.f;
+        for (int j = 0; j < (MASK == 3 ? 32 : 1); ++j) one[j] = 0.f;
         bool abort = false;
         for (uint32_t kb = 0; kb < nkb; ++kb) {
             const uint32_t b = kb & 1u;
@@ -409,92 +423,68 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if constexpr (MASK == 3) {
-                // four quarters: 128 accumulators leave room for 32 values in flight
+            // kIn columns in flight: 96 registers a thread (five warps on a scheduler)
+            // hold no more beside the accumulators. The buffer goes back to the MMA
+            // issuer before its last values are added.
+            constexpr int kIn = MASK == 3 ? 8 : FORM == kFormBf16x2 ? 16 : 32;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    uint32_t hv[16], lv[16];
-                    tmem_ld16(tbase + kBuf * b + 16 * q, hv);
-                    tmem_ld16(tbase + kBuf * b + kTN + 16 * q, lv);
-                    tmem_wait_ld();
-                    if (q == 3) {
-                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&tempty[b]);
-                    }
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        acc[16 * q + j] += __uint_as_float(hv[j]) + __uint_as_float(lv[j]);
-                        one[16 * q + j] += __uint_as_float(hv[j]);
-                    }
+            for (int q = 0; q < 32; q += kIn) {
+                uint32_t hv[kIn], lv[kIn];
+                tmem_ld(tbase + kBuf * b + q, hv);
+                if constexpr (FORM == kFormBf16x2) tmem_ld(tbase + kBuf * b + kTN + q, lv);
+                tmem_wait_ld();
+                if (q + kIn == 32) {
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&tempty[b]);
                 }
-            } else if constexpr (FORM == kFormBf16x2) {
-                // two halves of 32 columns: hi and lo loads in flight together, one
-                // wait each; the buffer goes back to the MMA issuer before the
-                // second half is added
-                uint32_t hv[32], lv[32];
-                tmem_ld32(tbase + kBuf * b, hv);
-                tmem_ld32(tbase + kBuf * b + kTN, lv);
-                tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 32; ++j) acc[j] += __uint_as_float(hv[j]) + __uint_as_float(lv[j]);
-                tmem_ld32(tbase + kBuf * b + 32, hv);
-                tmem_ld32(tbase + kBuf * b + kTN + 32, lv);
-                tmem_wait_ld();
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&tempty[b]);
-#pragma unroll
-                for (int j = 0; j < 32; ++j) acc[32 + j] += __uint_as_float(hv[j]) + __uint_as_float(lv[j]);
-            } else {
-                uint32_t hv[32], hw[32];
-                tmem_ld32(tbase + kBuf * b, hv);
-                tmem_ld32(tbase + kBuf * b + 32, hw);
-                tmem_wait_ld();
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&tempty[b]);
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    acc[j] += __uint_as_float(hv[j]);
-                    acc[32 + j] += __uint_as_float(hw[j]);
+                for (int j = 0; j < kIn; j += 2) {
+                    float2 h = make_float2(__uint_as_float(hv[j]), __uint_as_float(hv[j + 1])), t = h;
+                    if constexpr (FORM == kFormBf16x2)
+                        t = __fadd2_rn(h, make_float2(__uint_as_float(lv[j]), __uint_as_float(lv[j + 1])));
+                    t = __fadd2_rn(make_float2(acc[q + j], acc[q + j + 1]), t);
+                    acc[q + j] = t.x;
+                    acc[q + j + 1] = t.y;
+                    if constexpr (MASK == 3) {
+                        h = __fadd2_rn(make_float2(one[q + j], one[q + j + 1]), h);
+                        one[q + j] = h.x;
+                        one[q + j + 1] = h.y;
+                    }
                 }
             }
         }
         uint32_t ab = lane == 0 ? *(volatile uint32_t *)abort_flag : 0u;
         abort = abort || __shfl_sync(0xffffffffu, ab, 0) != 0u;    // warp-uniform
         const uint64_t row = uint64_t(row0) + quarter + lane;
+        // bits by column: undecided, first-pass signs
+        uint32_t und = 0u, sgn = 0u, decided = 0u, flips = 0u, open = 0u;
+        const uint32_t cbase = col0 + 32u * group;
         if (!abort && row < a.n) {
-            const float xn = a.xnorm[row];
-            float xr = 0.f, xs = 1.f;
-            xr = a.xres[row];
+            const float xn = a.xnorm[row], xr = a.xres[row];
+            float xs = 1.f;
             if constexpr (FORM == kFormFp8) xs = a.xscale[row];
             uint32_t cur_l = 0xFFFFFFFFu, cur_bits = 0u;
-            // this thread's two words of the masks: undecided, first-pass signs
-            const uint32_t pw = (a.P + 31) / 32, w0 = (col0 + 64u * half) / 32;
-            uint32_t und[2] = {0u, 0u}, sgn[2] = {0u, 0u}, decided = 0u, flips = 0u, open = 0u;
+            // this thread's word of the masks
+            const uint32_t pw = (a.P + 31) / 32, w0 = cbase / 32;
             uint32_t *mrow = MASK == 1 || MASK == 2 ? a.mask + row * (2 * pw) + w0 : nullptr;
+            uint32_t todo = 0xFFFFFFFFu, first = 0u;
             if constexpr (MASK == 2) {
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-                    if (w0 + i < pw) {
-                        und[i] = mrow[i];
-                        sgn[i] = mrow[pw + i];
-                    }
+                todo = w0 < pw ? mrow[0] : 0u;
+                first = w0 < pw ? mrow[pw] : 0u;
             }
 #pragma unroll
-            for (int j = 0; j < 64; ++j) {
-                const uint32_t col = col0 + 64u * half + j;
+            for (int j = 0; j < 32; ++j) {
+                const uint32_t col = cbase + j;
                 if (col >= a.P) break;
-                if (MASK == 2 && !((und[j / 32] >> (j % 32)) & 1u)) continue;
+                if (MASK == 2 && !((todo >> j) & 1u)) continue;
                 float p = acc[j];
-                if constexpr (FORM == kFormFp8) p *= xs * a.wscale[col];    // powers of two: exact
-                const float wn = a.wnorm[col];
+                if constexpr (FORM == kFormFp8) p *= xs * __ldg(a.wscale + col);    // powers of two: exact
+                const float wn = __ldg(a.wnorm + col), wr = __ldg(a.wres + col);
                 if (a.proj) a.proj[row * a.P + col] = MASK == 3 ? one[MASK == 3 ? j : 0] : p;
                 // residual term (Cauchy-Schwarz on the quantisation errors) plus
                 // accumulation on the quantised operands' norms, then slack
                 auto single_margin = [&](float v, float c) {
-                    const float wr = a.wres[col];
                     const float resid = fmaf(xn, wr, fmaf(xr, wn, 3.f * xr * wr));
                     const float accum = c * (xn + xr) * (wn + wr);
                     return (resid + accum + fmaf(ldexpf(1.f, -23), fabsf(v), fmaf(a.c_sub, xn + wn, a.tiny))) *
@@ -503,14 +493,13 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
                 bool first_pos = p > 0.f, again = MASK == 2;       // again: this is a second look
                 float margin;
                 if constexpr (FORM == kFormBf16x2) {
-                    const float wr = a.wres[col];
                     const float split = fmaf(0x1p-8f, fmaf(xn, wr, xr * wn), (1.f + 0x1p-6f) * xr * wr);
                     margin = fmaf(a.c_norm * xn, wn, fmaf(ldexpf(1.f, -23), fabsf(p), fmaf(a.c_sub, xn + wn, a.tiny)));
                     margin = (margin + split) * (1.f + ldexpf(1.f, -20));
                 } else {
                     margin = single_margin(p, a.c_norm);
                 }
-                if constexpr (MASK == 2) first_pos = ((sgn[j / 32] >> (j % 32)) & 1u) != 0u;
+                if constexpr (MASK == 2) first_pos = ((first >> j) & 1u) != 0u;
                 if constexpr (MASK == 3) {
                     const float v = one[j];
                     first_pos = v > 0.f;
@@ -532,33 +521,51 @@ k_srp_tc(const __grid_constant__ CUtensorMap mx1, const __grid_constant__ CUtens
                         }
                         cur_bits |= 1u << (col % a.K);
                     }
-                } else if constexpr (MASK == 1) {
-                    und[j / 32] |= 1u << (j % 32);
-                    if (p > 0.f) sgn[j / 32] |= 1u << (j % 32);
                 } else {
                     // the tentative sign a later re-check may reverse is the first pass's
-                    const unsigned long long slot = atomicAdd(a.rcount, 1ull);
-                    a.rlist[slot] = (first_pos ? kEntSign : 0ull) | ((unsigned long long)row << 20) | col;
+                    und |= 1u << j;
+                    if (first_pos) sgn |= 1u << j;
                 }
             }
             if (cur_bits) atomicOr(&a.codes[row * a.L + cur_l], cur_bits);
             if constexpr (MASK == 1) {
+                if (w0 < pw) {
+                    mrow[0] = und;
+                    mrow[pw] = sgn;
+                }
+            }
+        }
+        // lists and counters: one atomic a warp. One per undecided projection
+        // and per thread, all on a few words, were 10 us of a wave of tiles in the
+        // two-term form and 31 us in the BF16 form's.
+        const uint32_t c = __popc(und);
+        if constexpr (MASK == 1) {
+            const uint32_t all = __reduce_add_sync(0xffffffffu, c);
+            if (all && lane == 0) atomicAdd(a.nund, (unsigned long long)all);
+        } else if (__any_sync(0xffffffffu, c != 0u)) {
+            uint32_t incl = c;
 #pragma unroll
-                for (int i = 0; i < 2; ++i)
-                    if (w0 + i < pw) {
-                        mrow[i] = und[i];
-                        mrow[pw + i] = sgn[i];
-                    }
-                const uint32_t c = __popc(und[0]) + __popc(und[1]);
-                if (c) atomicAdd(a.nund, (unsigned long long)c);
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
+                if (lane >= d) incl += y;
             }
-            if constexpr (MASK == 3) {
-                if (open) atomicAdd(a.nund, (unsigned long long)open);
+            unsigned long long at = 0;
+            if (lane == 31) at = atomicAdd(a.rcount, (unsigned long long)incl);
+            at = __shfl_sync(0xffffffffu, at, 31) + (incl - c);
+            for (uint32_t m = und; m; m &= m - 1u) {
+                const uint32_t j = __ffs(m) - 1;
+                a.rlist[at++] = ((sgn >> j) & 1u ? kEntSign : 0ull) | ((unsigned long long)row << 20) | (cbase + j);
             }
-            if constexpr (MASK >= 2) {
-                if (decided) atomicAdd(&a.stats[3], (unsigned long long)decided);
-                if (flips) atomicAdd(&a.stats[4], (unsigned long long)flips);
-            }
+        }
+        if constexpr (MASK == 3) {
+            open = __reduce_add_sync(0xffffffffu, open);
+            if (open && lane == 0) atomicAdd(a.nund, (unsigned long long)open);
+        }
+        if constexpr (MASK >= 2) {
+            decided = __reduce_add_sync(0xffffffffu, decided);
+            flips = __reduce_add_sync(0xffffffffu, flips);
+            if (decided && lane == 0) atomicAdd(&a.stats[3], (unsigned long long)decided);
+            if (flips && lane == 0) atomicAdd(&a.stats[4], (unsigned long long)flips);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
