@@ -374,7 +374,7 @@ int flinng_hash_stats(const flinng_index *idx, uint64_t *n_recheck,
  * index: out[0] projections the first pass (fp32 FMA or tensor cores) could
  * not decide; out[1] those decided by the exact accumulator; out[2] fp64
  * re-checks; out[3] second-stage re-checks of the tensor-core precisions
- * (compensated fp32, or a dense pass on the two-term split for a large batch of
+ * (compensated fp32, or a dense pass on the two-term split in
  * a single-term form; none for a batch of at most 96 rows, which every
  * precision hashes in fp32 unless projections are asked for);
  * out[4] flips: first-pass signs that a re-check reversed (the hash-bit flip

@@ -534,8 +534,9 @@ size_t srp_workspace_bytes(const flinng_index *ix, uint64_t n)
 // Small batches take the fp32 warp-per-projection kernel: the GEMM's tiles would
 // be a few CTAs, each walking all of d. The lines lie where the two cross: 1,024
 // projections at d = 4096, 128 rows 145 us against 216 (tiles), 192 rows 208
-// against 216; the tensor-core path needs 118 us for any of them and crosses at
-// 96 rows (116). Less work per row (fewer projections) moves the fp32 line out
+// against 216; the tensor-core path needs 98 us for any of them (two-term; 108 and
+// 158 the single-term forms) against 94 at 72 rows and 118 at 96, and at d = 1024
+// 57 (58, 81) against 50 at 96: the line lies between. Less work per row (fewer projections) moves the fp32 line out
 // in proportion (384 projections at d = 512: equal at 512 rows). In the tensor-
 // core precisions only without projections to return: the codes are the same.
 bool srp_few_rows(const flinng_index *ix, uint64_t n, const float *proj)

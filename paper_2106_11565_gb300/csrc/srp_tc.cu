@@ -922,16 +922,16 @@ inline size_t qrow_bytes(uint32_t precision, uint32_t d)
 // A single-term form leaves a share of the projections undecided that grows
 // with its residual norms (about a sixth at d = 4096 in BF16, nearly all in
 // FP8). Re-checked one by one, each streams its row of W from L2 (2.3 ns per
-// projection at d = 4096 with every SM busy); a dense second pass on the
-// two-term split costs 0.05 ns per projection of the batch, decided or not, so
-// it wins from an undecided share of about 2 %: d >= 128 in BF16, any d in FP8,
-// once the batch fills the chip (2^20 projections: 64 tiles of 128 x 128). 8,192
-// embeddings in BF16: 4.04 ms re-checked one by one, 0.76 ms with a second pass,
-// 0.57 ms with both passes in one kernel (MASK = 3).
-inline bool dense_second_pass(uint32_t precision, uint64_t rows, uint32_t P, uint32_t d)
+// projection at d = 4096 with every SM busy, more for a batch of a few rows); a
+// dense second pass on the two-term split costs 0.05 ns per projection of a large
+// batch, decided or not, and no more than a tile's depth for a small one, so it
+// wins from an undecided share of about 2 %: d >= 128 in BF16, any d in FP8.
+// 8,192 embeddings in BF16: 4.04 ms re-checked one by one, 0.37 ms with both
+// passes in one kernel (MASK = 3); 97 of them 280 against 108 us, in FP8 1,043
+// against 158 (128 dimensions, 256 projections: 61 against 45, 77 against 65).
+inline bool dense_second_pass(uint32_t precision, uint32_t d)
 {
-    if (precision != FLINNG_PREC_BF16 && precision != FLINNG_PREC_FP8) return false;
-    return rows * P >= (1ull << 20) && (precision == FLINNG_PREC_FP8 || d >= 128);
+    return precision == FLINNG_PREC_FP8 || (precision == FLINNG_PREC_BF16 && d >= 128);
 }
 
 // two: also x2 behind x1 (the BF16 form's second pass)
@@ -991,16 +991,16 @@ int srp_tc_prepare_weights(flinng_index *ix)
 }
 
 // bytes per row of the quantised x: the two-term split where a second pass needs it
-static size_t x_bytes(const flinng_index *ix, uint64_t rows)
+static size_t x_bytes(const flinng_index *ix)
 {
-    return dense_second_pass(ix->cfg.precision, rows, ix->P, ix->cfg.dim) ? size_t(ix->cfg.dim) * 4
-                                                                          : qrow_bytes(ix->cfg.precision, ix->cfg.dim);
+    return dense_second_pass(ix->cfg.precision, ix->cfg.dim) ? size_t(ix->cfg.dim) * 4
+                                                             : qrow_bytes(ix->cfg.precision, ix->cfg.dim);
 }
 
 size_t srp_tc_workspace_bytes(const flinng_index *ix, uint64_t n)
 {
     const uint64_t rows = n < kTcChunkRows ? n : kTcChunkRows;
-    return carve_bytes<char>(rows * x_bytes(ix, rows)) + 3 * carve_bytes<float>(rows) +
+    return carve_bytes<char>(rows * x_bytes(ix)) + 3 * carve_bytes<float>(rows) +
            carve_bytes<unsigned long long>(8) + 2 * carve_bytes<unsigned long long>(rows * ix->P + 1) +
            3 * carve_bytes<uint32_t>(rows + 1) + carve_bytes<char>(scan_workspace_bytes(rows + 1)) + 4096;
 }
@@ -1017,7 +1017,7 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
     const uint64_t chunk = kTcChunkRows;
     const uint64_t cap = n < chunk ? n : chunk;     // rows the workspace was sized for
     Carver c(ws, ~size_t(0));
-    char *xq = c.take<char>(cap * x_bytes(ix, cap));
+    char *xq = c.take<char>(cap * x_bytes(ix));
     float *xn = c.take<float>(cap);
     float *xr = c.take<float>(cap);
     float *xsc = c.take<float>(cap);
@@ -1059,9 +1059,7 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
     for (uint64_t r0 = 0; r0 < n; r0 += chunk) {
         const uint64_t rows = (n - r0) < chunk ? (n - r0) : chunk;
         const float *xc = x + r0 * ld;
-        // capped by the rows the workspace was sized for, so that the last, shorter
-        // chunk goes the way its space allows
-        const bool dense = dense_second_pass(prec, cap, P, d) && dense_second_pass(prec, rows, P, d);
+        const bool dense = dense_second_pass(prec, d);
         const bool two = prec == FLINNG_PREC_BF16X2 || (dense && prec == FLINNG_PREC_BF16);
         FL_TRY(quant_rows(prec, xc, ld, rows, d, xq, xn, xr, xsc, two, st));
         CUtensorMap mx1, mx2;
@@ -1094,8 +1092,7 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
         a.err = ix->tc_err;
         a.wait_ns = ix->tc_wait_ns ? ix->tc_wait_ns - 1 : kWaitNs;
         if (prec == FLINNG_PREC_BF16X2) FL_TRY((launch_tc<kFormBf16x2, 0>(mx1, mx2, mw1, mw2, a, rows, st)));
-        else if (!dense && prec == FLINNG_PREC_BF16) FL_TRY((launch_tc<kFormBf16, 0>(mx1, mx1, mwq, mwq, a, rows, st)));
-        else if (!dense) FL_TRY((launch_tc<kFormFp8, 0>(mx1, mx1, mwq, mwq, a, rows, st)));
+        else if (!dense) FL_TRY((launch_tc<kFormBf16, 0>(mx1, mx1, mwq, mwq, a, rows, st)));
         else if (prec == FLINNG_PREC_BF16) {
             a.c_one = c_norm;
             a.c_norm = c_two;
@@ -1112,9 +1109,9 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
             a.proj = nullptr;
             FL_TRY((launch_tc<kFormBf16x2, 2>(mx1, mx2, mw1, mw2, a, rows, st)));
         }
-        // stage 2: compensated fp32; stage 3: fp64 / exact. A list of a sixth of
-        // the projections or more is grouped by row, so that each row of x is
-        // staged once; a short one is not worth the passes.
+        // stage 2: compensated fp32; stage 3: fp64 / exact. A
+        // single-term list (d < 128) is grouped by row, so that each row of x is
+        // staged once; the others are short and not worth the passes.
         if (rows_staged && !dense && prec != FLINNG_PREC_BF16X2) {
             // the list grouped by row into list2; stage 2 lists what stays undecided in list1
             FL_CUDA(cudaMemsetAsync(rowcnt, 0, (rows + 1) * sizeof(uint32_t), st));
