@@ -536,9 +536,10 @@ size_t srp_workspace_bytes(const flinng_index *ix, uint64_t n)
 // projections at d = 4096, 128 rows 145 us against 216 (tiles), 192 rows 208
 // against 216; the tensor-core path needs 98 us for any of them (two-term; 108 and
 // 158 the single-term forms) against 94 at 72 rows and 118 at 96, and at d = 1024
-// 57 (58, 81) against 50 at 96: the line lies between. Less work per row (fewer projections) moves the fp32 line out
-// in proportion (384 projections at d = 512: equal at 512 rows). In the tensor-
-// core precisions only without projections to return: the codes are the same.
+// 57 (58, 81) against 50 at 96: the line lies between. Less work per row (fewer
+// projections) moves the fp32 line out in proportion (384 projections at d = 512:
+// equal at 512 rows). In the tensor-core precisions only without projections to
+// return: the codes are the same.
 bool srp_few_rows(const flinng_index *ix, uint64_t n, const float *proj)
 {
     if (ix->cfg.precision == FLINNG_PREC_FP32) return n * ix->P <= 192 * 1024;
