@@ -90,7 +90,7 @@ struct QSmem {
     uint64_t *buf;       // cap candidate keys
     uint64_t *keep;      // kp keys (selection output, final sort)
     uint32_t *u;         // 8 scalars: nbuf, nkeep, digit / k-th score, rank / found, whole / count,
-                         // heavy tables, bound (u[6..7])
+                         // heavy tables (gather) / cells of a big level (decode), bound (u[6..7])
     uint32_t *lvl_n;     // nlev: repetition-0 cells per count, then cells at levels >= v
     uint32_t *shist;     // nlev: candidates in buf per score
     uint32_t *rhist;     // 256: radix histogram
@@ -899,13 +899,17 @@ __device__ void decode_topk(const QArgs &a, const QSmem &s, uint32_t q, uint32_t
             for (uint32_t b0 = 0; b0 < (big ? a.B : 1u); b0 += a.lcap) {
                 uint32_t first = above - seg_base, nc = s.lvl_n[t_end] - above;
                 if (big) {
+                    // a cursor of its own (u[5], free here): the words of lvl_cur are
+                    // those of c_pre, which is written below as soon as the count is
+                    // read, and t = kCh would be its closing word
                     first = 0;
-                    if (tid == 0) s.lvl_cur[t] = 0u;
+                    if (tid == 0) s.u[5] = 0u;
                     __syncthreads();
                     for (uint32_t b = b0 + tid; b < min(b0 + a.lcap, a.B); b += NT)
-                        if (cnt_at<CW>(s, b) == uint32_t(t)) s.lvl_cells[atomicAdd(&s.lvl_cur[t], 1u)] = uint16_t(b);
+                        if (cnt_at<CW>(s, b) == uint32_t(t)) s.lvl_cells[atomicAdd(&s.u[5], 1u)] = uint16_t(b);
                     __syncthreads();
-                    nc = s.lvl_cur[t];
+                    nc = s.u[5];
+                    __syncthreads();        // read by all before the next range's zero
                 }
                 // the filter pays while fewer than half the members pass it: about the
                 // share of cells that reach the admission bound (any repetition's counts
