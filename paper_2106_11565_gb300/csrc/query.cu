@@ -37,28 +37,44 @@ QArgs make_args(flinng_index *ix, const uint32_t *qb, uint32_t nq)
     a.t_min = ix->cfg.min_threshold;
     a.avg_cell = uint32_t((ix->n_points + ix->cfg.B - 1) / ix->cfg.B);
     a.gcells = 1;
+    a.id_bits = 1;
+    while (a.id_bits < 32 && (ix->cfg.capacity - 1) >> a.id_bits) ++a.id_bits;
     return a;
 }
 
+// Members that a query walks, by the average length of its tables' lists.
+uint64_t expected_members(const flinng_index *ix)
+{
+    const uint64_t per = (ix->n_points + ix->cfg.B - 1) / ix->cfg.B;
+    return ix->n_cells * ix->cfg.L / (ix->nslot * ix->cfg.R) * per;
+}
+
+constexpr uint64_t kLightMembers = 600;
+
 // Candidate buffer: room for one full round of members after a compaction
-// to k keys; tune->cap overrides the default when large enough. The default is
-// kept small: the buffer's 8 bytes per entry cost resident CTAs (10^4 URL
-// queries, k = 10: 1.25 ms with 512 entries, 1.34 with 1,024).
-void pick_buffer(QArgs &a, int NT, const QueryTuning *tune, size_t extra, size_t *smem_out, int cw)
+// to k keys; tune->cap overrides the default when large enough. The default
+// holds about four times k, so that a flood of equal scores is cut early and
+// seldom; its 8 bytes per entry cost resident CTAs (10^4 URL queries, k = 10:
+// 1.25 ms with 512 entries, 1.34 with 1,024), and past 2,048 entries (or what two
+// rounds of k need) they cost more than the cuts (4,000 configured genomic
+// queries, k = 1,024: 61 us with 2,048, 157 with 8,192). Queries of a few
+// hundred members flood nothing: the smallest.
+void pick_buffer(QArgs &a, int NT, const QueryTuning *tune, size_t extra, size_t *smem_out, int cw, bool light)
 {
     a.kp = pow2_at_least(a.k_max > 1 ? a.k_max : 2);
     // the decode appends freely up to cap - (NT + 32), then compacts: that
     // mark must stay above the kp keys a compaction keeps
     const uint32_t cap_min = pow2_at_least(a.kp + uint32_t(NT + 32) + 1);
-    uint32_t cap = pow2_at_least((tune && tune->cap) ? tune->cap : 4 * a.kp + uint32_t(NT + 32));
+    const uint32_t most = std::max(2048u, pow2_at_least(2 * a.kp + uint32_t(NT + 32)));
+    uint32_t cap = (tune && tune->cap) ? pow2_at_least(tune->cap)
+                   : light             ? cap_min
+                                       : std::min(most, pow2_at_least(4 * a.kp + uint32_t(NT + 32)));
     if (cap < cap_min) cap = cap_min;
-    a.cap = cap;
     a.lcap = a.B < kLevelCells ? (a.B + 7) & ~7u : kLevelCells;
-    size_t smem = qsmem_bytes(a.cap, a.kp, a.BR, a.lcap, NT, a.L, cw);
-    while (smem + extra > 227 * 1024 && a.cap > cap_min) {
-        a.cap >>= 1;
-        smem = qsmem_bytes(a.cap, a.kp, a.BR, a.lcap, NT, a.L, cw);
-    }
+    auto bytes = [&](uint32_t c) { return qsmem_bytes(c, a.kp, a.BR, a.lcap, NT, a.L, cw); };
+    while (bytes(cap) + extra > 227 * 1024 && cap > cap_min) cap >>= 1;
+    a.cap = cap;
+    const size_t smem = bytes(cap);
     *smem_out = smem;
     // one stop check per level group: the first of about 1,024 members (4 k for
     // larger k), then doubling to 16,384
@@ -67,7 +83,7 @@ void pick_buffer(QArgs &a, int NT, const QueryTuning *tune, size_t extra, size_t
     a.gcells = std::min(std::max(g0, 1u), a.lcap);
     a.gmax = std::min(std::max(16384u / per, a.gcells), a.lcap);
     // eight members per lane need cells that fill them
-    a.wide = a.avg_cell >= 8 ? 1u : 0u;
+    a.wide = a.R > 1 && a.avg_cell >= 8 ? 1u : 0u;
 }
 
 }  // namespace
@@ -97,25 +113,36 @@ int query_launch_counts(flinng_index *ix, const uint32_t *qbuckets, const uint16
     a.out_ids = out_ids;
     a.out_scores = out_scores;
     a.out_row = out_row;
-    // CTA size: the smallest that keeps the most threads on an SM (with large
-    // B*R shared memory admits only one or two CTAs)
+    // CTA size: 512 threads for a batch that is then resident at once, since it
+    // waits for its slowest query (80 and 300 queries, sets and vectors: 0.85 times
+    // the time of 256 threads), else the smallest that keeps the most threads on
+    // an SM (with large B*R shared memory admits only one or two CTAs)
+    if (!ix->sms) FL_CUDA(cudaDeviceGetAttribute(&ix->sms, cudaDevAttrMultiProcessorCount, ix->device));
+    const uint32_t sms = uint32_t(ix->sms);
+    const bool light = !counts && expected_members(ix) < kLightMembers;
     int NT = 256;
     size_t smem = 0;
     uint32_t most = 0;
     for (int nt = 256; nt <= 1024; nt *= 2) {
-        pick_buffer(a, nt, nullptr, 0, &smem, cw);
-        const uint32_t on = std::min(kPlainThreads, uint32_t(228 * 1024 / (smem + 1024)) * nt);
-        if (on > most) {
+        pick_buffer(a, nt, nullptr, 0, &smem, cw, light);
+        const uint32_t ctas = uint32_t(228 * 1024 / (smem + 1024)), on = std::min(1024u, ctas * nt);
+        if (on > most || (nt == 512 && nq <= sms * std::min(ctas, 2u))) {
             most = on;
             NT = nt;
         }
     }
-    pick_buffer(a, NT, nullptr, 0, &smem, cw);
+    pick_buffer(a, NT, nullptr, 0, &smem, cw, light);
+    // 32 registers a thread for a batch of more than one wave of such CTAs, where
+    // shared memory admits them: more queries overlap their chains of loads (4,000
+    // given counts of 60,000 reads in 128 tables, k = 10: 172 us with 64 registers,
+    // 130 so; a batch resident at once, 1,200 of them, 54 and 60; 16-bit counts,
+    // 4,000 queries of 512 tables, 144 and 188)
+    const uint32_t sm_threads = NT == 256 && cw == 1 && 228 * 1024 / (smem + 1024) > 4 && nq > 8 * sms ? 2048 : 1024;
     if (smem > 227 * 1024)
         return set_error(FLINNG_ERR_INVALID_ARG,
                          "query: k_max=%u with B*R=%u needs %zu bytes of shared memory (> 227 KB)",
                          k_max, a.BR, smem);
-    const void *fn = cw == 1 ? plain_kernel_c1(NT, ix->rw) : plain_kernel_c2(NT, ix->rw);
+    const void *fn = cw == 1 ? plain_kernel_c1(NT, ix->rw, sm_threads) : plain_kernel_c2(NT, ix->rw, sm_threads);
     FL_TRY(ensure_dyn_smem(fn, smem));
     void *args[] = {&a};
     FL_CUDA(cudaLaunchKernel(fn, dim3(nq), dim3(NT), args, smem, ix->stream));   // one CTA per query
@@ -182,14 +209,15 @@ static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t 
     // only before the decode keeps candidates, so it shares the candidate
     // buffer with the gather's heavy-table list (the buffer's last 2 NT words)
     // when both fit; otherwise it follows the query state.
+    const bool light = expected_members(ix) < kLightMembers;
     auto shape = [&](int nt) {
         size_t qbytes;
-        pick_buffer(a, nt, tune, 0, &qbytes, int(ix->cw));
+        pick_buffer(a, nt, tune, 0, &qbytes, int(ix->cw), light);
         if (hash_bytes + size_t(nt) * 8 <= size_t(a.cap) * 8) {
             h.hash_off = 0;
             P->smem = qbytes;
         } else {
-            pick_buffer(a, nt, tune, hash_bytes, &qbytes, int(ix->cw));
+            pick_buffer(a, nt, tune, hash_bytes, &qbytes, int(ix->cw), light);
             h.hash_off = qbytes;
             P->smem = qbytes + hash_bytes;
         }
@@ -200,7 +228,12 @@ static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t 
     // 128). A larger batch takes 256 when shared memory still admits four such
     // CTAs per SM, so that more queries overlap their phases (10^4 URL queries:
     // 1.24 ms against 1.46 with 512; 1,000 configured genomic queries: 35 us
-    // against 45), else 512.
+    // against 45), else 512. Where a query walks few members (the lists of its
+    // tables, by their average length, lead to a few hundred) its time is that of
+    // barriers and scans, which grow with the CTA: more than two such queries per
+    // SM take 256 threads, more than four 128, if that leaves the SM three quarters
+    // of its threads (30,000 reads in 16 tables, k = 10, 512 / 256 / 128 threads: 600
+    // queries 18.6 / 14.6 / 14.5 us, 4,000 queries 92 / 57 / 46).
     int NT = tune && tune->threads ? int(tune->threads) : 512;
     shape(NT);
     auto fit = [&]() { return uint32_t(228 * 1024 / (P->smem + 1024)); };
@@ -211,12 +244,21 @@ static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t 
     uint32_t sm_threads = srp ? 1024 : 2048;
     const bool both = !srp && ix->cw == 2;
     if (!tune || !tune->threads) {
+        const bool small = light && nq > 2 * uint32_t(sms);
         if (both && nq <= uint32_t(sms) * std::min(fit(), 2u)) {
             sm_threads = 1024;
-        } else if (nq > uint32_t(sms) * std::min(fit(), sm_threads / 512)) {
+        } else if (small || nq > uint32_t(sms) * std::min(fit(), sm_threads / 512)) {
             shape(256);
-            if (fit() >= 4) NT = 256;
-            else shape(512);
+            const uint32_t f256 = std::min(fit(), sm_threads / 256);
+            if (small && f256 >= 4 && nq > 4 * uint32_t(sms)) {
+                shape(128);
+                if (8 * std::min(fit(), sm_threads / 128) >= 11 * f256) NT = 128;
+                else shape(256);
+            }
+            if (NT == 512) {
+                if (f256 >= 4) NT = 256;
+                else shape(512);
+            }
         }
     }
     if (both && fit() * uint32_t(NT) <= 1024) sm_threads = 1024;
@@ -340,7 +382,10 @@ int counts_launch(flinng_index *ix, const uint32_t *qbuckets, uint32_t nq,
     return FLINNG_OK;
 }
 
-const void *plain_kernel_c1(int NT, uint32_t rw) { return plain_kernel_t<1>(NT, rw); }
+const void *plain_kernel_c1(int NT, uint32_t rw, uint32_t sm_threads)
+{
+    return plain_kernel_t<1>(NT, rw, sm_threads);
+}
 const void *fused_kernel_c1(int NT, uint32_t rw, bool srp, uint32_t sm_threads)
 {
     return fused_kernel_t<1>(NT, rw, srp, sm_threads);

@@ -5,7 +5,10 @@
 
 namespace flinng {
 
-const void *plain_kernel_c2(int NT, uint32_t rw) { return plain_kernel_t<2>(NT, rw); }
+const void *plain_kernel_c2(int NT, uint32_t rw, uint32_t sm_threads)
+{
+    return plain_kernel_t<2>(NT, rw, sm_threads);
+}
 const void *fused_kernel_c2(int NT, uint32_t rw, bool srp, uint32_t sm_threads)
 {
     return fused_kernel_t<2>(NT, rw, srp, sm_threads);

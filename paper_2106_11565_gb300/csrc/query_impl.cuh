@@ -40,8 +40,8 @@
 namespace flinng {
 
 constexpr int kQTmax = 256;              // CTA size of the counts kernel
-constexpr uint32_t kPlainThreads = 1024; // plain kernel: threads per SM its registers allow
 constexpr uint32_t kLevelCells = 2048;   // repetition-0 cells placed at a time, by level
+constexpr uint32_t kRankKeys = 256;      // compactions of at most this many keys rank them directly
 
 // key = (score_max - score) << 48 | lastcell << 32 | id
 template <int CW> struct CountWidth;
@@ -54,7 +54,7 @@ template <> struct CountWidth<2> {
     static constexpr uint64_t kKeyBits = (1ull << 60) - 1;
 };
 
-// cells per chunk of the walk, tables per chunk of the gather
+// cells per chunk of the walk, tables per round of the gather
 template <int NT> constexpr uint32_t kChunkCells = 2 * NT;
 constexpr uint32_t kWarpQueue = 64;      // filtered members a warp holds back (2 NT words in all)
 
@@ -77,7 +77,8 @@ struct QArgs {
     uint32_t gmax;     // up to this many
     uint32_t lcap;     // cells the level list holds
     uint32_t wide;     // 1: cells are large enough for the walk's filter (eight members per lane)
-    uint32_t avg_cell; // members per repetition-0 cell, rounded up (host side, sizes gcells)
+    uint32_t id_bits;  // bits of a point id
+    uint32_t avg_cell; // members per repetition-0 cell, rounded up
     uint32_t cap;      // candidate buffer entries (power of two)
     uint32_t kp;       // final sort width: power of two >= k_max
     uint32_t *out_ids;
@@ -92,7 +93,7 @@ struct QSmem {
     uint32_t *u;         // 8 scalars: nbuf, nkeep, digit / k-th score, rank / found, whole / count,
                          // heavy tables (gather) / cells of a big level (decode), bound (u[6..7])
     uint32_t *lvl_n;     // nlev: repetition-0 cells per count, then cells at levels >= v
-    uint32_t *shist;     // nlev: candidates in buf per score
+    uint32_t *shist;     // nlev: candidates in buf per score (score_hist)
     uint32_t *rhist;     // 256: radix histogram
     uint32_t *c_pre;     // kChunkCells + 4: exclusive prefix of unit counts, closed by ~0
     uint32_t *c_ms;      // kChunkCells: first member of each cell of a chunk; in the gather, first
@@ -223,14 +224,18 @@ __device__ inline uint32_t find_seg(const uint32_t *pre, uint32_t n, uint32_t j,
 // keys of a better score. Only the 48 bits below the score are searched.
 template <int NT, int CW>
 __device__ void block_select(const uint64_t *keys, uint32_t n, uint32_t kk, uint32_t score, uint32_t above,
-                             const QSmem &s, uint64_t &prefix_out, uint64_t &mask_out)
+                             uint32_t id_bits, const QSmem &s, uint64_t &prefix_out, uint64_t &mask_out)
 {
     const int tid = threadIdx.x, lane = tid & 31;
     uint64_t prefix = uint64_t(CountWidth<CW>::kScoreMax - score) << 48, mask = ~0ull << 48;
     uint32_t rem = kk - above;
+    for (int i = tid; i < 256; i += NT) s.rhist[i] = 0u;
+    __syncthreads();
     for (int shift = 40; shift >= 0; shift -= 8) {
-        for (int i = tid; i < 256; i += NT) s.rhist[i] = 0u;
-        __syncthreads();
+        if (shift < 32 && uint32_t(shift) >= id_bits) {     // all zeros
+            mask |= uint64_t(0xFF) << shift;
+            continue;
+        }
         // keys share their leading digits: aggregate per warp before the
         // shared-memory atomic (one per distinct digit per warp)
         for (uint32_t ib = tid & ~31u; ib < n; ib += NT) {
@@ -251,6 +256,7 @@ __device__ void block_select(const uint64_t *keys, uint32_t n, uint32_t kk, uint
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 h[j] = s.rhist[lane * 8 + j];
+                s.rhist[lane * 8 + j] = 0u;       // for the next digit
                 sum += h[j];
             }
             uint32_t incl = sum;
@@ -283,14 +289,38 @@ __device__ void block_select(const uint64_t *keys, uint32_t n, uint32_t kk, uint
         __syncthreads();
         const uint32_t d = s.u[2];
         rem = s.u[3];
-        const bool whole = s.u[4] != 0;
-        __syncthreads();
+        const bool whole = s.u[4] != 0;           // written again only after the next digit's barrier
         prefix |= uint64_t(d) << shift;
         mask |= uint64_t(0xFF) << shift;
         if (whole) break;
     }
+    __syncthreads();
     prefix_out = prefix;
     mask_out = mask;
+}
+
+// Candidates of buf[0..n) per score, of scores in [lo, hi] (the others are not
+// counted). Contains __syncthreads.
+template <int NT, int CW>
+__device__ void score_hist(const QSmem &s, uint32_t n, uint32_t lo, uint32_t hi)
+{
+    constexpr uint32_t kScoreMax = CountWidth<CW>::kScoreMax;
+    const uint32_t lane = threadIdx.x & 31;
+    for (uint32_t v = lo + threadIdx.x; v <= hi; v += NT) s.shist[v] = 0u;
+    __syncthreads();
+    for (uint32_t ib = threadIdx.x & ~31u; ib < n; ib += NT) {
+        const uint32_t i = ib + lane;
+        const uint32_t score = i < n ? kScoreMax - uint32_t(s.buf[i] >> 48) : 0u;
+        const bool in = i < n && score >= lo;
+        const uint32_t any = __ballot_sync(0xffffffffu, in);
+        if (!any) continue;
+        // candidates mostly tie: one addition for those that share the first one's score
+        const uint32_t lead = __ffs(any) - 1, first = __shfl_sync(0xffffffffu, score, lead);
+        const uint32_t same = __ballot_sync(0xffffffffu, in && score == first);
+        if (lane == lead) atomicAdd(&s.shist[first], __popc(same));
+        else if (in && score != first) atomicAdd(&s.shist[score], 1u);
+    }
+    __syncthreads();
 }
 
 // The kk-th best candidate's score, from the score histogram (scores in [lo,
@@ -334,8 +364,44 @@ __device__ inline bool kth_score_of(const QSmem &s, uint32_t lo, uint32_t hi, ui
     return found;
 }
 
+// The nk lowest of list[0..n) to keep[0..nk) in order: the keys are distinct, so
+// a key's rank is the number of smaller keys, counted by four lanes.
+template <int NT>
+__device__ __forceinline__ void rank_keys(const uint64_t *list, uint32_t n, uint32_t nk, uint64_t *keep)
+{
+    const uint32_t part = threadIdx.x & 3;
+    for (uint32_t ib = 0; ib < n; ib += NT / 4) {          // uniform: whole warps shuffle
+        const uint32_t i = ib + (threadIdx.x >> 2);
+        const uint64_t x = i < n ? list[i] : 0ull;
+        uint32_t r = 0;
+        for (uint32_t j = part; j < n; j += 4) r += list[j] < x ? 1u : 0u;
+        r += __shfl_xor_sync(0xffffffffu, r, 1);
+        r += __shfl_xor_sync(0xffffffffu, r, 2);
+        if (part == 0 && i < n && r < nk) keep[r] = x;
+    }
+}
+
+// The kk best of buf[0..nbuf), at most kRankKeys of them, to keep[0..kk) in order;
+// returns the kk-th. Contains __syncthreads.
+template <int NT>
+__device__ __forceinline__ uint64_t rank_keep(const QSmem &s, uint32_t nbuf, uint32_t kk)
+{
+    rank_keys<NT>(s.buf, nbuf, kk, s.keep);
+    __syncthreads();
+    return s.keep[kk - 1];
+}
+
+// buf[0..kk) = keep[0..kk). Contains __syncthreads.
+template <int NT>
+__device__ __forceinline__ void take_kept(const QSmem &s, uint32_t kk)
+{
+    for (uint32_t i = threadIdx.x; i < kk; i += NT) s.buf[i] = s.keep[i];
+    if (threadIdx.x == 0) s.u[0] = kk;
+    __syncthreads();
+}
+
 // Keep the kk best of buf[0..nbuf) in buf[0..kk); score: the kk-th best's, m:
-// candidates of at least it (kth_score_of). The histogram follows; returns
+// candidates of at least it (kth_score_of, whose histogram is read). Returns
 // the new admission bound: the largest kept key (later keys above it can never
 // enter the top kk).
 template <int NT, int CW>
@@ -344,8 +410,7 @@ __device__ uint64_t block_compact(const QArgs &a, const QSmem &s, uint32_t nbuf,
     const int lane = threadIdx.x & 31;
     const uint32_t above = m - s.shist[score];
     uint64_t prefix, mask;
-    block_select<NT, CW>(s.buf, nbuf, kk, score, above, s, prefix, mask);
-    for (uint32_t v = threadIdx.x; v <= score; v += NT) s.shist[v] = v < score ? 0u : kk - above;
+    block_select<NT, CW>(s.buf, nbuf, kk, score, above, a.id_bits, s, prefix, mask);
     if (threadIdx.x == 0) s.u[1] = 0u;
     __syncthreads();
     for (uint32_t ib = threadIdx.x & ~31u; ib < nbuf; ib += NT) {
@@ -428,7 +493,7 @@ __device__ __forceinline__ void planes_to_bytes(uint32_t (&pl)[8], uint32_t (&ou
     }
 }
 
-// Per-cell collision counts of one query (Sec. 5), 2 NT tables at a time (a
+// Per-cell collision counts of one query (Sec. 5), up to 2 NT tables at a time (a
 // thread's two offset pairs are in flight together).
 // Tables whose bucket is heavy contribute their cell bitmap: each thread owns
 // one bitmap word position (32 cells) and sums it over the heavy tables in
@@ -445,12 +510,15 @@ __device__ void gather_counts(const QArgs &a, const QSmem &s, const uint32_t *qb
     const int tid = threadIdx.x;
     constexpr uint32_t kTab = 2 * NT;
     for (uint32_t l0 = 0; l0 < a.L; l0 += kTab) {
+        // one table per thread while that covers them (32 tables on 16 threads
+        // took 600 cycles more than on 32)
+        const uint32_t nl = min(kTab, a.L - l0), tpt = nl <= uint32_t(NT) ? 1u : 2u;
         uint32_t o0[2] = {0u, 0u}, o1[2] = {0u, 0u}, units[2];
         uint64_t slot[2];
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const uint32_t l = l0 + tid * 2 + i;
-            if (l < a.L) {
+        for (uint32_t i = 0; i < 2; ++i) {
+            const uint32_t l = l0 + tid * tpt + i;
+            if (i < tpt && l < a.L) {
                 slot[i] = (uint64_t(l) << a.W) | qb[l];
                 o0[i] = a.off[slot[i]];
                 o1[i] = a.off[slot[i] + 1];
@@ -467,14 +535,15 @@ __device__ void gather_counts(const QArgs &a, const QSmem &s, const uint32_t *qb
             }
             units[i] = o1[i] > o0[i] ? ((o1[i] - 1) >> 3) - (o0[i] >> 3) + 1 : 0u;
         }
-        if (tid == 0) s.c_pre[kTab] = ~0u;   // ends every forward search of c_pre
+        if (tid == 0) s.c_pre[NT * tpt] = ~0u;   // ends every forward search of c_pre
         uint32_t total;
         const uint32_t pre = block_excl_scan<NT>(units[0] + units[1], s.wsum, &total);
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            s.c_pre[tid * 2 + i] = pre + (i ? units[0] : 0u);
-            s.c_ms[tid * 2 + i] = o0[i];
-            s.q_m[tid * 2 + i] = o1[i] - o0[i];
+        for (uint32_t i = 0; i < 2; ++i) {
+            if (i >= tpt) break;
+            s.c_pre[tid * tpt + i] = pre + (i ? units[0] : 0u);
+            s.c_ms[tid * tpt + i] = o0[i];
+            s.q_m[tid * tpt + i] = o1[i] - o0[i];
         }
         __syncthreads();
         const uint32_t nh = s.u[5];
@@ -510,7 +579,7 @@ __device__ void gather_counts(const QArgs &a, const QSmem &s, const uint32_t *qb
                             e = c;
                         }
                     }
-                    // back to packed counters; a pass adds at most 247 to a cell.
+                    // back to packed counters; a pass adds at most 248 to a cell.
                     // cntw is padded to whole 32-cell words (q_count_words).
                     uint32_t by[8];
                     planes_to_bytes(pl, by);
@@ -541,7 +610,6 @@ __device__ void gather_counts(const QArgs &a, const QSmem &s, const uint32_t *qb
             }
             __syncthreads();
         }
-        const uint32_t nl = min(kTab, a.L - l0);
         // each warp counts a contiguous slice of the flattened units, so a lane's
         // table index moves forward by a few tables per step (c_pre is total
         // past the last table and ~0 at the end, which ends the search)
@@ -624,7 +692,6 @@ __device__ inline void zero_query_state(const QArgs &a, const QSmem &s)
     const uint32_t nlev = q_nlev(a.L);
     for (uint32_t i = tid; i < nlev; i += NT) {
         s.lvl_n[i] = 0u;
-        s.shist[i] = 0u;
     }
     if (tid < 8) s.u[tid] = 0u;
 }
@@ -647,49 +714,177 @@ __device__ __forceinline__ void for_level_cells(const QArgs &a, const QSmem &s, 
     }
 }
 
-// The members of a chunk's cells (c_pre, c_ms; ncc cells whose ids are
-// cell_of[0..ncc), M units in all), decoded into candidate keys. A unit is
-// 2^VS consecutive members, aligned. VS = 3: a lane reads the repetition-1
-// groups of its unit's members with one 16-byte load and drops those whose
-// repetition-1 cell is below the admission bound; of the thousands of members
-// a query walks almost all go there, at 2 bytes and about five instructions
-// each instead of a record of 8 to 32 bytes and a key. Those that pass are
-// queued and decoded 32 at a time. VS = 0, for cells of a few members, or while
-// most would pass the filter: one member per lane, decoded at once.
-//
-// Candidates are appended without reservations: a warp reads the buffer fill
-// first and appends (at most 32 keys) only while it is at or below hwm. Above
-// it the warp pauses with its pending members; once every warp has paused or
-// finished, the block compacts and the warps resume. Once the fill passes hwm
-// every warp appends at most once more, so hwm = cap - (NT + 32) cannot overflow.
-template <int NT, int RW, int CW, int VS>
-__device__ void walk_members(const QArgs &a, const QSmem &s, const uint16_t *cell_of, uint32_t M, uint32_t ncc,
-                             uint32_t kq, uint32_t hi_level, uint64_t &bound, uint32_t &bscore)
+// Score of an admission bound: lower scores cannot enter (0 for kKeyBits).
+template <int CW>
+__device__ __forceinline__ uint32_t bound_score(uint64_t bound)
 {
-    constexpr uint32_t kScoreMax = CountWidth<CW>::kScoreMax;
+    return CountWidth<CW>::kScoreMax - uint32_t(bound >> 48);
+}
+
+// Room for n candidates in the buffer, for a warp (uniform): the first place, or
+// ~0 where the buffer is too full. There are no reservations: a warp reads the
+// fill first and appends at most 32 keys while it is at or below hwm. Once the
+// fill passes hwm every warp appends at most once more, so hwm = cap - (NT + 32)
+// cannot overflow.
+__device__ __forceinline__ uint32_t append_at(const QSmem &s, uint32_t n, uint32_t hwm)
+{
+    uint32_t at = kEmpty32;
+    if ((threadIdx.x & 31) == 0 && *reinterpret_cast<volatile uint32_t *>(&s.u[0]) <= hwm) at = atomicAdd(&s.u[0], n);
+    return __shfl_sync(0xffffffffu, at, 0);
+}
+
+// Key of the member with record w in repetition-0 cell `cell`; kKeyNone if its
+// score is below smin. No branches: the walk's lanes stay together.
+template <int RW, int CW>
+__device__ __forceinline__ uint64_t member_key(const QArgs &a, const QSmem &s, const uint32_t (&w)[RW], uint32_t cell,
+                                               uint32_t smin)
+{
+    uint32_t score = cnt_at<CW>(s, cell), last = cell;       // repetition 0: the cell itself, at its level
+#pragma unroll
+    for (int r = 1; r < 2 * RW - 1; ++r) {
+        if (r >= int(a.R)) break;
+        const uint32_t g = (w[1 + (r - 1) / 2] >> (16 * ((r - 1) & 1))) & 0xFFFFu;
+        const uint32_t c = uint32_t(r) * a.B + g;
+        const uint32_t v = cnt_at<CW>(s, c);
+        last = v <= score ? c : last;
+        score = min(score, v);
+    }
+    const uint64_t key = (uint64_t(CountWidth<CW>::kScoreMax - score) << 48) | (uint64_t(last) << 32) | w[0];
+    return score >= smin ? key : kKeyNone;
+}
+
+// The walk's end: true if every warp reached its slice's end; else (a warp paused
+// at the buffer's mark) the block compacts and the warps resume.
+template <int NT, int CW>
+__device__ __forceinline__ bool walk_done(const QArgs &a, const QSmem &s, uint32_t kq, uint32_t hwm, uint32_t smin,
+                                          uint32_t hi_level, uint64_t &bound)
+{
+    __syncthreads();
+    const uint32_t nb0 = s.u[0];   // same value in every thread (read after the barrier)
+    if (nb0 <= hwm) return true;
+    if (nb0 <= kRankKeys) {
+        bound = rank_keep<NT>(s, nb0, kq);              // hwm >= kq: there are kq
+        take_kept<NT>(s, kq);
+    } else {
+        uint32_t score, n;
+        score_hist<NT, CW>(s, nb0, smin, hi_level);
+        kth_score_of(s, smin, hi_level, kq, &score, &n);
+        bound = block_compact<NT, CW>(a, s, nb0, kq, score, n);
+    }
+    return false;
+}
+
+// The members of a chunk's cells (c_pre, c_ms; ncc cells whose ids are
+// cell_of[0..ncc), M members in all), decoded into candidate keys, every record
+// read: U members per lane and step, their loads in flight together. Each warp
+// walks its own contiguous slice, so its cell index only moves forward.
+template <int NT, int RW, int CW, int U>
+__device__ void walk_all(const QArgs &a, const QSmem &s, const uint16_t *cell_of, uint32_t M, uint32_t ncc, uint32_t kq,
+                         uint32_t hi_level, uint64_t &bound)
+{
     const int tid = threadIdx.x, lane = tid & 31;
-    // Each warp walks its own contiguous slice of the units, 32 at a time, so
-    // its cell index only moves forward. Few units are still spread over all
-    // warps, since each warp's chain of loads is what a small chunk waits for.
-    const uint32_t per = ((M + NT / 32 - 1) / (NT / 32) + 7) & ~7u;
+    const uint32_t per = ((M + NT / 32 - 1) / (NT / 32) + 31) & ~31u;
     uint32_t jb = min(uint32_t(tid >> 5) * per, M);   // this warp's cursor (warp-uniform)
     const uint32_t je = min(jb + per, M);
-    // the cell holding unit jb (warp-uniform; the largest such index is never an empty cell)
+    // the cell holding member jb (warp-uniform; the largest such index is never an empty cell)
+    uint32_t cur = jb < je ? find_seg(s.c_pre, ncc, jb) : 0u;
+    const uint32_t hwm = a.cap - uint32_t(NT + 32);
+    for (;;) {
+        const uint32_t smin = max(a.t_min, bound_score<CW>(bound));
+        while (jb < je) {
+            // lanes to cells: one warp-uniform pass over the cell boundaries
+            // inside this step; c_pre is M past the chunk's last cell and ~0 at
+            // the array's end, so the pass stops at the step's last member
+            const uint32_t last_j = min(jb + 32u * U, je) - 1u;
+            uint32_t my[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) my[u] = cur;
+            uint32_t k = cur + 1, bnd = s.c_pre[k];
+            while (bnd <= last_j) {
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (jb + uint32_t(u) * 32 + lane >= bnd) my[u] = k;
+                bnd = s.c_pre[++k];
+            }
+            uint32_t w[U][RW], cell[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t j = jb + uint32_t(u) * 32 + lane;
+                cell[u] = 0;
+#pragma unroll
+                for (int i = 0; i < RW; ++i) w[u][i] = 0u;
+                if (j < je) {
+                    cell[u] = cell_of[my[u]];
+                    load_record<RW>(a.mrec, s.c_ms[my[u]] + (j - s.c_pre[my[u]]), w[u]);
+                }
+            }
+            // the keys are made again for the few that are wanted, rather than held
+            // (one member per lane, in flight: 125 us with the key held, 110 so)
+            const uint32_t below = (1u << lane) - 1u;
+            uint32_t wm[U], total = 0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint64_t key = member_key<RW, CW>(a, s, w[u], cell[u], smin);
+                wm[u] = __ballot_sync(0xffffffffu, jb + uint32_t(u) * 32 + lane < je && key <= bound);
+                total += __popc(wm[u]);
+            }
+            int did = U;
+            if (total) {
+                // in one go where they are at most 32
+                uint32_t at = total <= 32u ? append_at(s, total, hwm) : 0u;
+                if (at == kEmpty32) did = 0;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (u >= did || !wm[u]) continue;
+                    if (total > 32u) at = append_at(s, __popc(wm[u]), hwm);
+                    if (at == kEmpty32) {
+                        did = u;
+                        continue;
+                    }
+                    if ((wm[u] >> lane) & 1u)
+                        s.buf[at + __popc(wm[u] & below)] = member_key<RW, CW>(a, s, w[u], cell[u], smin);
+                    at += __popc(wm[u]);
+                }
+            }
+            if (did < U) {                     // paused: the step's rest after the compaction
+                jb += 32u * did;
+                if (did && jb < je) cur = find_seg(s.c_pre, ncc, jb);
+                break;
+            }
+            jb += 32 * U;
+            cur = k - 1;                       // the cell holding member last_j
+        }
+        if (walk_done<NT, CW>(a, s, kq, hwm, smin, hi_level, bound)) return;
+    }
+}
+
+// The same through the repetition-1 groups: a unit is eight consecutive members,
+// aligned. A lane reads the repetition-1 groups of its unit's members with one
+// 16-byte load and drops those whose repetition-1 cell is below the admission
+// bound; of the thousands of members a query walks almost all go there, at 2
+// bytes and about five instructions each instead of a record of 8 to 32 bytes
+// and a key. Those that pass are queued and decoded 32 at a time. M: units.
+template <int NT, int RW, int CW>
+__device__ void walk_filtered(const QArgs &a, const QSmem &s, const uint16_t *cell_of, uint32_t M, uint32_t ncc,
+                              uint32_t kq, uint32_t hi_level, uint64_t &bound)
+{
+    const int tid = threadIdx.x, lane = tid & 31;
+    // Few units are still spread over all warps, since each warp's chain of
+    // loads is what a small chunk waits for.
+    const uint32_t per = ((M + NT / 32 - 1) / (NT / 32) + 7) & ~7u;
+    uint32_t jb = min(uint32_t(tid >> 5) * per, M);
+    const uint32_t je = min(jb + per, M);
     uint32_t cur = jb < je ? find_seg(s.c_pre, ncc, jb) : 0u;
     const uint32_t hwm = a.cap - uint32_t(NT + 32);
     uint32_t *qm = s.q_m + (tid >> 5) * kWarpQueue;
     uint16_t *qc = s.q_c + (tid >> 5) * kWarpQueue;
     uint32_t qn = 0;                             // queued members (warp-uniform)
-    uint32_t pend = 0u, m0 = 0u, my_cell = 0u;   // this lane's members m0 + bit to decode at once
+    uint32_t pend = 0u, m0 = 0u, my_cell = 0u;   // this lane's members m0 + bit still to queue
     for (;;) {
-        const uint32_t smin = max(a.t_min, bscore);   // lower scores cannot enter
+        const uint32_t smin = max(a.t_min, bound_score<CW>(bound));
         for (;;) {
             const bool more = __any_sync(0xffffffffu, pend != 0u);
-            const bool dense = VS == 0 && more;
             if (!more && qn < 32u && jb < je) {
-                // lanes to cells: one warp-uniform pass over the cell boundaries
-                // inside this step; c_pre is M past the chunk's last cell and ~0 at
-                // the array's end, so the pass stops at the step's last unit
                 const uint32_t last_j = min(jb + 32u, je) - 1u, j = jb + lane;
                 uint32_t my = cur, k = cur + 1, bnd = s.c_pre[k];
                 while (bnd <= last_j) {
@@ -700,32 +895,24 @@ __device__ void walk_members(const QArgs &a, const QSmem &s, const uint16_t *cel
                 jb += 32;
                 if (j < je) {
                     const uint32_t ms = s.c_ms[my];
-                    const uint32_t u = (ms >> VS) + (j - s.c_pre[my]);
+                    const uint32_t u = (ms >> 3) + (j - s.c_pre[my]);
                     my_cell = cell_of[my];
-                    m0 = u << VS;
-                    if constexpr (VS == 0) {
-                        pend = 1u;
-                    } else {
-                        // members of neighbouring cells and the zeroed padding share
-                        // the unit: valid group ids, masked out
-                        const uint32_t me = __ldg(a.moff + my_cell + 1);
-                        const uint4 g = __ldg(reinterpret_cast<const uint4 *>(a.mg1) + u);
-                        const uint32_t lo = ms > m0 ? ms - m0 : 0u, hi = min(me - m0, 8u);
-                        pend = ((1u << hi) - 1u) & ~((1u << lo) - 1u);
-                        if constexpr (RW > 1) {
-                            const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
-                            uint32_t ok = 0u;
+                    m0 = u << 3;
+                    // members of neighbouring cells and the zeroed padding share
+                    // the unit: valid group ids, masked out
+                    const uint32_t me = __ldg(a.moff + my_cell + 1);
+                    const uint4 g = __ldg(reinterpret_cast<const uint4 *>(a.mg1) + u);
+                    const uint32_t lo = ms > m0 ? ms - m0 : 0u, hi = min(me - m0, 8u);
+                    pend = ((1u << hi) - 1u) & ~((1u << lo) - 1u);
+                    const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
+                    uint32_t ok = 0u;
 #pragma unroll
-                            for (int i = 0; i < 8; ++i)
-                                ok |= (cnt_at<CW>(s, a.B + ((gw[i / 2] >> (16 * (i & 1))) & 0xFFFFu)) >= smin ? 1u : 0u)
-                                      << i;
-                            pend &= ok;
-                        }
-                    }
+                    for (int i = 0; i < 8; ++i)
+                        ok |= (cnt_at<CW>(s, a.B + ((gw[i / 2] >> (16 * (i & 1))) & 0xFFFFu)) >= smin ? 1u : 0u) << i;
+                    pend &= ok;
                 }
-                if constexpr (VS == 0) continue;
             }
-            if (VS == 3 && qn < 32u && __any_sync(0xffffffffu, pend != 0u)) {
+            if (qn < 32u && __any_sync(0xffffffffu, pend != 0u)) {
                 // the members that passed go to the queue, as many as fit; the
                 // others wait in pend, so that 32 are always decoded together
                 const uint32_t np = __popc(pend);
@@ -744,92 +931,49 @@ __device__ void walk_members(const QArgs &a, const QSmem &s, const uint16_t *cel
                 __syncwarp();
                 continue;
             }
-            if (VS == 3 && qn < 32u && jb < je) continue;      // nothing passed: the next step
-            // decode one member per lane: the step's (VS = 0), or the queue's last
-            uint32_t m = 0, last = 0, qb = 0;
-            bool has;
-            if (dense) {
-                has = pend != 0u;
-                m = m0 + __ffs(pend) - 1;
-                last = my_cell;
-            } else {
-                if (qn == 0u) break;
-                qb = qn > 32u ? qn - 32u : 0u;
-                has = qb + lane < qn;
-                if (has) {
-                    m = qm[qb + lane];
-                    last = qc[qb + lane];
-                }
-            }
-            bool want = false;
-            uint64_t key = 0;
-            if (has) {
-                uint32_t w[RW];
-                load_record<RW>(a.mrec, m, w);
-                uint32_t score = cnt_at<CW>(s, last);    // repetition 0: the cell itself, at its level
+            if (qn < 32u && jb < je) continue;      // nothing passed: the next step
+            if (qn == 0u) break;
+            // the queue's last members, one per lane
+            const uint32_t qb = qn > 32u ? qn - 32u : 0u;
+            const bool has = qb + lane < qn;
+            uint32_t w[RW], cell = 0;
 #pragma unroll
-                for (int r = 1; r < 2 * RW - 1; ++r) {
-                    if (r >= int(a.R)) break;
-                    const uint32_t g = (w[1 + (r - 1) / 2] >> (16 * ((r - 1) & 1))) & 0xFFFFu;
-                    const uint32_t c = uint32_t(r) * a.B + g;
-                    const uint32_t v = cnt_at<CW>(s, c);
-                    if (v <= score) {
-                        last = c;
-                        score = v;
-                    }
-                }
-                if (score >= smin) {
-                    key = (uint64_t(kScoreMax - score) << 48) | (uint64_t(last) << 32) | w[0];
-                    want = key <= bound;
-                }
+            for (int i = 0; i < RW; ++i) w[i] = 0u;
+            if (has) {
+                cell = qc[qb + lane];
+                load_record<RW>(a.mrec, qm[qb + lane], w);
             }
+            const uint64_t key = member_key<RW, CW>(a, s, w, cell, smin);
+            const bool want = has && key <= bound;
             const uint32_t wm = __ballot_sync(0xffffffffu, want);
             if (wm) {
-                // the fill, read once per warp (lane 0) so the decision is warp-uniform
-                uint32_t fill = lane == 0 ? *reinterpret_cast<volatile uint32_t *>(&s.u[0]) : 0u;
-                fill = __shfl_sync(0xffffffffu, fill, 0);
-                if (fill > hwm) break;
-                uint32_t base = 0;
-                if (lane == __ffs(wm) - 1) base = atomicAdd(&s.u[0], __popc(wm));
-                base = __shfl_sync(0xffffffffu, base, __ffs(wm) - 1);
-                if (want) {
-                    s.buf[base + __popc(wm & ((1u << lane) - 1u))] = key;
-                    atomicAdd(&s.shist[kScoreMax - uint32_t(key >> 48)], 1u);
-                }
+                const uint32_t at = append_at(s, __popc(wm), hwm);
+                if (at == kEmpty32) break;
+                if (want) s.buf[at + __popc(wm & ((1u << lane) - 1u))] = key;
             }
-            if (dense) {
-                pend &= pend - 1u;
-            } else {
-                qn = qb;
-                __syncwarp();              // entries read before they are written again
-            }
+            qn = qb;
+            __syncwarp();              // entries read before they are written again
         }
-        __syncthreads();
-        const uint32_t nb0 = s.u[0];   // same value in every thread (read after the barrier)
-        if (nb0 <= hwm) break;          // no warp paused: every cursor is at its end
-        uint32_t score, n;
-        kth_score_of(s, smin, hi_level, kq, &score, &n);    // hwm >= kq: there are kq
-        bound = block_compact<NT, CW>(a, s, nb0, kq, score, n);
-        bscore = score;
+        if (walk_done<NT, CW>(a, s, kq, hwm, smin, hi_level, bound)) return;
     }
 }
 
 // Group tests, AND-over-R decode and top-k of query q, from the counts in
 // shared memory; writes row q of the outputs.
-template <int NT, int RW, int CW>
+template <int NT, int RW, int CW, int U>
 __device__ void decode_topk(const QArgs &a, const QSmem &s, uint32_t q, uint32_t kq)
 {
     constexpr uint32_t kScoreMax = CountWidth<CW>::kScoreMax;
-    constexpr uint32_t kCh = kChunkCells<NT>;
     const int tid = threadIdx.x, lane = tid & 31;
-    bool have_k = false;                 // kq candidates held at the last check
-    uint32_t kth_score = 0, kth_n = 0;   // score of the kq-th best then, candidates of at least it
+    bool in_order = false;               // keep holds the kq best, in order
+    uint32_t kth_score = 0, kth_n = 0;   // score of the kq-th best at the last check, candidates of at least it
     if (kq > 0) {
         // group tests of repetition 0: cells per count level
         for_level_cells<NT, CW>(a, s, a.t_min, [&](uint32_t, uint32_t v) { atomicAdd(&s.lvl_n[v], 1u); });
         __syncthreads();
-        // lvl_n[v] becomes the number of cells at levels >= v: thread i takes the
-        // i-th run of consecutive levels from L down to t_min
+        // lvl_n[v] becomes the number of cells at levels >= v, lvl_cur[v] those at
+        // levels above v: thread i takes the i-th run of consecutive levels from L
+        // down to t_min
         {
             const uint32_t nl = a.L - a.t_min + 1, per = (nl + NT - 1) / NT;
             uint32_t local = 0;
@@ -841,6 +985,7 @@ __device__ void decode_topk(const QArgs &a, const QSmem &s, uint32_t q, uint32_t
             for (uint32_t i = 0; i < per; ++i) {
                 const uint32_t pos = uint32_t(tid) * per + i;
                 if (pos < nl) {
+                    s.lvl_cur[a.L - pos] = run;
                     run += s.lvl_n[a.L - pos];
                     s.lvl_n[a.L - pos] = run;
                 }
@@ -851,7 +996,6 @@ __device__ void decode_topk(const QArgs &a, const QSmem &s, uint32_t q, uint32_t
         // been seen (its repetition-0 cell has count >= t), so the walk stops
         // once the kq-th best candidate scores >= t: no later point can enter.
         uint64_t bound = CountWidth<CW>::kKeyBits;   // admission: key <= bound
-        uint32_t bscore = 0;                 // the bound's score: lower scores cannot enter
         // Levels are placed in the level list a segment at a time: as many whole
         // levels, from t down, as the list holds (most queries stop within the
         // first segment, so the list need not hold all B cells and the lower
@@ -872,10 +1016,18 @@ __device__ void decode_topk(const QArgs &a, const QSmem &s, uint32_t q, uint32_t
             return lo;
         };
         int t = int(a.L);
-        if (s.lvl_n[t] == 0u) t = extent(int(a.t_min), t, 0u) - 1;   // the highest level with a cell
+        // the highest level with a cell, where the levels are many
+        if (a.L > 64u && s.lvl_n[t] == 0u) t = extent(int(a.t_min), t, 0u) - 1;
         const uint32_t hi_level = uint32_t(t);                       // no point scores more
         int seg_lo = t + 1;
         uint32_t seg_base = 0, glim = a.gcells;
+        // the first group is four times as large where k is large and an early bound
+        // helps little: the filter drops most members without one, or the walk that
+        // reads all records has several in flight and, with few tables, scores mostly
+        // tie (60,000 reads in 128 tables, 600 queries, k = 100: 68 us with the small
+        // group, 53 with the large one; 512 tables, two shards: 64 and 73; 2,000
+        // embeddings in 64 tables, k = 10: 131 and 158)
+        if (kq >= 32u && ((U > 1 && a.R > 1 && a.L < 256u) || (a.wide && all * 2u < a.B))) glim = min(glim * 4u, a.gmax);
         while (t >= int(a.t_min)) {
             const uint32_t above = t < int(a.L) ? s.lvl_n[t + 1] : 0u;   // cells at levels above t
             if (above == all) break;                                     // none left
@@ -883,17 +1035,18 @@ __device__ void decode_topk(const QArgs &a, const QSmem &s, uint32_t q, uint32_t
             int t_end = t;
             if (!big) {
                 if (t < seg_lo) {
-                    seg_lo = extent(int(a.t_min), t, above + a.lcap);
+                    seg_lo = all - above <= a.lcap ? int(a.t_min) : extent(int(a.t_min), t, above + a.lcap);
                     seg_base = above;
-                    for (int v = seg_lo + tid; v <= t; v += NT)
-                        s.lvl_cur[v] = (v < int(a.L) ? s.lvl_n[v + 1] : 0u) - seg_base;
-                    __syncthreads();
+                    if (above) {                   // nothing walked yet: lvl_cur is there already, t < L otherwise
+                        for (int v = seg_lo + tid; v <= t; v += NT) s.lvl_cur[v] = s.lvl_n[v + 1] - seg_base;
+                        __syncthreads();
+                    }
                     for_level_cells<NT, CW>(a, s, uint32_t(seg_lo), [&](uint32_t b, uint32_t v) {
                         if (v <= uint32_t(t)) s.lvl_cells[atomicAdd(&s.lvl_cur[v], 1u)] = uint16_t(b);
                     });
                     __syncthreads();
                 }
-                t_end = extent(seg_lo, t, above + glim);
+                t_end = all - above <= glim ? seg_lo : extent(seg_lo, t, above + glim);
             }
             // a group's cells, in one part or, for a big level, in ranges of cell ids
             for (uint32_t b0 = 0; b0 < (big ? a.B : 1u); b0 += a.lcap) {
@@ -901,7 +1054,7 @@ __device__ void decode_topk(const QArgs &a, const QSmem &s, uint32_t q, uint32_t
                 if (big) {
                     // a cursor of its own (u[5], free here): the words of lvl_cur are
                     // those of c_pre, which is written below as soon as the count is
-                    // read, and t = kCh would be its closing word
+                    // read, its closing word ahead of a barrier
                     first = 0;
                     if (tid == 0) s.u[5] = 0u;
                     __syncthreads();
@@ -911,67 +1064,80 @@ __device__ void decode_topk(const QArgs &a, const QSmem &s, uint32_t q, uint32_t
                     nc = s.u[5];
                     __syncthreads();        // read by all before the next range's zero
                 }
-                // the filter pays while fewer than half the members pass it: about the
-                // share of cells that reach the admission bound (any repetition's counts
-                // are alike). 1,528 queries of 568,482 URL sets in 17 tables, whose
-                // scores mostly tie: 378 us, 500 with the line at a quarter
-                const bool wide = a.wide && s.lvl_n[max(a.t_min, bscore)] * 2u < a.B;
-                for (uint32_t c0 = 0; c0 < nc; c0 += kCh) {
-                    constexpr uint32_t kPer = kCh / NT;
-                    uint32_t ms[kPer], units[kPer], mine = 0;
+                // the filter pays while fewer than half the members pass it (a quarter
+                // where the other walk has two records in flight): about the share of
+                // cells that reach the admission bound (any repetition's counts are
+                // alike). 1,528 queries of 568,482 URL sets in 17 tables, whose scores
+                // mostly tie, one record in flight: 378 us, 500 with the line at a
+                // quarter. It has a second load in its chain, so a chunk that the other
+                // walk reads in two steps goes there.
+                const bool wide = a.wide && s.lvl_n[max(a.t_min, bound_score<CW>(bound))] * 2u * U < a.B &&
+                                  min(nc, uint32_t(2 * NT)) * a.avg_cell > 2u * U * NT;
+                // cells per thread: two where there are more than one for each, since cells
+                // of a few members make small chunks
+                const uint32_t per = nc <= uint32_t(NT) ? 1u : 2u;
+                for (uint32_t c0 = 0; c0 < nc; c0 += 2 * NT) {
+                    uint32_t ms[2], units[2];
 #pragma unroll
-                    for (uint32_t i = 0; i < kPer; ++i) {
-                        const uint32_t ci = c0 + tid * kPer + i;
+                    for (uint32_t i = 0; i < 2; ++i) {
+                        const uint32_t ci = c0 + tid * per + i;
                         ms[i] = units[i] = 0;
-                        if (ci < nc) {
+                        if (i < per && ci < nc) {
                             const uint32_t b = s.lvl_cells[first + ci];
                             // a member's score is at most its repetition-0 cell's level:
                             // members of cells below the bound's score cannot enter
-                            if (cnt_at<CW>(s, b) >= bscore) {
+                            if (cnt_at<CW>(s, b) >= bound_score<CW>(bound)) {
                                 ms[i] = a.moff[b];
                                 units[i] = a.moff[b + 1];
                             }
                         }
                     }
 #pragma unroll
-                    for (uint32_t i = 0; i < kPer; ++i) {
+                    for (uint32_t i = 0; i < 2; ++i) {
                         const uint32_t me = units[i];
                         units[i] = me - ms[i];
                         if (wide && units[i]) units[i] = ((me - 1) >> 3) - (ms[i] >> 3) + 1;
-                        mine += units[i];
                     }
-                    if (tid == 0) s.c_pre[kCh] = ~0u;   // ends every forward search of c_pre
+                    if (tid == 0) s.c_pre[NT * per] = ~0u;   // ends every forward search of c_pre
                     uint32_t M;
-                    uint32_t pre = block_excl_scan<NT>(mine, s.wsum, &M);
-#pragma unroll
-                    for (uint32_t i = 0; i < kPer; ++i) {
-                        s.c_pre[tid * kPer + i] = pre;
-                        s.c_ms[tid * kPer + i] = ms[i];
-                        pre += units[i];
+                    const uint32_t pre = block_excl_scan<NT>(units[0] + units[1], s.wsum, &M);
+                    s.c_pre[tid * per] = pre;
+                    s.c_ms[tid * per] = ms[0];
+                    if (per == 2) {
+                        s.c_pre[tid * 2 + 1] = pre + units[0];
+                        s.c_ms[tid * 2 + 1] = ms[1];
                     }
-                    const uint32_t ncc = min(kCh, nc - c0);
+                    const uint32_t ncc = min(uint32_t(2 * NT), nc - c0);
                     __syncthreads();
                     const uint16_t *cell_of = s.lvl_cells + first + c0;
-                    if (wide) walk_members<NT, RW, CW, 3>(a, s, cell_of, M, ncc, kq, hi_level, bound, bscore);
-                    else walk_members<NT, RW, CW, 0>(a, s, cell_of, M, ncc, kq, hi_level, bound, bscore);
+                    if (wide) walk_filtered<NT, RW, CW>(a, s, cell_of, M, ncc, kq, hi_level, bound);
+                    else walk_all<NT, RW, CW, U>(a, s, cell_of, M, ncc, kq, hi_level, bound);
                 }
             }
-            // the buffer fill and the histogram are final after the walk's last
-            // barrier (no cells: as at the last check)
+            // the buffer's fill is final after the walk's last barrier (no cells: as at
+            // the last check); every level >= t_end is complete, so points of score >=
+            // t_end are all seen
             const uint32_t nb = s.u[0];
-            if (nb >= kq && kth_score_of(s, max(a.t_min, bscore), hi_level, kq, &kth_score, &kth_n)) {
-                have_k = true;
+            if (nb >= kq && nb <= kRankKeys) {
+                bound = rank_keep<NT>(s, nb, kq);
+                kth_score = bound_score<CW>(bound);
+                if (kth_score >= uint32_t(t_end) || s.lvl_n[t_end] == all) {
+                    in_order = true;
+                    break;
+                }
+                if (nb != kq) take_kept<NT>(s, kq);
+            } else if (nb >= kq) {
+                const uint32_t lo = max(a.t_min, bound_score<CW>(bound));
+                score_hist<NT, CW>(s, nb, lo, hi_level);
+                kth_score_of(s, lo, hi_level, kq, &kth_score, &kth_n);
                 if (kth_n > max(2 * kq, 64u)) {
                     // many candidates tie: bound by the kq-th key, not by its score
                     bound = block_compact<NT, CW>(a, s, nb, kq, kth_score, kth_n);
-                    kth_n = kq;
-                } else if (kth_score > bscore) {
+                } else if (kth_score > bound_score<CW>(bound)) {
                     bound = (uint64_t(kScoreMax - kth_score) << 48) | 0xFFFFFFFFFFFFull;
                 }
-                bscore = kth_score;
+                if (kth_score >= uint32_t(t_end)) break;
             }
-            // every level >= t_end is complete: points of score >= t_end are all seen
-            if (have_k && kth_score >= uint32_t(t_end)) break;
             t = t_end - 1;
             glim = min(glim * 2, a.gmax);
         }
@@ -981,7 +1147,7 @@ __device__ void decode_topk(const QArgs &a, const QSmem &s, uint32_t q, uint32_t
     uint32_t nbuf = s.u[0];
     const uint32_t nk = nbuf < kq ? nbuf : kq;
     uint64_t *list = s.buf;
-    if (nbuf > kq) {
+    if (!in_order && nbuf > kq) {
         // the last check saw every candidate
         if (kth_n <= min(256u, uint32_t(NT))) {
             // those of at least the kq-th score are few more than kq: collected
@@ -1008,19 +1174,9 @@ __device__ void decode_topk(const QArgs &a, const QSmem &s, uint32_t q, uint32_t
             nbuf = kq;
         }
     }
-    if (nbuf <= uint32_t(NT)) {
-        // rank sort: the keys are distinct, so a key's rank is the number of
-        // smaller keys, counted by four lanes; ranks of kq and above are cut
-        const uint32_t part = lane & 3;
-        for (uint32_t ib = 0; ib < nbuf; ib += NT / 4) {       // uniform: whole warps shuffle
-            const uint32_t i = ib + (tid >> 2);
-            const uint64_t x = i < nbuf ? list[i] : 0ull;
-            uint32_t r = 0;
-            for (uint32_t j = part; j < nbuf; j += 4) r += list[j] < x ? 1u : 0u;
-            r += __shfl_xor_sync(0xffffffffu, r, 1);
-            r += __shfl_xor_sync(0xffffffffu, r, 2);
-            if (part == 0 && i < nbuf && r < nk) s.keep[r] = x;
-        }
+    if (in_order) {
+    } else if (nbuf <= uint32_t(NT)) {
+        rank_keys<NT>(list, nbuf, nk, s.keep);
         __syncthreads();
     } else {
         for (uint32_t i = tid; i < a.kp; i += NT) s.keep[i] = (i < nk) ? s.buf[i] : kKeyNone;
@@ -1053,8 +1209,9 @@ __device__ void decode_topk(const QArgs &a, const QSmem &s, uint32_t q, uint32_t
     __syncthreads();
 }
 
-template <int NT, int RW, int CW>
-__global__ void __launch_bounds__(NT, kPlainThreads / NT)
+// FT: threads per SM that its registers allow.
+template <int NT, int RW, int CW, int FT>
+__global__ void __launch_bounds__(NT, FT / NT)
 k_query(QArgs a)
 {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -1068,7 +1225,7 @@ k_query(QArgs a)
             if (a.cnt_in) load_counts<NT, CW>(a, s, a.cnt_in + size_t(q) * a.BR);
             else gather_counts<NT, CW>(a, s, a.qb + size_t(q) * a.L);
         }
-        decode_topk<NT, RW, CW>(a, s, q, kq);
+        decode_topk<NT, RW, CW, FT == 1024 ? 2 : 1>(a, s, q, kq);
     }
 }
 
@@ -1279,7 +1436,7 @@ k_query_fused(QArgs a, HArgs h)
         } else {
             __syncthreads();
         }
-        decode_topk<NT, RW, CW>(a, s, q, kq);
+        decode_topk<NT, RW, CW, HASH == 1 && FT == 1024 ? 2 : 1>(a, s, q, kq);
         if (!h.qnext) break;
     }
 }
@@ -1288,7 +1445,7 @@ k_query_fused(QArgs a, HArgs h)
 // tables, 12,288 cells, 512 queries: 20.7 us with 2-byte stores; two shards'
 // counts, their sum and the decode 67.6 us, 62.8 with eight counts per access).
 template <int CW>
-__global__ void __launch_bounds__(kQTmax)
+__global__ void __launch_bounds__(kQTmax, 2048 / kQTmax)
 k_counts(QArgs a)
 {
     constexpr int NT = kQTmax;
@@ -1324,18 +1481,19 @@ k_counts(QArgs a)
 
 // Kernel entry points of one count width, by CTA size and record width.
 template <int CW>
-const void *plain_kernel_t(int NT, uint32_t rw)
+const void *plain_kernel_t(int NT, uint32_t rw, uint32_t sm_threads)
 {
-#define FL_PLAIN(N) \
+#define FL_PLAIN(N, FT) \
     switch (rw) { \
-    case 1: return (const void *)k_query<N, 1, CW>; \
-    case 2: return (const void *)k_query<N, 2, CW>; \
-    case 4: return (const void *)k_query<N, 4, CW>; \
-    default: return (const void *)k_query<N, 8, CW>; \
+    case 1: return (const void *)k_query<N, 1, CW, FT>; \
+    case 2: return (const void *)k_query<N, 2, CW, FT>; \
+    case 4: return (const void *)k_query<N, 4, CW, FT>; \
+    default: return (const void *)k_query<N, 8, CW, FT>; \
     }
-    if (NT == 1024) { FL_PLAIN(1024) }
-    if (NT == 512) { FL_PLAIN(512) }
-    FL_PLAIN(256)
+    if (NT == 1024) { FL_PLAIN(1024, 1024) }
+    if (NT == 512) { FL_PLAIN(512, 1024) }
+    if (sm_threads == 2048) { FL_PLAIN(256, 2048) }
+    FL_PLAIN(256, 1024)
 #undef FL_PLAIN
 }
 
@@ -1369,10 +1527,10 @@ const void *fused_kernel_t(int NT, uint32_t rw, bool srp, uint32_t sm_threads)
 
 // Per count width: the plain, fused and counts kernels (query.cu: CW = 1,
 // query_c16.cu: CW = 2).
-const void *plain_kernel_c1(int NT, uint32_t rw);
+const void *plain_kernel_c1(int NT, uint32_t rw, uint32_t sm_threads);
 const void *fused_kernel_c1(int NT, uint32_t rw, bool srp, uint32_t sm_threads);
 const void *counts_kernel_c1();
-const void *plain_kernel_c2(int NT, uint32_t rw);
+const void *plain_kernel_c2(int NT, uint32_t rw, uint32_t sm_threads);
 const void *fused_kernel_c2(int NT, uint32_t rw, bool srp, uint32_t sm_threads);
 const void *counts_kernel_c2();
 
