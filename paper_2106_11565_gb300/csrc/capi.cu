@@ -576,6 +576,10 @@ int flinng_tune_query(flinng_index *idx, const flinng_points *q, uint32_t nq, ui
     }
     if (k_max > kMaxKMax) return set_error(FLINNG_ERR_INVALID_ARG, "tune: k_max > %u", kMaxKMax);
     FL_TRY(check_points(idx, q, nq, on_device));
+    if (!query_fused_fits(idx, k_max)) {
+        if (chosen) chosen[0] = chosen[1] = chosen[2] = 0;
+        return FLINNG_OK;
+    }
     const cudaStream_t st = idx->stream;
     const size_t need = 4096 + stage_bytes(idx, q, nq, on_device) + carve_bytes<uint32_t>(uint64_t(nq) * k_max) +
                         carve_bytes<uint16_t>(uint64_t(nq) * k_max);
@@ -745,7 +749,8 @@ static int query_common(flinng_index *idx, const flinng_points *q, const uint32_
     // large projection matrix the batched GEMM (plain form) hashes far better.
     const bool big_srp = idx->cfg.metric == FLINNG_COSINE_SRP && uint64_t(idx->P) * idx->cfg.dim > (1ull << 18);
     const bool fused = q && !big_srp && !probe &&
-                       (idx->query_mode == FLINNG_QUERY_FUSED || idx->query_mode == FLINNG_QUERY_GRAPH);
+                       (idx->query_mode == FLINNG_QUERY_FUSED || idx->query_mode == FLINNG_QUERY_GRAPH) &&
+                       query_fused_fits(idx, k_max);
     if (fused && !on_device) {
         bool done = false;
         FL_TRY(query_small_host(idx, q, nq, k, k_max, out_ids, out_scores, &done));

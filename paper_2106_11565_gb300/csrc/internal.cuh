@@ -247,6 +247,8 @@ struct FusedQuery {
 };
 int query_fused_launch(flinng_index *ix, const FusedQuery &fq, const uint32_t *k, uint32_t k_max,
                        uint32_t *out_ids, uint16_t *out_scores, const QueryTuning *tune);
+// Some fused CTA fits shared memory (else batches are hashed first: query_launch).
+bool query_fused_fits(const flinng_index *ix, uint32_t k_max);
 int query_graph_launch(flinng_index *ix, const FusedQuery &fq, const uint32_t *k, uint32_t k_max,
                        uint32_t *out_ids, uint16_t *out_scores, const QueryTuning *tune);
 void destroy_graphs(flinng_index *ix);

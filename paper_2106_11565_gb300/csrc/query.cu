@@ -8,6 +8,8 @@
 namespace flinng {
 namespace {
 
+constexpr size_t kMaxSmem = 227 * 1024;   // dynamic shared memory of a CTA
+
 inline uint32_t pow2_at_least(uint32_t v)
 {
     uint32_t p = 1;
@@ -72,7 +74,7 @@ void pick_buffer(QArgs &a, int NT, const QueryTuning *tune, size_t extra, size_t
     if (cap < cap_min) cap = cap_min;
     a.lcap = a.B < kLevelCells ? (a.B + 7) & ~7u : kLevelCells;
     auto bytes = [&](uint32_t c) { return qsmem_bytes(c, a.kp, a.BR, a.lcap, NT, a.L, cw); };
-    while (bytes(cap) + extra > 227 * 1024 && cap > cap_min) cap >>= 1;
+    while (bytes(cap) + extra > kMaxSmem && cap > cap_min) cap >>= 1;
     a.cap = cap;
     const size_t smem = bytes(cap);
     *smem_out = smem;
@@ -138,7 +140,7 @@ int query_launch_counts(flinng_index *ix, const uint32_t *qbuckets, const uint16
     // 130 so; a batch resident at once, 1,200 of them, 54 and 60; 16-bit counts,
     // 4,000 queries of 512 tables, 144 and 188)
     const uint32_t sm_threads = NT == 256 && cw == 1 && 228 * 1024 / (smem + 1024) > 4 && nq > 8 * sms ? 2048 : 1024;
-    if (smem > 227 * 1024)
+    if (smem > kMaxSmem)
         return set_error(FLINNG_ERR_INVALID_ARG,
                          "query: k_max=%u with B*R=%u needs %zu bytes of shared memory (> 227 KB)",
                          k_max, a.BR, smem);
@@ -162,6 +164,36 @@ struct FusedPlan {
     void *args[2];
 };
 
+// Shared memory of a fused CTA of nt threads; a's buffer sizes and the hash
+// region's offset are set. The hash region (query buckets, hash scratch, the
+// query slot) is live only before the decode keeps candidates, so it shares the
+// candidate buffer with the gather's heavy-table list (the buffer's last 2 nt
+// words) when both fit; otherwise it follows the query state.
+static size_t fused_smem(const flinng_index *ix, QArgs &a, int nt, const QueryTuning *tune, bool light, size_t *hash_off)
+{
+    const size_t scratch = ix->cfg.metric == FLINNG_COSINE_SRP ? ix->cfg.dim : ix->P + (ix->P + 31) / 32;
+    const size_t hash_bytes = (size_t((ix->cfg.L + 3) & ~3u) * 4 + 16 + scratch * 4 + 15) & ~size_t(15);
+    size_t qbytes;
+    pick_buffer(a, nt, tune, 0, &qbytes, int(ix->cw), light);
+    *hash_off = 0;
+    if (hash_bytes + size_t(nt) * 8 <= size_t(a.cap) * 8) return qbytes;
+    pick_buffer(a, nt, tune, hash_bytes, &qbytes, int(ix->cw), light);
+    *hash_off = qbytes;
+    return qbytes + hash_bytes;
+}
+
+bool query_fused_fits(const flinng_index *ix, uint32_t k_max)
+{
+    QArgs a{};
+    a.L = ix->cfg.L;
+    a.B = ix->cfg.B;
+    a.R = ix->cfg.R;
+    a.BR = ix->BR;
+    a.k_max = k_max;
+    size_t off;
+    return fused_smem(ix, a, 128, nullptr, true, &off) <= kMaxSmem;
+}
+
 static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t *k, uint32_t k_max,
                          uint32_t *out_ids, uint16_t *out_scores, const QueryTuning *tune,
                          uint32_t grid_for, FusedPlan *P)
@@ -181,7 +213,6 @@ static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t 
     const bool srp = ix->cfg.metric == FLINNG_COSINE_SRP;
     h.K = ix->cfg.K;
     h.qnext = ix->qnext;
-    size_t hash_bytes = size_t((ix->cfg.L + 3) & ~3u) * 4 + 16;
     if (srp) {
         h.x = fq.x;
         h.ldx = fq.ldx;
@@ -191,7 +222,6 @@ static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t 
         h.tiny = float(h.d) * ldexpf(1.0f, -146);
         h.gamma64 = ix->srp_gamma64;
         h.stats = ix->stats;
-        hash_bytes += size_t(h.d) * 4;
     } else {
         h.q_off = fq.off;
         h.q_el = fq.elems;
@@ -202,26 +232,9 @@ static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t 
         h.ba = ix->bucket_a;
         h.bc = ix->bucket_c;
         h.draw = ix->doph_draw;
-        hash_bytes += size_t(h.nb + (h.nb + 31) / 32) * 4;
     }
-    hash_bytes = (hash_bytes + 15) & ~size_t(15);
-    // The hash region (query buckets, hash scratch, the query slot) is live
-    // only before the decode keeps candidates, so it shares the candidate
-    // buffer with the gather's heavy-table list (the buffer's last 2 NT words)
-    // when both fit; otherwise it follows the query state.
     const bool light = expected_members(ix) < kLightMembers;
-    auto shape = [&](int nt) {
-        size_t qbytes;
-        pick_buffer(a, nt, tune, 0, &qbytes, int(ix->cw), light);
-        if (hash_bytes + size_t(nt) * 8 <= size_t(a.cap) * 8) {
-            h.hash_off = 0;
-            P->smem = qbytes;
-        } else {
-            pick_buffer(a, nt, tune, hash_bytes, &qbytes, int(ix->cw), light);
-            h.hash_off = qbytes;
-            P->smem = qbytes + hash_bytes;
-        }
-    };
+    auto shape = [&](int nt) { P->smem = fused_smem(ix, a, nt, tune, light, &h.hash_off); };
     // CTA size, unless tuned. A batch that is resident at once takes 512 threads:
     // it waits for its slowest query, whose phases scale with its CTA (1 query
     // of the recall-target genomic index: 35 us with 512, 43 with 256, 65 with
@@ -261,8 +274,10 @@ static int fused_prepare(flinng_index *ix, const FusedQuery &fq, const uint32_t 
             }
         }
     }
+    // a shape that asks for too much (the usual one or a tuned one): smaller CTAs
+    while (P->smem > kMaxSmem && NT > 128) shape(NT /= 2);
     if (both && fit() * uint32_t(NT) <= 1024) sm_threads = 1024;
-    if (P->smem > 227 * 1024)
+    if (P->smem > kMaxSmem)
         return set_error(FLINNG_ERR_INVALID_ARG, "fused query: %zu bytes of shared memory needed (> 227 KB)", P->smem);
     P->fn = ix->cw == 1 ? fused_kernel_c1(NT, ix->rw, srp, sm_threads) : fused_kernel_c2(NT, ix->rw, srp, sm_threads);
     P->threads = NT;

@@ -272,10 +272,12 @@ int launch_batch(flinng_server *srv, Slot &slot, const flinng_request *reqs, uin
     const uint32_t *dk = reinterpret_cast<const uint32_t *>(dh + ho_.k);
     uint32_t *dids = reinterpret_cast<uint32_t *>(d + Lo.ids);
     uint16_t *dsc = reinterpret_cast<uint16_t *>(d + Lo.sc);
-    if (big_srp) {
+    if (big_srp || !query_fused_fits(ix, km)) {
         uint32_t *qb = reinterpret_cast<uint32_t *>(d + Lo.qb);
-        rc = srp_hash(ix, reinterpret_cast<const float *>(d + Lo.in_el), ix->cfg.dim, nb, qb, nullptr, d + Lo.srp,
-                      srv->max_srp);
+        rc = srp ? srp_hash(ix, reinterpret_cast<const float *>(d + Lo.in_el), ix->cfg.dim, nb, qb, nullptr, d + Lo.srp,
+                            srv->max_srp)
+                 : doph_hash(ix, reinterpret_cast<const uint64_t *>(dh + ho_.in_off),
+                             reinterpret_cast<const uint32_t *>(d + Lo.in_el), nb, qb, nullptr);
         if (slot.direct) {
             dids = out_ids;
             dsc = out_scores;
