@@ -407,11 +407,12 @@ uint64_t flinng_kernel_launches(void);
  * out_ids and out_scores are device memory; the call is asynchronous on the
  * index's stream. The index's device must be the current device.
  * Limits: nq * L <= 262144, and for cosine indices nq * L * K <= 655296.
- * Cosine indices of a tensor-core precision also stage every query row's
- * quantised parts (at most 4 * dim bytes: FLINNG_PREC_BF16X2) and two
- * re-check lists in the same 5 MiB part of
- * the array: about nq * (4 * dim + 16 * L * K + 12) + 8192 <= 5242880 bytes
- * (the call computes the exact figure). Larger batches are rejected with
+ * Cosine indices of a tensor-core precision also stage query rows' quantised
+ * parts (q * dim bytes a row, q = 4 for FLINNG_PREC_BF16X2, 2 for
+ * FLINNG_PREC_BF16, 1 for FLINNG_PREC_FP8) and two re-check lists in the same
+ * 5 MiB part of the array: about nq * (q * dim + 16 * L * K + 24) + 8192 <=
+ * 5242880 bytes (the call computes the exact figure; a single-term form whose
+ * second pass needs more takes the batch in parts). Larger batches are rejected with
  * FLINNG_ERR_INVALID_ARG before anything runs (split them, or use
  * flinng_query).
  * The first call in a device's CUDA context looks up the scratch array's

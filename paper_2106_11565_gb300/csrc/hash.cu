@@ -549,10 +549,9 @@ bool srp_few_rows(const flinng_index *ix, uint64_t n, const float *proj)
 int srp_hash(flinng_index *ix, const float *x, uint64_t ld, uint64_t n,
              uint32_t *buckets, float *proj, void *ws, size_t ws_bytes)
 {
-    (void)ws_bytes;
     if (ix->h_flag[3]) return set_error(FLINNG_ERR_TIMEOUT, "tensor-core SRP: a pipeline wait timed out");
     const bool few = srp_few_rows(ix, n, proj);
-    if (ix->cfg.precision != FLINNG_PREC_FP32 && !few) return srp_hash_tc(ix, x, ld, n, buckets, proj, ws);
+    if (ix->cfg.precision != FLINNG_PREC_FP32 && !few) return srp_hash_tc(ix, x, ld, n, buckets, proj, ws, ws_bytes);
     const cudaStream_t st = ix->stream;
     const uint32_t L = ix->cfg.L, K = ix->cfg.K, d = ix->cfg.dim, P = ix->P;
     Carver c(ws, ~size_t(0));

@@ -206,8 +206,9 @@ int add_counter(unsigned long long *dst, const unsigned long long *src, cudaStre
 // ---- srp_tc.cu (tensor-core precision form)
 int srp_tc_prepare_weights(flinng_index *ix);
 size_t srp_tc_workspace_bytes(const flinng_index *ix, uint64_t n);
+size_t srp_tc_least_bytes(const flinng_index *ix, uint64_t n);
 int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint32_t *buckets, float *proj,
-                void *ws);
+                void *ws, size_t ws_bytes);
 
 // ---- build.cu
 size_t perm_check_workspace_bytes(uint32_t R, uint64_t n);

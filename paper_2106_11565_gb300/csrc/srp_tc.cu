@@ -1005,17 +1005,36 @@ size_t srp_tc_workspace_bytes(const flinng_index *ix, uint64_t n)
            3 * carve_bytes<uint32_t>(rows + 1) + carve_bytes<char>(scan_workspace_bytes(rows + 1)) + 4096;
 }
 
+// The same with the rows quantised in the form's own width: what a caller with a
+// fixed scratch needs (srp_hash_tc takes as many rows at a time as fit).
+size_t srp_tc_least_bytes(const flinng_index *ix, uint64_t n)
+{
+    const uint64_t rows = n < kTcChunkRows ? n : kTcChunkRows;
+    return srp_tc_workspace_bytes(ix, n) - carve_bytes<char>(rows * x_bytes(ix)) +
+           carve_bytes<char>(rows * qrow_bytes(ix->cfg.precision, ix->cfg.dim));
+}
+
 // Codes of n rows of x (stride ld) on the tensor cores; same contract as srp_hash.
 int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint32_t *buckets, float *proj,
-                void *ws)
+                void *ws, size_t ws_bytes)
 {
     // a wait that timed out in an earlier call (the flag is sticky on the device)
     if (ix->h_flag[3]) return set_error(FLINNG_ERR_TIMEOUT, "tensor-core SRP: a pipeline wait timed out");
     const cudaStream_t st = ix->stream;
     const uint32_t L = ix->cfg.L, K = ix->cfg.K, d = ix->cfg.dim, P = ix->P, prec = ix->cfg.precision;
     const bool bytes = prec == FLINNG_PREC_FP8;
-    const uint64_t chunk = kTcChunkRows;
-    const uint64_t cap = n < chunk ? n : chunk;     // rows the workspace was sized for
+    uint64_t cap = n < kTcChunkRows ? n : kTcChunkRows;     // rows that the workspace holds
+    if (srp_tc_workspace_bytes(ix, cap) > ws_bytes) {
+        uint64_t lo = 1;
+        while (lo < cap) {
+            const uint64_t mid = (lo + cap + 1) / 2;
+            if (srp_tc_workspace_bytes(ix, mid) <= ws_bytes) lo = mid;
+            else cap = mid - 1;
+        }
+        if (srp_tc_workspace_bytes(ix, cap) > ws_bytes)
+            return set_error(FLINNG_ERR_INVALID_ARG, "internal: tensor-core SRP scratch of %zu bytes", ws_bytes);
+    }
+    const uint64_t chunk = cap;
     Carver c(ws, ~size_t(0));
     char *xq = c.take<char>(cap * x_bytes(ix));
     float *xn = c.take<float>(cap);
