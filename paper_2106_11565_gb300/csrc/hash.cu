@@ -14,6 +14,7 @@
 // j = splitmix64(seed ^ (i << 32 | attempt)) mod nb, attempt = 1, 2, ...
 // (4096 tries, then the next non-empty bin cyclically). Table l combines its
 // K values as ((sum_j a_{l,j} v_{lK+j} + c_l) mod 2^64) >> (64 - W).
+#include <cfloat>
 #include <cmath>
 
 #include "internal.cuh"
@@ -200,8 +201,11 @@ k_srp_fp32(const float *__restrict__ X, uint64_t ldx, uint64_t n, const float *_
             unpack2(tot[i / 2][j], lo, hi);
             const float p = (i & 1) ? hi : lo;
             if (proj) proj[gr * P + gc] = p;
-            const float margin = fmaf(c_norm * nx, wnorm[gc], tiny);
-            if (fabsf(p) > margin) {
+            // the norms' product first: a factor of 1e-6 would lose a tiny row's bound to
+            // underflow. A sum that overflowed on the way decides nothing (its margin may
+            // be finite).
+            const float margin = fmaf(c_norm, nx * wnorm[gc], tiny);
+            if (fabsf(p) > margin && fabsf(p) <= FLT_MAX) {
                 const uint32_t l = gc / K;
                 if (l != cur_l) {
                     if (bits) atomicOr(&codes[gr * L + cur_l], bits);
