@@ -263,8 +263,11 @@ bool pinned_points(const flinng_index *ix, const flinng_points *pts, uint64_t n,
 // the results memcpy'd out after one wait. For a few KB this replaces up to five
 // asynchronous copies of pageable memory and the buffers' pointer queries, which
 // cost more than the query (1 genomic read: 59 -> 31 us a call). Larger batches
-// move at copy-engine rates instead. The staging is in use only within a call,
-// which waits for the kernel; calls on one index do not overlap.
+// move at copy-engine rates instead. Page-locked vectors are read in place, in
+// stream order: work queued before the call may still be filling them (offsets,
+// elements and k are the host's to read, which checks them, so they are there).
+// The staging is in use only within a call, which waits for the kernel; calls on
+// one index do not overlap.
 int query_small_host(flinng_index *ix, const flinng_points *q, uint32_t nq, const uint32_t *k, uint32_t k_max,
                      uint32_t *out_ids, uint16_t *out_scores, bool *done)
 {
@@ -278,7 +281,11 @@ int query_small_host(flinng_index *ix, const flinng_points *q, uint32_t nq, cons
     if (need > kSmallStage) return FLINNG_OK;
     Carver c(reinterpret_cast<char *>(ix->h_flag) + 256, kSmallStage);
     FusedQuery fq{nq, nullptr, ix->cfg.dim, nullptr, nullptr};
-    if (srp) {
+    Staged in_place;
+    if (srp && pinned_points(ix, q, nq, in_place)) {
+        fq.x = in_place.x;
+        fq.ldx = in_place.ld;
+    } else if (srp) {
         float *x = c.take<float>(ne);
         for (uint32_t i = 0; i < nq; ++i)
             std::memcpy(x + size_t(i) * ix->cfg.dim, q->x + size_t(i) * q->ld, ix->cfg.dim * sizeof(float));
