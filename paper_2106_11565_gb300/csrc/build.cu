@@ -737,7 +737,9 @@ int insert_hashed(flinng_index *ix, uint32_t *buckets, const uint32_t *perm, con
     const uint64_t n_old = ix->n_points, N = n_old + n, nslot = ix->nslot;
     const bool have_old = ix->n_cells > 0;
     const uint64_t D = n * L * R;   // new (table, cell) entries before deduplication
-    const bool delta = delta_insert_applies(ix, n) || delta_part_applies(ix, n);
+    // a batch with a partition past what a CTA sorts (buckets that many points
+    // share; told by the wait for the input checks) takes the full merge
+    const bool delta = delta_insert_applies(ix, n) || (delta_part_applies(ix, n) && !(ix->h_flag[0] & kFlagHot));
     Carver c(ws, ~size_t(0));
     uint32_t *mcur = c.take<uint32_t>(BR + 1);
     if (delta) {
@@ -745,9 +747,7 @@ int insert_hashed(flinng_index *ix, uint32_t *buckets, const uint32_t *perm, con
         void *dws = c.base + ((c.used + 255) & ~size_t(255));
         FL_TRY(member_stage(ix, perm, groups, n, mcur, dws));
         TraceRange stage2("reverse index (delta)");
-        bool done = false;
-        FL_TRY(insert_delta(ix, buckets, n, dws, &done));
-        if (done) return FLINNG_OK;
+        return insert_delta(ix, buckets, n, dws);
     }
     if (n_old == 0 && part_build_applies(ix, n)) {
         // from scratch: sorted partition by partition in shared memory
@@ -775,7 +775,7 @@ int insert_hashed(flinng_index *ix, uint32_t *buckets, const uint32_t *perm, con
     uint16_t *dbuf = have_old ? c.take<uint16_t>(D) : ix->cells_tmp;
     void *scan_ws = c.base + ((c.used + 255) & ~size_t(255));
 
-    if (!delta) FL_TRY(member_stage(ix, perm, groups, n, mcur, scan_ws));
+    FL_TRY(member_stage(ix, perm, groups, n, mcur, scan_ws));
 
     TraceRange stage2("reverse index");    // 1. the new entries by slot: counting sort (histogram, scan, scatter)
     uint32_t *hist = ix->slot_a;

@@ -919,29 +919,36 @@ bool plan_for(const flinng_index *ix, uint64_t n, PartPlan *pl)
 
 }  // namespace
 
-// Steps 1 and 2 for n new points: part (n x L entries) grouped by (table, top C
-// bucket bits) with the groups' bases in pbase (L << C of them, the total last);
-// bt: room for L x n buckets (dead afterwards; may be anything but buckets and
-// part), pcur: L << C words of scratch.
-int partition_entries(flinng_index *ix, const uint32_t *buckets, uint64_t n, uint32_t C, uint32_t idbits, uint32_t *bt,
-                      uint32_t *part, uint32_t *pbase, uint32_t *pcur, void *scan_ws)
+// Step 1 for n new points: bt (room for L x n words; may be anything but buckets)
+// receives the transposed buckets, pcur (L << C words) the entries of each
+// (table, top C bucket bits).
+int partition_count(flinng_index *ix, const uint32_t *buckets, uint64_t n, uint32_t C, uint32_t *bt, uint32_t *pcur)
+{
+    const cudaStream_t st = ix->stream;
+    const uint32_t L = ix->cfg.L, low = ix->cfg.range_bits - C;
+    FL_CUDA(cudaMemsetAsync(pcur, 0, (uint64_t(L) << C) * sizeof(uint32_t), st));
+    k_transpose<<<dim3(unsigned((n + 31) / 32), (L + 31) / 32), 256, 0, st>>>(buckets, n, L, bt);
+    count_launch();
+    FL_CUDA(cudaGetLastError());
+    k_part_count<<<dim3(unsigned((n + kTile - 1) / kTile), L), kT, sizeof(uint32_t) << C, st>>>(bt, n, C, low, pcur);
+    count_launch();
+    FL_CUDA(cudaGetLastError());
+    return FLINNG_OK;
+}
+
+// Step 2, after it: part (n x L entries) grouped by partition, with the groups'
+// bases in pbase (L << C of them, the total last); bt is dead afterwards.
+int partition_scatter(flinng_index *ix, uint64_t n, uint32_t C, uint32_t idbits, const uint32_t *bt, uint32_t *part,
+                      uint32_t *pbase, uint32_t *pcur, void *scan_ws)
 {
     const cudaStream_t st = ix->stream;
     const uint32_t L = ix->cfg.L, low = ix->cfg.range_bits - C;
     const uint64_t parts = uint64_t(L) << C;
-    FL_CUDA(cudaMemsetAsync(pcur, 0, parts * sizeof(uint32_t), st));
-    k_transpose<<<dim3(unsigned((n + 31) / 32), (L + 31) / 32), 256, 0, st>>>(buckets, n, L, bt);
-    count_launch();
-    FL_CUDA(cudaGetLastError());
-    const dim3 tiles(unsigned((n + kTile - 1) / kTile), L);
-    k_part_count<<<tiles, kT, sizeof(uint32_t) << C, st>>>(bt, n, C, low, pcur);
-    count_launch();
-    FL_CUDA(cudaGetLastError());
     FL_TRY(scan_exclusive(pcur, pbase, parts, scan_ws, st));
     FL_CUDA(cudaMemcpyAsync(pcur, pbase, parts * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st));
     const size_t ssm = (sizeof(uint32_t) * 2 << C) + kTile * 6 + (kT / 32) * 4;
     FL_TRY(ensure_dyn_smem((const void *)k_part_scatter, ssm));
-    k_part_scatter<<<tiles, kT, ssm, st>>>(bt, n, C, low, idbits, pcur, part);
+    k_part_scatter<<<dim3(unsigned((n + kTile - 1) / kTile), L), kT, ssm, st>>>(bt, n, C, low, idbits, pcur, part);
     count_launch();
     FL_CUDA(cudaGetLastError());
     return FLINNG_OK;
@@ -1001,7 +1008,8 @@ int part_build(flinng_index *ix, uint32_t *buckets, uint64_t n, void *ws, uint32
     uint32_t *part = buckets;
     FL_CUDA(cudaMemsetAsync(cnt, 0, 8 * sizeof(uint32_t), st));
     FL_CUDA(cudaMemsetAsync(wbm, 0, nwide * ix->BRw * sizeof(uint32_t), st));
-    FL_TRY(partition_entries(ix, buckets, n, pl.C, pl.idbits, bt, part, pbase, pcur, scan_ws));
+    FL_TRY(partition_count(ix, buckets, n, pl.C, bt, pcur));
+    FL_TRY(partition_scatter(ix, n, pl.C, pl.idbits, bt, part, pbase, pcur, scan_ws));
     FineArgs a{};
     a.part = part;
     a.pbase = pbase;

@@ -398,6 +398,7 @@ int insert_common(flinng_index *ix, const flinng_points *pts, uint64_t n, const 
     } else {
         FL_TRY(hash_staged(ix, s, n, buckets, nullptr, nullptr, hws, hb));
     }
+    if (!reset) FL_TRY(delta_count(ix, buckets, n, iws));
     FL_TRY(check_result(ix));
     if (reset) {
         ix->n_points = 0;

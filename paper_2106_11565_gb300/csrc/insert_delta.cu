@@ -106,15 +106,14 @@ __device__ __forceinline__ uint32_t rank_u16(const uint16_t *a, uint32_t n, uint
 // when W + CB <= 31; P2 (a power of two, 32 .. E blockDim, >= the segment's
 // cells) of them in shared memory, E per thread. Segment l is table l, or with
 // pbase partition l: W is then the bits below the partition's, part its packed
-// entries, and a partition of more than P2max cells only sets *over.
+// entries (at most P2max cells: delta_count).
 template <class KT, int E>
 __global__ void __launch_bounds__(kDeltaThreads)
 k_delta_table(const uint32_t *__restrict__ buckets, const uint16_t *__restrict__ gid, uint64_t n_old, uint32_t n,
               uint32_t L, uint32_t W, uint32_t R, uint32_t B, uint32_t rp, uint32_t P2max, uint32_t CB,
               const uint32_t *__restrict__ off, const uint16_t *__restrict__ cells, uint16_t *__restrict__ rcell,
               uint2 *__restrict__ rt, uint32_t *__restrict__ A, uint32_t *__restrict__ T,
-              const uint32_t *__restrict__ pbase, const uint32_t *__restrict__ part, uint32_t idbits,
-              uint32_t *__restrict__ over)
+              const uint32_t *__restrict__ pbase, const uint32_t *__restrict__ part, uint32_t idbits)
 {
     constexpr KT kNone = ~KT(0);
     extern __shared__ __align__(16) unsigned char dsm[];
@@ -126,10 +125,7 @@ k_delta_table(const uint32_t *__restrict__ buckets, const uint16_t *__restrict__
     uint32_t P2 = P2max;
     if (pbase) {
         if (nR == 0 || nR > P2max) {
-            if (tid == 0) {
-                A[l] = T[l] = 0u;
-                if (nR) atomicOr(over, 1u);
-            }
+            if (tid == 0) A[l] = T[l] = 0u;
             return;
         }
         for (P2 = 32 * E; P2 < nR; P2 <<= 1) {}
@@ -543,6 +539,13 @@ namespace {
 // kPartCells, a third of what its CTA sorts (kPartThreads x 8).
 constexpr uint32_t kPartCells = 640, kPartThreads = 256;
 
+// Raises kFlagHot where a partition holds more than `most` entries.
+__global__ void k_delta_hot(const uint32_t *__restrict__ cnt, uint64_t parts, uint32_t most, uint32_t *flag)
+{
+    for (uint64_t p = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < parts; p += uint64_t(gridDim.x) * blockDim.x)
+        if (cnt[p] > most) atomicOr(flag, kFlagHot);
+}
+
 struct DeltaPlan {
     uint32_t C, low, idbits;
     uint64_t segs;             // tables or partitions
@@ -587,12 +590,45 @@ size_t delta_workspace_bytes(const flinng_index *ix, uint64_t n)
            4 * carve_bytes<uint32_t>(D + 1) + carve_bytes<uint16_t>(D) + carve_bytes<uint32_t>(D + 1) +
            carve_bytes<uint32_t>(4) + scan_workspace_bytes(pl.segs + 1) +
            2 * carve_bytes<uint32_t>(std::max(ix->nslot + 1, ix->n_cells + D) / kChunk + 3) +
-           (part ? carve_bytes<uint32_t>(n * ix->cfg.L) + 2 * carve_bytes<uint32_t>(pl.segs + 1) : 0);
+           (part ? carve_bytes<uint32_t>(n * ix->cfg.L) + 2 * carve_bytes<uint32_t>(pl.segs + 1) +
+                       carve_bytes<char>(scan_workspace_bytes(size_t(ix->BR) + 1))
+                 : 0);
 }
 
-int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws, bool *done)
+namespace {
+
+// The partitions' counters, behind what the member-list stage uses of dws.
+Carver delta_carver(const flinng_index *ix, const DeltaPlan &pl, bool part, void *dws, uint32_t **pcur)
 {
-    *done = false;
+    Carver c(dws, ~size_t(0));
+    *pcur = nullptr;
+    if (part) {
+        c.take<char>(scan_workspace_bytes(size_t(ix->BR) + 1));
+        *pcur = c.take<uint32_t>(pl.segs + 1);
+    }
+    return c;
+}
+
+}  // namespace
+
+int delta_count(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws)
+{
+    DeltaPlan pl;
+    if (!delta_part_applies(ix, n) || !delta_plan(ix, n, true, &pl)) return FLINNG_OK;
+    Carver c(ws, ~size_t(0));
+    c.take<uint32_t>(ix->BR + 1);
+    uint32_t *pcur;
+    delta_carver(ix, pl, true, c.base + ((c.used + 255) & ~size_t(255)), &pcur);
+    // the transposed buckets pass through the list scratch, written only by the merge
+    FL_TRY(partition_count(ix, buckets, n, pl.C, reinterpret_cast<uint32_t *>(ix->cells_tmp), pcur));
+    k_delta_hot<<<blocks_of(pl.segs, 256), 256, 0, ix->stream>>>(pcur, pl.segs, kPartThreads * 8 / ix->cfg.R, ix->flag);
+    count_launch();
+    FL_CUDA(cudaGetLastError());
+    return FLINNG_OK;
+}
+
+int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *dws)
+{
     const cudaStream_t st = ix->stream;
     const uint32_t R = ix->cfg.R, B = ix->cfg.B, W = ix->cfg.range_bits;
     const uint64_t n_old = ix->n_points, nslot = ix->nslot, n_cells = ix->n_cells;
@@ -603,7 +639,8 @@ int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws
         return set_error(FLINNG_ERR_INVALID_ARG, "internal: delta insert of %llu points", (unsigned long long)n);
     const uint32_t L = uint32_t(pl.segs), low = part ? pl.low : W;       // L: segments from here on
     const uint32_t nR = part ? 0u : uint32_t(n * R);
-    Carver c(ws, ~size_t(0));
+    uint32_t *pcur;
+    Carver c = delta_carver(ix, pl, part, dws, &pcur);
     uint16_t *rcell = c.take<uint16_t>(D);
     uint2 *rt = c.take<uint2>(D);
     uint32_t *A = c.take<uint32_t>(L + 1), *T = c.take<uint32_t>(L + 1);
@@ -615,18 +652,17 @@ int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws
     const uint64_t nchunk = std::max(nslot + 1, n_cells) / kChunk + 2;
     uint32_t *off_j = c.take<uint32_t>(nchunk + 1), *mov_lo = c.take<uint32_t>(nchunk);
     uint32_t *cnt = c.take<uint32_t>(4);
-    uint32_t *ent = nullptr, *pbase = nullptr, *pcur = nullptr;
+    uint32_t *ent = nullptr, *pbase = nullptr;
     if (part) {
         ent = c.take<uint32_t>(n * ix->cfg.L);
         pbase = c.take<uint32_t>(L + 1);
-        pcur = c.take<uint32_t>(L + 1);
     }
     void *scan_ws = c.base + ((c.used + 255) & ~size_t(255));
 
     FL_CUDA(cudaMemsetAsync(cnt, 0, 4 * sizeof(uint32_t), st));
-    // the transposed buckets pass through the list scratch, written only by the merge
-    if (part) FL_TRY(partition_entries(ix, buckets, n, pl.C, pl.idbits, reinterpret_cast<uint32_t *>(ix->cells_tmp), ent,
-                                       pbase, pcur, scan_ws));
+    if (part)
+        FL_TRY(partition_scatter(ix, n, pl.C, pl.idbits, reinterpret_cast<uint32_t *>(ix->cells_tmp), ent, pbase, pcur,
+                                 scan_ws));
     const uint32_t P2 = part ? kPartThreads * 8 : pow2_ceil(nR < 32 ? 32u : nR);
     uint32_t CB = 1;
     while ((1u << CB) < ix->BR) ++CB;
@@ -634,19 +670,12 @@ int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws
     const uint32_t threads = part ? kPartThreads : uint32_t(kDeltaThreads);
     if (low + CB <= 31)        // all-ones marks padding: real keys stay below it
         FL_TRY(launch_table<uint32_t>(E, L, threads, P2, st, buckets, ix->gid, n_old, uint32_t(n), L, low, R, B, ix->rp,
-                                      P2, CB, ix->off, ix->cells, rcell, rt, A, T, pbase, ent, pl.idbits, cnt + 1));
+                                      P2, CB, ix->off, ix->cells, rcell, rt, A, T, pbase, ent, pl.idbits));
     else
         FL_TRY(launch_table<uint64_t>(E, L, threads, P2, st, buckets, ix->gid, n_old, uint32_t(n), L, low, R, B, ix->rp,
-                                      P2, CB, ix->off, ix->cells, rcell, rt, A, T, pbase, ent, pl.idbits, cnt + 1));
+                                      P2, CB, ix->off, ix->cells, rcell, rt, A, T, pbase, ent, pl.idbits));
     count_launch();
     FL_CUDA(cudaGetLastError());
-    if (part) {
-        // a partition past what a CTA sorts (buckets that many points share): the
-        // full merge, before anything of the index changes
-        FL_CUDA(cudaMemcpyAsync(ix->h_flag, cnt + 1, 4, cudaMemcpyDeviceToHost, st));
-        FL_CUDA(cudaStreamSynchronize(st));
-        if (ix->h_flag[0]) return FLINNG_OK;
-    }
     FL_TRY(scan_exclusive(A, Apre, L, scan_ws, st));
     FL_TRY(scan_exclusive(T, Tpre, L, scan_ws, st));
     k_delta_flatten<<<L, part ? 128 : 256, 0, st>>>(Apre, Tpre, L, low, nR, pbase, R, rcell, rt, ix->off, gslot, gdbeg,
@@ -713,7 +742,6 @@ int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws
     ix->n_cells = n_cells + added;
     ix->n_heavy += nh_new;
     ix->n_points = n_old + n;
-    *done = true;
     return FLINNG_OK;
 }
 

@@ -231,8 +231,9 @@ int heavy_bitmaps(flinng_index *ix, const uint32_t *list, const uint32_t *count)
 // ---- build_part.cu
 // A build from scratch sorts its entries partition by partition in shared
 // memory where part_build_applies.
-int partition_entries(flinng_index *ix, const uint32_t *buckets, uint64_t n, uint32_t C, uint32_t idbits, uint32_t *bt,
-                      uint32_t *part, uint32_t *pbase, uint32_t *pcur, void *scan_ws);
+int partition_count(flinng_index *ix, const uint32_t *buckets, uint64_t n, uint32_t C, uint32_t *bt, uint32_t *pcur);
+int partition_scatter(flinng_index *ix, uint64_t n, uint32_t C, uint32_t idbits, const uint32_t *bt, uint32_t *part,
+                      uint32_t *pbase, uint32_t *pcur, void *scan_ws);
 bool part_build_applies(const flinng_index *ix, uint64_t n);
 size_t part_workspace_bytes(const flinng_index *ix, uint64_t n);
 int part_build(flinng_index *ix, uint32_t *buckets, uint64_t n, void *ws, uint32_t **list_out, uint32_t **count_out);
@@ -274,10 +275,14 @@ constexpr uint32_t kDeltaMaxKeys = 8192;
 bool delta_insert_applies(const flinng_index *ix, uint64_t n);
 bool delta_part_applies(const flinng_index *ix, uint64_t n);
 size_t delta_workspace_bytes(const flinng_index *ix, uint64_t n);
-// After insert_hashed's group and member-list stage: the reverse index.
-// *done stays false, and the index as it was, when a partition of a
-// partitioned batch was too large (the caller takes the full merge).
-int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws, bool *done);
+// Ahead of the wait for the input checks (check_result): counts a partitioned
+// batch's entries by partition and raises kFlagHot in ix->flag if one is past
+// what a CTA sorts. ws: insert_hashed's.
+constexpr uint32_t kFlagHot = 16u;
+int delta_count(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *ws);
+// After insert_hashed's group and member-list stage, unless that flag was raised:
+// the reverse index. dws: the workspace behind insert_hashed's member cursors.
+int insert_delta(flinng_index *ix, const uint32_t *buckets, uint64_t n, void *dws);
 
 // ---- probe.cu
 // Multi-probe counts (probes P >= 1 per table): nq x B*R uint16, each <= L.
