@@ -569,14 +569,17 @@ bool delta_plan(const flinng_index *ix, uint64_t n, bool part, DeltaPlan *pl)
 // index's: into 20,000 reads at the recall-target parameters, 6,000 more take
 // 1.40 ms against 2.14 with the full merge's six passes over all 67 M slots,
 // 19,000 more 3.30 against 2.78; into 100,000, 10,000 take 2.34 against 3.42,
-// 20,000 3.79 against 4.00. At most 2^25 cells (32 bytes of workspace each).
+// 20,000 3.79 against 4.00. And while the batch's cells are no more than the slots:
+// the full merge's passes over few slots are cheap (12,000 reads into 40,000, 64
+// tables of 4,096 slots: 0.33 ms against 0.28). At most 2^25 cells (32 bytes of
+// workspace each).
 // R >= 2: the list scratch has room for the transposed buckets.
 bool delta_part_applies(const flinng_index *ix, uint64_t n)
 {
     const uint64_t D = n * ix->cfg.L * ix->cfg.R;
     DeltaPlan pl;
     return ix->n_cells > 0 && ix->cfg.R >= 2 && n * ix->cfg.R > kDeltaMaxKeys && 3 * D <= ix->n_cells &&
-           D <= (1ull << 25) && delta_plan(ix, n, true, &pl);
+           D <= ix->nslot && D <= (1ull << 25) && delta_plan(ix, n, true, &pl);
 }
 
 size_t delta_workspace_bytes(const flinng_index *ix, uint64_t n)
