@@ -14,6 +14,7 @@
 // j = splitmix64(seed ^ (i << 32 | attempt)) mod nb, attempt = 1, 2, ...
 // (4096 tries, then the next non-empty bin cyclically). Table l combines its
 // K values as ((sum_j a_{l,j} v_{lK+j} + c_l) mod 2^64) >> (64 - W).
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
 
@@ -416,9 +417,13 @@ __global__ void k_doph_draws(uint32_t nb, uint64_t seed, uint16_t *__restrict__ 
     if (t < nb * kDophTable) draw[t] = uint16_t(doph_draw_of(t / kDophTable, t % kDophTable + 1, nb, seed));
 }
 
-// 32-bit words of shared memory per set: bin minima, occupancy, empty bins
-__host__ __device__ inline uint32_t doph_words(uint32_t nb) { return nb + (nb + 31) / 32 + (nb + 1) / 2; }
+// 32-bit words of shared memory per set: bin minima, occupancy and, with LIST, the empty bins
+__host__ __device__ inline uint32_t doph_words(uint32_t nb, bool list)
+{
+    return nb + (nb + 31) / 32 + (list ? (nb + 1) / 2 : 0);
+}
 
+template <bool LIST>
 __global__ void __launch_bounds__(kDophWarps * 32)
 k_doph(const uint64_t *__restrict__ off, const uint32_t *__restrict__ elems,
        uint64_t n, uint32_t nb, uint32_t a, uint32_t b, uint64_t seed, uint32_t L,
@@ -429,7 +434,7 @@ k_doph(const uint64_t *__restrict__ off, const uint32_t *__restrict__ elems,
     extern __shared__ uint32_t sm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t nbw = (nb + 31) / 32;
-    uint32_t *val = sm + warp * doph_words(nb);
+    uint32_t *val = sm + warp * doph_words(nb, LIST);
     uint32_t *occ = val + nb;
     uint16_t *empty = reinterpret_cast<uint16_t *>(occ + nbw);     // nb: the empty bins
     const uint64_t gw = uint64_t(blockIdx.x) * kDophWarps + warp;
@@ -472,15 +477,17 @@ k_doph(const uint64_t *__restrict__ off, const uint32_t *__restrict__ elems,
             // idle through the other lanes' draws (with doph_source's table,
             // 100,000 genomic reads, 512 bins: 300 -> 200 us; 10^6 URL sets, 64
             // bins: 801 -> 461 us)
-            const uint32_t none = ~bits & (nb - k0 >= 32 ? 0xffffffffu : (1u << (nb - k0)) - 1u);
-            if ((none >> lane) & 1u) empty[ne + __popc(none & ((1u << lane) - 1u))] = uint16_t(k);
-            ne += __popc(none);
+            if constexpr (LIST) {
+                const uint32_t none = ~bits & (nb - k0 >= 32 ? 0xffffffffu : (1u << (nb - k0)) - 1u);
+                if ((none >> lane) & 1u) empty[ne + __popc(none & ((1u << lane) - 1u))] = uint16_t(k);
+                ne += __popc(none);
+            }
         }
         __syncwarp();
         if (end > beg) {
-            for (uint32_t i = lane; i < ne; i += 32) {
-                const uint32_t k = empty[i];
-                val[k] = val[doph_source(k, nb, seed, draw, occ)];
+            for (uint32_t i = lane; i < (LIST ? ne : nb); i += 32) {
+                const uint32_t k = LIST ? empty[i] : i;
+                if (LIST || !((occ[k >> 5] >> (k & 31)) & 1u)) val[k] = val[doph_source(k, nb, seed, draw, occ)];
             }
         }
         __syncwarp();
@@ -546,7 +553,9 @@ size_t srp_workspace_bytes(const flinng_index *ix, uint64_t n)
 // return: the codes are the same.
 bool srp_few_rows(const flinng_index *ix, uint64_t n, const float *proj)
 {
-    if (ix->cfg.precision == FLINNG_PREC_FP32) return n * ix->P <= 192 * 1024;
+    // (a short row leaves most of a warp idle: 2,000 rows x 64 projections of 32
+    // dimensions 31 us, 26 in tiles)
+    if (ix->cfg.precision == FLINNG_PREC_FP32) return n * ix->P <= (ix->cfg.dim < 128 ? 96 : 192) * 1024;
     return !proj && n <= 96 && n * ix->P <= 96 * 1024;
 }
 
@@ -615,11 +624,17 @@ int doph_hash(flinng_index *ix, const uint64_t *off, const uint32_t *elems,
 {
     if (n == 0) return FLINNG_OK;
     const uint32_t nb = ix->P;
-    const size_t smem = size_t(kDophWarps) * doph_words(nb) * sizeof(uint32_t);
-    FL_TRY(ensure_dyn_smem((const void *)k_doph, smem));
+    // the list of empty bins while it costs no resident CTA (100,000 URL sets, 2,048
+    // bins: 92 ms with it and two CTAs per SM, 74 without and three)
+    auto bytes = [&](bool list) { return size_t(kDophWarps) * doph_words(nb, list) * sizeof(uint32_t); };
+    auto ctas = [&](size_t b) { return std::min<size_t>(228 * 1024 / (b + 1024), 2048 / (kDophWarps * 32)); };
+    const bool list = ctas(bytes(true)) >= ctas(bytes(false));
+    const size_t smem = bytes(list);
+    auto fn = list ? k_doph<true> : k_doph<false>;
+    FL_TRY(ensure_dyn_smem((const void *)fn, smem));
     uint64_t blocks = (n + kDophWarps - 1) / kDophWarps;
     if (blocks > 152ull * 64) blocks = 152ull * 64;
-    k_doph<<<(unsigned)blocks, kDophWarps * 32, smem, ix->stream>>>(
+    fn<<<(unsigned)blocks, kDophWarps * 32, smem, ix->stream>>>(
         off, elems, n, nb, ix->doph_a, ix->doph_b, ix->doph_seed, ix->cfg.L, ix->cfg.K,
         ix->cfg.range_bits, ix->bucket_a, ix->bucket_c, ix->doph_draw, buckets, values);
     count_launch();
