@@ -375,8 +375,9 @@ int flinng_hash_stats(const flinng_index *idx, uint64_t *n_recheck,
  * not decide; out[1] those decided by the exact accumulator; out[2] fp64
  * re-checks; out[3] second-stage re-checks of the tensor-core precisions
  * (compensated fp32, or a dense pass on the two-term split in
- * a single-term form; none for a batch of at most 96 rows, which every
- * precision hashes in fp32 unless projections are asked for);
+ * a single-term form; none for a batch of at most 96 rows and 98,304
+ * projections, n * L * K, which every precision hashes in fp32 unless
+ * projections are asked for);
  * out[4] flips: first-pass signs that a re-check reversed (the hash-bit flip
  * rate before re-check is out[4] / (n * L * K)). out: 5 HOST uint64, written
  * after the index's stream is synchronised. Errors: INVALID_ARG for NULL. */

@@ -26,13 +26,6 @@ namespace {
 
 constexpr int kWarpsPerBlock = 8;
 
-inline unsigned warp_blocks(uint64_t items)
-{
-    uint64_t b = (items + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    if (b > 152ull * 128) b = 152ull * 128;
-    return (unsigned)(b ? b : 1);
-}
-
 inline unsigned thread_blocks(uint64_t items, int threads = 256)
 {
     uint64_t b = (items + threads - 1) / threads;

@@ -34,7 +34,7 @@
 // general path -> this one, whole build with hashing: recall-target genomic
 // index (100,000 reads, 512 tables, 67 M slots, 154 M cells) 5.08 -> 1.88 ms, of
 // which k_part_fine 0.87, k_part_finish 0.24, k_doph 0.20; URL index (10^6 sets,
-// 64 tables, 136 M cells, buckets of up to half the points) 28.2 -> 3.3 ms, where
+// 64 tables, 136 M cells, buckets of up to half the points) 23.6 -> 3.3 ms, where
 // the general path's warp per slot walked the hot buckets alone.
 #include <algorithm>
 

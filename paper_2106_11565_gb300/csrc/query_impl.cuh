@@ -1,5 +1,5 @@
 // Batched query: collision counts, group tests, AND-over-R decode and top-k
-// (Sec. 5, Alg. 2 and Alg. 3). One CTA of 256 threads per query.
+// (Sec. 5, Alg. 2 and Alg. 3). One CTA of 128 to 1,024 threads per query.
 //
 // Alg. 3 walks cells by count (descending, ties by cell id) and emits a point
 // when the last of its R cells is reached. That order is the ascending order
@@ -24,12 +24,12 @@
 //     rest read their full record and get a key from all R group ids (the AND
 //     over R). Stop once >= k points of score >= t were seen: no unseen point
 //     can precede them.
-//  4. top-k: candidates go to one shared buffer and a histogram of their
-//     scores. After each group of levels the k-th best score, read off the
-//     histogram, becomes the admission bound. When many candidates share that
-//     score, or the buffer would overflow, a radix select over the rest of the
-//     keys keeps exactly the k best and the bound becomes the k-th key. At the
-//     end the best k are ranked against each other.
+//  4. top-k: candidates go to one shared buffer. After each group of levels, or
+//     when the buffer would overflow, at most 256 of them are ranked against each
+//     other, the k best are kept and the k-th key becomes the admission bound. Of
+//     more candidates a histogram of their scores gives the k-th best score as
+//     the bound; when many share it a radix select over the rest of the keys
+//     keeps exactly the k best. At the end the best k are ranked.
 //
 // The kernels are templates on the count width; query.cu instantiates CW = 1
 // and query_c16.cu CW = 2, each in its own translation unit.

@@ -90,7 +90,6 @@ constexpr int kEpiWarps = 16;                     // four per TMEM lane quarter,
 constexpr int kTcThreads = 64 + 32 * kEpiWarps;
 constexpr uint64_t kWaitNs = 1000000000ull;       // bounded mbarrier waits: 1 s
 constexpr uint64_t kTcChunkRows = 16384;          // rows split and hashed per launch
-constexpr size_t kRecheckRowBytes = 160 * 1024;   // largest row of x the re-check stages in shared memory
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
@@ -1047,9 +1046,6 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
     uint32_t *rowoff = c.take<uint32_t>(cap + 1);
     uint32_t *fill = c.take<uint32_t>(cap + 1);
     void *scan_ws = c.take<char>(scan_workspace_bytes(cap + 1));
-    // stage 2 by row when a row of x fits in shared memory
-    const bool rows_staged = size_t(d) * sizeof(float) <= kRecheckRowBytes;
-    if (rows_staged) FL_TRY(ensure_dyn_smem((const void *)k_srp_recheck2_rows, size_t(d) * sizeof(float)));
     FL_CUDA(cudaMemsetAsync(ix->stats, 0, kStats * sizeof(unsigned long long), st));
     if (n == 0) return FLINNG_OK;
     FL_CUDA(cudaMemsetAsync(buckets, 0, n * L * sizeof(uint32_t), st));
@@ -1131,7 +1127,7 @@ int srp_hash_tc(flinng_index *ix, const float *x, uint64_t ld, uint64_t n, uint3
         // stage 2: compensated fp32; stage 3: fp64 / exact. A
         // single-term list (d < 128) is grouped by row, so that each row of x is
         // staged once; the others are short and not worth the passes.
-        if (rows_staged && !dense && prec != FLINNG_PREC_BF16X2) {
+        if (!dense && prec != FLINNG_PREC_BF16X2) {
             // the list grouped by row into list2; stage 2 lists what stays undecided in list1
             FL_CUDA(cudaMemsetAsync(rowcnt, 0, (rows + 1) * sizeof(uint32_t), st));
             FL_CUDA(cudaMemsetAsync(fill, 0, (rows + 1) * sizeof(uint32_t), st));
