@@ -1,5 +1,5 @@
 """The decode's choices by size, against the oracle: few and many candidates at a
-check (ranked directly up to 256, selected by digits above), floods of equal
+check (ranked directly up to 128, selected by digits above), floods of equal
 scores that fill the candidate buffer, one and several records in flight (batches
 resident at once, larger ones), cells of any size with and without the filter,
 one repetition, and the gather's lists taken cell by cell."""
@@ -31,7 +31,7 @@ def test_floods(F, R, B, N, L):
             np.where(rng.random(B * R) < 0.3, rng.integers(1, 4, B * R), 0),
             np.where(rng.random(B * R) < 0.05, L, 1)]
     rows = np.stack(rows).astype(np.uint16)
-    for k in (1, 31, 32, 64, 255, 256, 257, 513, 1024):
+    for k in (1, 31, 32, 64, 127, 128, 129, 255, 256, 257, 513, 1024):
         want = [O.alg3(r, moff, mem, N, R, B, k, k_max=k) for r in rows]
         for nq in (5, 310, 1300):           # 512 threads, 256, 256 with 32 registers
             ids, sc = ix.query_counts(np.tile(rows, (nq // 5, 1)), k, L)
